@@ -176,9 +176,10 @@ TrainGeom train_geom(const apsm_params *p, int P, int n_prev, int evict = -1) {
         g.T = T;
         g.RMAX = 2 * T + g.W;
         g.RS = round_up(g.RMAX, 32);
+        if (g.WP <= 24) g.RS = std::max(g.RS, 64);  // the blocked form: a warp besides the window warp
         g.KXS = round_up(2 * T, 32);
-        // tracking needs the blocked form (padded window <= 24) and a warp besides the window warp
-        g.track = want_track && g.WP <= 24 && g.RS >= 64 && 2 * T <= 2 * (g.RS - 32) ? 1 : 0;
+        // tracking needs the blocked form (padded window <= 24), whose other warps do it
+        g.track = want_track && g.WP <= 24 && 2 * T <= 2 * (g.RS - 32) ? 1 : 0;
         if (T == 1 || ChunkSmem(g).bytes <= kMaxSmemBytes) break;
     }
     g.n_chunks = P > 0 ? (P + T - 1) / T : 0;

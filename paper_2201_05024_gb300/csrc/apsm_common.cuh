@@ -91,6 +91,33 @@ __device__ __forceinline__ float ex2(float x) {
     return y;
 }
 
+// Packed pairs of FP32 values: two IEEE operations per instruction, each rounded as its scalar form.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+__device__ __forceinline__ uint64_t ffma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t v;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
+    return v;
+}
+__device__ __forceinline__ uint64_t fmul2(uint64_t a, uint64_t b) {
+    uint64_t v;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+    return v;
+}
+__device__ __forceinline__ uint64_t fadd2(uint64_t a, uint64_t b) {
+    uint64_t v;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+    return v;
+}
+__device__ __forceinline__ float sum2(uint64_t a) {  // low + high
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a));
+    return lo + hi;
+}
+
 // Gray square QAM of apsm_params.modulation, one axis: L = 2^half levels (2i - (L-1)) a.  The
 // level is the number of decision boundaries (2b - L) a, b = 1..L-1, at or below y (QPSK: the
 // sign, 0 counting as non-negative); the axis label is the Gray code of L - 1 - level.

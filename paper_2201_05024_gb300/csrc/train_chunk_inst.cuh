@@ -23,17 +23,17 @@ cudaError_t launch_chunk_sw(const ChunkArgs &a, int smem, cudaStream_t stream) {
 template <bool kExt>
 ChunkLauncher chunk_table(int WP) {
     constexpr int S = APSM_CHUNK_S;
-    switch (WP) {
-        case 4: return launch_chunk_sw<S, 4, kExt>;
-        case 8: return launch_chunk_sw<S, 8, kExt>;
-        case 12: return launch_chunk_sw<S, 12, kExt>;
-        case 16: return launch_chunk_sw<S, 16, kExt>;
-        case 20: return launch_chunk_sw<S, 20, kExt>;
-        case 24: return launch_chunk_sw<S, 24, kExt>;
-        case 32: return launch_chunk_sw<S, 32, kExt>;
-        default: break;
-    }
-    if constexpr (S >= 2) {
+    if (WP == 32) return launch_chunk_sw<S, 32, kExt>;
+    if constexpr (S >= 2) {  // (the blocked form has a warp besides the window warp)
+        switch (WP) {
+            case 4: return launch_chunk_sw<S, 4, kExt>;
+            case 8: return launch_chunk_sw<S, 8, kExt>;
+            case 12: return launch_chunk_sw<S, 12, kExt>;
+            case 16: return launch_chunk_sw<S, 16, kExt>;
+            case 20: return launch_chunk_sw<S, 20, kExt>;
+            case 24: return launch_chunk_sw<S, 24, kExt>;
+            default: break;
+        }
         if (WP == 48) return launch_chunk_sw<S, 48, kExt>;
         if (WP == 64) return launch_chunk_sw<S, 64, kExt>;
     }
@@ -48,7 +48,7 @@ ChunkLauncher chunk_table(int WP) {
 
 // One launcher table per translation unit: live-range warp count APSM_CHUNK_S, plain or extended
 // instantiations (APSM_CHUNK_EXT); padded windows per S: S = 1 holds up to 32 live-range samples
-// (windows <= 32), S = 2 up to 64, and so on.
+// (windows 25 to 32 only), S = 2 up to 64, and so on.
 ChunkLauncher APSM_CHUNK_CAT(APSM_CHUNK_CAT(chunk_launcher_s, APSM_CHUNK_S), APSM_CHUNK_CAT(_x, APSM_CHUNK_EXT))(int WP) {
     return chunk_table<APSM_CHUNK_EXT != 0>(WP);
 }

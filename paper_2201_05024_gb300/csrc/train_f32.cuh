@@ -128,6 +128,13 @@ struct ChunkArgs {
     int pdl_mode;
 };
 
+constexpr int kRingMax = 32;  // windows up to this padded size keep their kernel column in registers
+constexpr int kBlockMin = 8;  // shortest step block of the blocked form (padded windows up to 24)
+
+// Zero rows after the live range in the staged kernel table: the blocked form's lanes load whole
+// row sets of a block that may end past it.
+__host__ __device__ constexpr int chunk_zero_rows(int WP) { return WP + kBlockMin <= 32 ? 32 - WP : 0; }
+
 // Shared-memory layout of phase B (bytes; every region 16-byte aligned).
 struct ChunkSmem {
     int bar, kmat, gev, egam, beta, dg, tgt, clin, pil, trk, bytes;
@@ -135,8 +142,8 @@ struct ChunkSmem {
         const int RS = g.RS;
         const int npil = g.T + (g.W + 1) / 2 + 1;
         bar = 0;
-        kmat = 16;                                   // WP zero rows, then RS rows of RS
-        gev = kmat + (g.WP + RS) * RS * 4;
+        kmat = 16;                                   // WP zero rows, RS rows of RS, the zero rows after them
+        gev = kmat + (g.WP + RS + chunk_zero_rows(g.WP)) * RS * 4;
         egam = gev + (g.evict ? g.T * 2 * RS * 4 : 0);     // dropped-entry table only with eviction
         beta = egam + round_up(g.T * 2 * 4, 16);
         dg = beta + (4 * RS + 2 * g.WP + 224) * 4;  // beta ring, or p / gamma / b / 1/kappa + rings + mu q tables
@@ -147,9 +154,6 @@ struct ChunkSmem {
         bytes = trk + (g.track ? 32 * 4 + g.M * 8 : 0);
     }
 };
-
-constexpr int kRingMax = 32;  // windows up to this padded size keep their kernel column in registers
-constexpr int kBlockMin = 8;  // shortest step block of the blocked form (padded windows up to 24)
 
 // Phase B of one chunk for one user (blockIdx.x = k).  Thread u owns live-range sample u
 // (RS = 32 S threads); a step is one CTA barrier: window threads publish their beta, then every
@@ -211,7 +215,7 @@ __global__ void __launch_bounds__(32 * S, 1) train_chunk_kernel(const ChunkArgs 
     // chunk decides the carried samples' targets)
     float b = 0.f;
     auto read_target = [&]() {
-        if (valid) {
+        if (valid && !(a.decide && m >= s0)) {  // (0 until it is decided)
             const float2 sy = __ldcg(a.sym + (size_t)pa * K + k);
             b = l ? sy.y : sy.x;  // b_{2t} = Re b(t), b_{2t+1} = Im b(t)
         }
@@ -219,6 +223,7 @@ __global__ void __launch_bounds__(32 * S, 1) train_chunk_kernel(const ChunkArgs 
     if (!a.decide) read_target();
     for (int i = u; i < 2 * (WP + RS); i += RS) s_beta[i] = 0.f;
     for (int i = u; i < WP * RS; i += RS) s_kmat[i - WP * RS] = 0.f;
+    for (int i = u; i < chunk_zero_rows(WP) * RS; i += RS) s_kmat[R * RS + i] = 0.f;
     float rk = 0.f;  // 1 / kappa(x_j, x_j)
     // Every thread reaches this wait; the CTA votes on its outcome so that either all threads
     // go on or all leave together (no thread may skip a later barrier the others wait at).
@@ -314,7 +319,8 @@ __global__ void __launch_bounds__(32 * S, 1) train_chunk_kernel(const ChunkArgs 
     // Blocked form with more than one warp: the idle warps also accumulate the filter change
     // c_k += sum_j dgamma_j x~_j block by block (thread = antenna x part of the block's lanes).
     constexpr bool kBlocked = WP + kBlockMin - 1 <= 32;
-    constexpr bool kDcInRegs = kBlocked && S > 1;
+    static_assert(!kBlocked || S > 1, "the blocked form has warps beside the window warp");
+    constexpr bool kDcInRegs = kBlocked;
     const int ntr = RS - 32, tu = u - 32;
     const int dc_parts = max(1, ntr / M);
     float dcx[2] = {0.f, 0.f}, dcy[2] = {0.f, 0.f};
@@ -323,20 +329,25 @@ __global__ void __launch_bounds__(32 * S, 1) train_chunk_kernel(const ChunkArgs 
     const float *kcol = s_kmat + u;          // column u of the kernel table
     if constexpr (kBlocked) {
         // Blocked form.  Over a block of B = 32 - WP steps from n0, every sample that is in a
-        // window of the block lies in [n0 - WP + 1, n0 + B - 1]: 31 samples, one per lane of warp 0.
-        // That warp runs the B steps alone: the window lanes compute mu q beta (Eq. beta, written
-        // as beta = clamp(p, b - eps, b + eps) - p over kappa_jj), publish it in a 32-float ring and
-        // every lane adds the window sum to its own prediction with the kernel values held in
-        // registers; one warp barrier per step.  Since kappa(x_j, x_m) does not depend on the step,
-        // the block then moves every later sample m >= n0 + B by
-        //   sum_j kappa(x_j, x_m) sum_{n in block} mu q_n beta_j(n)
-        // at once: the lanes publish their summed updates and all threads apply them.
+        // window of the block lies in [n0 - WP + 1, n0 + B - 1]: 31 samples, one per lane of warp 0,
+        // which holds each one's residual d = b - f(x) and its kernel values against the others in
+        // registers and runs the B steps alone.  A step of the window warp is one dependent chain
+        // (mu q beta = mu q (max(d, eps) + min(d, -eps)) / kappa_jj, Eq. beta; one exchange through a
+        // 32-float ring; a WP-term sum in packed FMAs), so everything else stays off it:
+        //  * a block's summed coefficient changes move every later sample at once
+        //    (kappa(x_j, x_m) does not depend on the step); the window warp does that itself for the
+        //    next block's B new samples, the other warps for all later ones while the next block
+        //    runs, so that a block ends with a single CTA barrier nobody is waited for at;
+        //  * a lane's kernel values of its next block are loaded, a few per step, into a second
+        //    register set (rows B.. of that set become the next block's);
+        //  * outputs at arrival are kept in the lane and written at the end of the block.
         constexpr int B = 32 - WP;
         constexpr int NL = WP + B - 1;
-        float *s_p = s_beta, *s_g = s_p + RS, *s_b = s_g + RS, *s_rk = s_b + RS, *s_agg = s_rk + RS;  // [2][32]
+        constexpr int kLater = 2 * B < 32 ? 2 * B : 32;  // samples below it are never "later" ones
+        float *s_d = s_beta, *s_g = s_d + RS, *s_b = s_g + RS, *s_rk = s_b + RS, *s_agg = s_rk + RS;  // [2][32]
         float *s_w = s_agg + 64, *s_muq = s_w + 64;
         if (valid) {
-            s_p[u] = p;
+            s_d[u] = b - p;
             s_g[u] = gam;
             s_b[u] = b;
             s_rk[u] = rk;
@@ -346,174 +357,121 @@ __global__ void __launch_bounds__(32 * S, 1) train_chunk_kernel(const ChunkArgs 
             s_muq[u] = a.mu / (float)(u + 1);                 // mu q while the window is filling (n < W - 1)
             s_muqv[u] = u == 0 ? 0.f : a.mu / (float)u;       // mu q with q = 1/|V_n|, |V_n| = u
         }
-        for (int i = u; i < 64; i += RS) s_w[i] = 0.f;
         __syncthreads();
-        const int lane = u & 31;
-        // Tracking threads (warps 1..S-1, idle while warp 0 runs a block) keep the next chunk's
-        // samples: starting value during the first block, then each block's summed coefficient
-        // changes (published by warp 0) applied during the following block, kernel values from
-        // the next-chunk table in global memory (off the recurrence's critical path).
+        auto block_barrier = [] { asm volatile("bar.sync 2, %0;" ::"n"(RS) : "memory"); };
         const int n_next = track ? 2 * min(g.T, g.P - (t0 + Tc)) : 0;
-        float tp[2] = {0.f, 0.f};
-        // x~ = r(t) for r1(t) and -i r(t) for r2(t); lanes outside L carry a zero change
-        auto dc_apply = [&](const float *agg, int wl0b) {
-#pragma unroll
-            for (int it = 0; it < 2; ++it) {
-                const int idx = tu + it * ntr;
-                if (idx >= dc_parts * M) continue;
-                const int mm = idx % M, part = idx / M;
-                const int j0 = part * NL / dc_parts, j1 = (part + 1) * NL / dc_parts;
-                for (int j = j0; j < j1; ++j) {
-                    const float d = agg[j];
-                    const int ms = wl0b + j;
-                    const int pi = min(max((ms >> 1) - pa0, 0), npil - 1);
-                    const float2 x = s_pil[pi * M + mm];
-                    if (ms & 1) { dcx[it] = fmaf(d, x.y, dcx[it]); dcy[it] = fmaf(-d, x.x, dcy[it]); }
-                    else        { dcx[it] = fmaf(d, x.x, dcx[it]); dcy[it] = fmaf(d, x.y, dcy[it]); }
-                }
-            }
-        };
-        // At this chunk's start the entries of L hold gamma only at the carried samples (the new
-        // ones start at 0), so the tracked part of f_{s0} at a next-chunk sample x is
-        //   w_L <w, x> + w_G sum_{carried j} gamma_j kappa_G(x_j, x)
-        //     = w_L <w - sum_{carried j} gamma_j x_j, x> + sum_{carried j} gamma_j kappa(x_j, x),
-        // the second form using the tabulated sum kernel; the tracking threads form the reduced
-        // filter, meet at a named barrier of their own, then evaluate their samples.
-        auto track_init = [&]() {
-            for (int mm = tu; mm < M; mm += ntr) {
-                float2 c = s_clin[mm];
-                for (int j = 0; j < nc; ++j) {
-                    const float d = -s_gcar[j];
-                    const float2 x = s_pil[(((l0 + j) >> 1) - pa0) * M + mm];
-                    if ((l0 + j) & 1) { c.x = fmaf(d, x.y, c.x); c.y = fmaf(-d, x.x, c.y); }
-                    else              { c.x = fmaf(d, x.x, c.x); c.y = fmaf(d, x.y, c.y); }
-                }
-                s_clinw[mm] = c;
-            }
-            asm volatile("bar.sync 1, %0;" ::"r"(ntr) : "memory");
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int v = tu + i * ntr;
-                if (v >= n_next) continue;
-                const int tv = t0 + Tc + (v >> 1), lvv = v & 1;
-                const float2 *rv = a.rx + (size_t)tv * M;
-                float l0s = 0.f, l1s = 0.f;
-                for (int mm = 0; mm < M; mm += 2) {
-                    const float4 x = __ldcg(reinterpret_cast<const float4 *>(rv + mm));
-                    const float2 c = s_clinw[mm], cb = s_clinw[mm + 1];
-                    l0s = lvv ? fmaf(c.x, x.y, fmaf(-c.y, x.x, l0s)) : fmaf(c.x, x.x, fmaf(c.y, x.y, l0s));
-                    l1s = lvv ? fmaf(cb.x, x.w, fmaf(-cb.y, x.z, l1s)) : fmaf(cb.x, x.z, fmaf(cb.y, x.w, l1s));
-                }
-                // s_gcar is zero past the carried samples; rows clamped into the table
-                float acc4[4] = {a.wL * (l0s + l1s), 0.f, 0.f, 0.f};
-#pragma unroll
-                for (int j = 0; j < 32; ++j)
-                    acc4[j & 3] = fmaf(s_gcar[j], __ldcg(a.kx + (size_t)min(j, R - 1) * g.KXS + v), acc4[j & 3]);
-                tp[i] = (acc4[0] + acc4[1]) + (acc4[2] + acc4[3]);
-            }
-        };
-        auto track_apply = [&](const float *agg, int r0) {
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int v = tu + i * ntr;
-                if (v >= n_next) continue;
-                // rows outside [0, R) belong to lanes whose summed change is zero: clamp, no branch,
-                // so that all NL loads are in flight together
-                float kv[NL];
-#pragma unroll
-                for (int j = 0; j < NL; ++j) kv[j] = __ldcg(a.kx + (size_t)min(max(r0 + j, 0), R - 1) * g.KXS + v);
-                float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                for (int j = 0; j < NL; ++j) acc[j & 3] = fmaf(agg[j], kv[j], acc[j & 3]);
-                tp[i] += (acc[0] + acc[1]) + (acc[2] + acc[3]);
-            }
-        };
         int blk = 0;
-        for (int n0 = s0; n0 < s1; n0 += B, ++blk) {
-            const int wl0 = n0 - WP + 1;  // sample of lane 0
-            float *agg_cur = s_agg + (blk & 1) * 32;
-            if (S > 1 && u >= 32 && blk > 0) dc_apply(s_agg + ((blk - 1) & 1) * 32, wl0 - B);
-            if (S > 1 && track && u >= 32) {
-                if (blk == 0) track_init();
-                else track_apply(s_agg + ((blk - 1) & 1) * 32, wl0 - B - l0);
-            }
-            if (u < 32) {
-                const int ms = wl0 + lane, lu = ms - l0;
-                const bool lv = lane < NL && ms >= l0 && ms < s1;
-                const int col = lv ? lu : 0;
-                float pl = 0.f, c1 = 0.f, c2 = 0.f, rkl = 0.f, agg = 0.f, bl = 0.f;
-                if (lv) {
-                    pl = s_p[lu];
-                    bl = s_b[lu];
-                    c1 = bl - a.eps;  // the hyperslab [b - eps, b + eps]
-                    c2 = bl + a.eps;
-                    rkl = s_rk[lu];
-                }
-                float kc[NL];  // kappa(x_{wl0+j}, x of this lane)
+        if (u < 32) {
+            // ================= window warp =================
+            constexpr int NP = (32 + B) / 2;               // row pairs a lane loads for its next sample
+            constexpr int kPairsPerStep = (NP + B - 1) / B;
+            const int lane = u;
+            const int lw = lane - (WP - W);
+            bool lv = lane < NL && s0 - WP + 1 + lane >= l0 && s0 - WP + 1 + lane < s1;
+            int col = lv ? s0 - WP + 1 + lane - l0 : 0;
+            float d = lv ? s_d[col] : 0.f, bl = lv ? s_b[col] : 0.f, rkl = lv ? s_rk[col] : 0.f;
+            // kernel values against rows [wl0, wl0 + 32) in row pairs (row 31 meets a zero change only;
+            // rows outside the live range are zero rows)
+            uint64_t kc[16], kn[NP];
 #pragma unroll
-                for (int j = 0; j < NL; ++j) {
-                    // rows >= -WP + 1 (the zero rows); rows past R belong to invalid lanes, whose
-                    // beta is 0: clamp instead of branching so that the loads issue together
-                    kc[j] = s_kmat[min(wl0 + j - l0, R - 1) * RS + col];
-                }
-                // kChecked: a partial last block, the filling window (n < W - 1), case logging,
-                // outputs at arrival or decided targets; kViol: weights on the violated slabs
+            for (int i = 0; i < 16; ++i) {
+                const float *kr = s_kmat + (s0 - WP + 1 - l0 + 2 * i) * RS + col;
+                kc[i] = pack2(kr[0], kr[RS]);
+            }
+            for (int n0 = s0; n0 < s1; n0 += B, ++blk) {
+                const int wl0 = n0 - WP + 1, ms = wl0 + lane;  // sample of lane 0, of this lane
+                const bool has_next = n0 + B < s1;
+                const bool lvn = has_next && lane < NL && ms + B >= l0 && ms + B < s1;
+                const int coln = lvn ? ms + B - l0 : 0;      // the sample this lane holds in the next block
+                const float *krow = s_kmat + (has_next ? (wl0 - l0) * RS + coln : 0);
+                const float nsc_full = -muq_full * rkl;      // -mu q / kappa_jj (0 in a lane without a sample)
+                float gn = 0.f, evn = 0.f, darr = 0.f;       // minus the summed change; evictions at coln
+                const float b_before = bl;
+                // kChecked: a partial last block, the filling window (n < W - 1) or case logging;
+                // kViol: weights on the violated slabs
                 auto steps = [&](auto checked_c, auto evict_c, auto viol_c) {
                     constexpr bool kChecked = decltype(checked_c)::value, kEvict = decltype(evict_c)::value;
                     constexpr bool kViol = decltype(viol_c)::value;
 #pragma unroll
                     for (int s = 0; s < B; ++s) {
                         const int n = n0 + s;
-                        if (kChecked && n >= s1) break;
+                        if (kChecked && n >= s1) {  // (only in the last block, which loads nothing ahead)
+                            break;
+                        }
                         if (kEvict && !(n & 1) && (n >> 1) + tb >= D) {
                             const int e = (n >> 1) - t0;
-                            pl -= a.wG * fmaf(s_egam[2 * e], s_gev[e * 2 * RS + col],
-                                              s_egam[2 * e + 1] * s_gev[(e * 2 + 1) * RS + col]);
+                            const float e0 = s_egam[2 * e], e1 = s_egam[2 * e + 1];
+                            const float *ge = s_gev + e * 2 * RS;
+                            d = fmaf(a.wG, fmaf(e0, ge[col], e1 * ge[RS + col]), d);
+                            evn = fmaf(a.wG, fmaf(e0, ge[coln], e1 * ge[RS + coln]), evn);
                         }
-                        if (kExt && kChecked && lane == s + WP - 1) {  // sample n arrives: pl = f_n(x_n)
-                            if (a.soft_out) a.soft_out[((size_t)((n - n_first) >> 1) * K + k) * 2 + (n & 1)] = pl;
-                            if (a.decide) {  // its target: the decision on the filter's own output
-                                bl = pam_value(pam_level(pl, a.qam_half, a.qam_a), a.qam_half, a.qam_a);
-                                c1 = bl - a.eps;
-                                c2 = bl + a.eps;
+                        if constexpr (kExt) {  // sample n arrives with f_n(x_n) = b - d
+                            const bool arrives = lane == s + WP - 1;
+                            darr = arrives ? d : darr;
+                            if (a.decide) {  // its target: the decision on the filter's own output -d
+                                const float bd = a.qam_half == 1
+                                                     ? (d <= 0.f ? a.qam_a : -a.qam_a)
+                                                     : pam_value(pam_level(-d, a.qam_half, a.qam_a), a.qam_half, a.qam_a);
+                                bl = arrives ? bd : bl;
+                                d = arrives ? d + bd : d;
                             }
                         }
                         // window J_n = samples [n - W + 1, n] = lanes [s + WP - W, s + WP - 1]
-                        const bool inw = lv && lane >= s + WP - W && lane <= s + WP - 1;
-                        float muq;
+                        const bool inw = (unsigned)(lw - s) < (unsigned)W;
+                        float nsc;
                         if constexpr (kViol) {  // mu q with q = 1/|V_n| on the violated slabs
-                            const bool viol = inw && (pl < c1 || pl > c2);
-                            muq = s_muqv[__popc(__ballot_sync(0xffffffffu, viol))];
-                        } else {                // mu q with q = 1/|J_n|
-                            muq = kChecked && n + sb < W - 1 ? s_muq[n + sb] : muq_full;
+                            const bool viol = inw && lv && fabsf(d) > a.eps;
+                            const float muq = s_muqv[__popc(__ballot_sync(0xffffffffu, viol))];  // (every lane)
+                            nsc = inw ? -muq * rkl : 0.f;
+                        } else if (kChecked && n + sb < W - 1) {  // mu q with q = 1/|J_n|
+                            nsc = inw ? -s_muq[n + sb] * rkl : 0.f;
+                        } else {
+                            nsc = inw ? nsc_full : 0.f;
                         }
-                        const float sc = inw ? muq * rkl : 0.f;
-                        const float mb = (fminf(fmaxf(pl, c1), c2) - pl) * sc;  // mu q beta_j
-                        agg += mb;
-                        if (kChecked && log_cases && inw)
-                            a.case_log[((size_t)(n - n_first) * W + (ms - n + W - 1)) * K + k] =
-                                (int8_t)(pl < c1 ? -1 : (pl > c2 ? 1 : 0));
+                        const float nm = (fmaxf(d, a.eps) + fminf(d, -a.eps)) * nsc;  // -mu q beta_j
                         float *ring = s_w + (s & 1) * 32;
-                        ring[lane] = mb;
+                        ring[lane] = nm;
+                        gn += nm;
+                        if (kChecked && log_cases && inw && lv)
+                            a.case_log[((size_t)(n - n_first) * W + (ms - n + W - 1)) * K + k] =
+                                (int8_t)(d > a.eps ? -1 : (d < -a.eps ? 1 : 0));
                         __syncwarp();
-                        float acc[4] = {pl, 0.f, 0.f, 0.f};
-                        const int b4 = s & ~3;
+                        // lanes outside the window hold 0 in the ring: whole pairs around it
+                        uint64_t acc[4];
+                        acc[0] = pack2(d, 0.f);
+                        constexpr int kMaxPairs = WP / 2 + 1;
+                        uint64_t rv[kMaxPairs + 2];
+                        const int p0 = (s >> 1) & ~1, np = ((s + WP + 1) >> 1) - (s >> 1), off = (s >> 1) - p0;
 #pragma unroll
-                        for (int q4 = 0; q4 < WP + 4; q4 += 4) {
-                            const float4 v = *reinterpret_cast<const float4 *>(ring + b4 + q4);
-                            const float vv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                            for (int r = 0; r < 4; ++r) {
-                                const int j = b4 + q4 + r;
-                                if (j >= s && j < s + WP) acc[(j - s) & 3] = fmaf(vv[r], kc[j], acc[(j - s) & 3]);
+                        for (int q = 0; q < kMaxPairs + 1; q += 2) {
+                            if (q < np + off) {
+                                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(ring + 2 * (p0 + q));
+                                rv[q] = v.x;
+                                rv[q + 1] = v.y;
                             }
                         }
-                        pl = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+#pragma unroll
+                        for (int q = 0; q < kPairsPerStep; ++q) {  // the next block's kernel values
+                            const int i = s * kPairsPerStep + q;
+                            if (i < NP) kn[i] = pack2(krow[2 * i * RS], krow[(2 * i + 1) * RS]);
+                        }
+#pragma unroll
+                        for (int q = 0; q < kMaxPairs; ++q) {
+                            if (q < np) {
+                                const uint64_t kv = kc[(s >> 1) + q];
+                                if (q == 0 || q >= 4) acc[q & 3] = ffma2(rv[off + q], kv, acc[q & 3]);
+                                else acc[q] = fmul2(rv[off + q], kv);
+                            }
+                        }
+                        if (np > 1) acc[0] = fadd2(acc[0], acc[1]);
+                        if (np > 3) acc[2] = fadd2(acc[2], acc[3]);
+                        if (np > 2) acc[0] = fadd2(acc[0], acc[2]);
+                        d = sum2(acc[0]);
                     }
                 };
                 using T_ = std::true_type;
                 using F_ = std::false_type;
-                const bool checked = n0 + B > s1 || n0 + sb < W - 1 || log_cases || (kExt && (a.decide || a.soft_out));
+                const bool checked = n0 + B > s1 || n0 + sb < W - 1 || log_cases;
                 if (kExt && a.qviol) {
                     if constexpr (kExt) {
                         if (evict) steps(T_{}, T_{}, T_{});
@@ -526,46 +484,183 @@ __global__ void __launch_bounds__(32 * S, 1) train_chunk_kernel(const ChunkArgs 
                     if (checked) steps(T_{}, F_{}, F_{});
                     else steps(F_{}, F_{}, F_{});
                 }
+                float *agg = s_agg + (blk & 1) * 32;
+                agg[lane] = lv ? -gn : 0.f;
                 if (lv) {
-                    s_p[lu] = pl;
-                    s_g[lu] += agg;
-                    s_b[lu] = bl;
+                    s_d[col] = d;
+                    s_g[col] -= gn;
+                    if (kExt) s_b[col] = bl;
+                    if (kExt && a.soft_out && lane >= WP - 1)
+                        a.soft_out[((size_t)((ms - n_first) >> 1) * K + k) * 2 + (ms & 1)] = b_before - darr;
                 }
-                agg_cur[lane] = lv ? agg : 0.f;
-            }
-            __syncthreads();
-            // the block's moves of every later sample, and its dropped entries
-            if (valid && m >= n0 + B) {
-                const int r0 = wl0 - l0;
-                float acc[4] = {0.f, 0.f, 0.f, 0.f};
+                if (has_next) {  // the block's move of this lane's next sample, if it is a new one
+                    __syncwarp();
+                    uint64_t acc[4];
 #pragma unroll
-                for (int j = 0; j < NL; ++j)  // rows past R: lanes with zero change (rows < 0: zero rows)
-                    acc[j & 3] = fmaf(agg_cur[j], kcol[min(r0 + j, R - 1) * RS], acc[j & 3]);
-                float pv = s_p[u] + ((acc[0] + acc[1]) + (acc[2] + acc[3]));
-                if (evict) {
-                    for (int n = n0 + (n0 & 1); n < min(n0 + B, s1); n += 2) {
-                        if ((n >> 1) + tb < D) continue;
-                        const int e = (n >> 1) - t0;
-                        pv -= a.wG * fmaf(s_egam[2 * e], s_gev[e * 2 * RS + u],
-                                          s_egam[2 * e + 1] * s_gev[(e * 2 + 1) * RS + u]);
+                    for (int i = 0; i < 16; i += 2) {
+                        const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(agg + 2 * i);
+                        if (i < 4) {
+                            acc[i] = fmul2(v.x, kn[i]);
+                            acc[i + 1] = fmul2(v.y, kn[i + 1]);
+                        } else {
+                            acc[i & 3] = ffma2(v.x, kn[i], acc[i & 3]);
+                            acc[(i + 1) & 3] = ffma2(v.y, kn[i + 1], acc[(i + 1) & 3]);
+                        }
+                    }
+                    const float move = sum2(fadd2(fadd2(acc[0], acc[1]), fadd2(acc[2], acc[3])));
+                    block_barrier();  // the blocks before this one have reached the next block's samples
+                    const float d_old = __shfl_down_sync(0xffffffffu, d, B);
+                    d = lane < WP - 1 ? d_old : s_d[coln] + (evn - move);
+                    lv = lvn;
+                    col = coln;
+                    bl = lv ? s_b[col] : 0.f;
+                    rkl = lv ? s_rk[col] : 0.f;
+                    d = lv ? d : 0.f;
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) kc[i] = kn[i + B / 2];
+                } else {
+                    block_barrier();
+                }
+            }
+        } else {
+            // ================= the other warps =================
+            float tp[2] = {0.f, 0.f};  // tracked part of f at this thread's next-chunk samples
+            // filter change of one block: x~ = r(t) for r1(t) and -i r(t) for r2(t); lanes outside L
+            // carry a zero change
+            auto dc_apply = [&](const float *agg, int wl0b) {
+#pragma unroll
+                for (int it = 0; it < 2; ++it) {
+                    const int idx = tu + it * ntr;
+                    if (idx >= dc_parts * M) continue;
+                    const int mm = idx % M, part = idx / M;
+                    const int j0 = part * NL / dc_parts, j1 = (part + 1) * NL / dc_parts;
+                    for (int j = j0; j < j1; ++j) {
+                        const float dg = agg[j];
+                        const int ms = wl0b + j;
+                        const int pi = min(max((ms >> 1) - pa0, 0), npil - 1);
+                        const float2 x = s_pil[pi * M + mm];
+                        if (ms & 1) { dcx[it] = fmaf(dg, x.y, dcx[it]); dcy[it] = fmaf(-dg, x.x, dcy[it]); }
+                        else        { dcx[it] = fmaf(dg, x.x, dcx[it]); dcy[it] = fmaf(dg, x.y, dcy[it]); }
                     }
                 }
-                s_p[u] = pv;
-            }
-            __syncthreads();
-        }
-        if (S > 1 && u >= 32 && blk > 0) dc_apply(s_agg + ((blk - 1) & 1) * 32, s0 + (blk - 1) * B - WP + 1);
-        if (S > 1 && track && u >= 32) {  // the last block's changes, then hand over
-            if (blk == 0) track_init();
-            else track_apply(s_agg + ((blk - 1) & 1) * 32, s0 + (blk - 1) * B - WP + 1 - l0);
+            };
+            // At this chunk's start the entries of L hold gamma only at the carried samples (the new
+            // ones start at 0), so the tracked part of f_{s0} at a next-chunk sample x is
+            //   w_L <w, x> + w_G sum_{carried j} gamma_j kappa_G(x_j, x)
+            //     = w_L <w - sum_{carried j} gamma_j x_j, x> + sum_{carried j} gamma_j kappa(x_j, x),
+            // the second form using the tabulated sum kernel; the tracking threads form the reduced
+            // filter, meet at a named barrier of their own, then evaluate their samples.
+            auto track_init = [&]() {
+                for (int mm = tu; mm < M; mm += ntr) {
+                    float2 c = s_clin[mm];
+                    for (int j = 0; j < nc; ++j) {
+                        const float dg = -s_gcar[j];
+                        const float2 x = s_pil[(((l0 + j) >> 1) - pa0) * M + mm];
+                        if ((l0 + j) & 1) { c.x = fmaf(dg, x.y, c.x); c.y = fmaf(-dg, x.x, c.y); }
+                        else              { c.x = fmaf(dg, x.x, c.x); c.y = fmaf(dg, x.y, c.y); }
+                    }
+                    s_clinw[mm] = c;
+                }
+                asm volatile("bar.sync 1, %0;" ::"r"(ntr) : "memory");
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int v = tu + i * ntr;
-                if (v < n_next) a.track_out[v * K + k] = tp[i];
+                for (int i = 0; i < 2; ++i) {
+                    const int v = tu + i * ntr;
+                    if (v >= n_next) continue;
+                    const int tv = t0 + Tc + (v >> 1), lvv = v & 1;
+                    const float2 *rv = a.rx + (size_t)tv * M;
+                    float l0s = 0.f, l1s = 0.f;
+                    for (int mm = 0; mm < M; mm += 2) {
+                        const float4 x = __ldcg(reinterpret_cast<const float4 *>(rv + mm));
+                        const float2 c = s_clinw[mm], cb = s_clinw[mm + 1];
+                        l0s = lvv ? fmaf(c.x, x.y, fmaf(-c.y, x.x, l0s)) : fmaf(c.x, x.x, fmaf(c.y, x.y, l0s));
+                        l1s = lvv ? fmaf(cb.x, x.w, fmaf(-cb.y, x.z, l1s)) : fmaf(cb.x, x.z, fmaf(cb.y, x.w, l1s));
+                    }
+                    // s_gcar is zero past the carried samples; rows clamped into the table
+                    float acc4[4] = {a.wL * (l0s + l1s), 0.f, 0.f, 0.f};
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        acc4[j & 3] = fmaf(s_gcar[j], __ldcg(a.kx + (size_t)min(j, R - 1) * g.KXS + v), acc4[j & 3]);
+                    tp[i] = (acc4[0] + acc4[1]) + (acc4[2] + acc4[3]);
+                }
+            };
+            auto track_apply = [&](const float *agg, int r0) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    const int v = tu + i * ntr;
+                    if (v >= n_next) continue;
+                    // rows outside [0, R) belong to lanes whose summed change is zero: clamp, no branch,
+                    // so that all NL loads are in flight together
+                    float kv[NL];
+#pragma unroll
+                    for (int j = 0; j < NL; ++j) kv[j] = __ldcg(a.kx + (size_t)min(max(r0 + j, 0), R - 1) * g.KXS + v);
+                    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                    for (int j = 0; j < NL; ++j) acc[j & 3] = fmaf(agg[j], kv[j], acc[j & 3]);
+                    tp[i] += (acc[0] + acc[1]) + (acc[2] + acc[3]);
+                }
+            };
+            // block bb (steps from nb): its moves of the samples from nb + 2 B on, and its dropped entries
+            auto near_apply = [&](const float *agg, int nb) {
+                const int r0 = nb - WP + 1 - l0;
+                for (int i = kLater + tu; i < R; i += ntr) {
+                    if (l0 + i < nb + 2 * B) continue;
+                    const float *kr = s_kmat + r0 * RS + i;
+                    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                    for (int j = 0; j < NL; ++j) acc[j & 3] = fmaf(agg[j], kr[j * RS], acc[j & 3]);
+                    float dv = s_d[i] - ((acc[0] + acc[1]) + (acc[2] + acc[3]));
+                    if (evict) {
+                        for (int n = nb + (nb & 1); n < nb + B; n += 2) {
+                            if ((n >> 1) + tb < D) continue;
+                            const int e = (n >> 1) - t0;
+                            dv = fmaf(a.wG, fmaf(s_egam[2 * e], s_gev[e * 2 * RS + i],
+                                                 s_egam[2 * e + 1] * s_gev[(e * 2 + 1) * RS + i]), dv);
+                        }
+                    }
+                    s_d[i] = dv;
+                }
+            };
+            for (int n0 = s0; n0 < s1; n0 += B, ++blk) {
+                if (blk == 0) {
+                    if (track) track_init();
+                } else {
+                    const float *agg = s_agg + ((blk - 1) & 1) * 32;
+                    near_apply(agg, n0 - B);
+                    dc_apply(agg, n0 - B - WP + 1);
+                    if (track) track_apply(agg, n0 - B - WP + 1 - l0);
+                }
+                if (n0 + B >= s1) {
+                    // beside the last block: the chunk's new dictionary entries (slot (tb + t) % D) and
+                    // their norms, spread over the K user CTAs, which all hold the chunk's pilots
+                    for (int i = k * ntr + tu; i < Tc * M; i += K * ntr) {
+                        const int t = t0 + i / M, mm = i % M;
+                        a.dict[(size_t)((tb + t) % D) * M + mm] = s_pil[(t - pa0) * M + mm];
+                    }
+                    for (int i = k * ntr + tu; i < Tc; i += K * ntr) {
+                        const float2 *rv = s_pil + (t0 + i - pa0) * M;
+                        float nrm = 0.f;
+                        for (int mm = 0; mm < M; ++mm) nrm = fmaf(rv[mm].x, rv[mm].x, fmaf(rv[mm].y, rv[mm].y, nrm));
+                        a.dict_norm[(tb + t0 + i) % D] = nrm;
+                    }
+                }
+                block_barrier();
+            }
+            if (blk > 0) {  // the last block's changes, then hand over
+                const float *agg = s_agg + ((blk - 1) & 1) * 32;
+                const int wl0 = s0 + (blk - 1) * B - WP + 1;
+                dc_apply(agg, wl0);
+                if (track) {
+                    track_apply(agg, wl0 - l0);
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        const int v = tu + i * ntr;
+                        if (v < n_next) a.track_out[v * K + k] = tp[i];
+                    }
+                }
             }
         }
         if (valid) {
-            p = s_p[u];
+            p = s_b[u] - s_d[u];
             gam = s_g[u];
             b = s_b[u];
         }
@@ -744,12 +839,12 @@ __global__ void __launch_bounds__(32 * S, 1) train_chunk_kernel(const ChunkArgs 
     }
 
     // ---- new dictionary entries of this chunk (slot (tb + t) % D), their norms, bookkeeping --
-    // (spread over the K user CTAs, which all hold the chunk's pilots)
-    for (int i = k * RS + u; i < Tc * M; i += K * RS) {
+    // (the blocked form has written them beside its last block)
+    for (int i = k * RS + u; !kBlocked && i < Tc * M; i += K * RS) {
         const int t = t0 + i / M, mm = i % M;
         a.dict[(size_t)((tb + t) % D) * M + mm] = s_pil[(t - pa0) * M + mm];
     }
-    for (int i = k * RS + u; i < Tc; i += K * RS) {
+    for (int i = k * RS + u; !kBlocked && i < Tc; i += K * RS) {
         const float2 *rv = s_pil + (t0 + i - pa0) * M;
         float nrm = 0.f;
         for (int mm = 0; mm < M; ++mm) nrm = fmaf(rv[mm].x, rv[mm].x, fmaf(rv[mm].y, rv[mm].y, nrm));
