@@ -176,10 +176,10 @@ TrainGeom train_geom(const apsm_params *p, int P, int n_prev, int evict = -1) {
         g.T = T;
         g.RMAX = 2 * T + g.W;
         g.RS = round_up(g.RMAX, 32);
-        if (g.WP <= 24) g.RS = std::max(g.RS, 64);  // the blocked form: a warp besides the window warp
         g.KXS = round_up(2 * T, 32);
-        // tracking needs the blocked form (padded window <= 24), whose other warps do it
-        g.track = want_track && g.WP <= 24 && 2 * T <= 2 * (g.RS - 32) ? 1 : 0;
+        // tracking needs the blocked form (padded window <= 24), whose other warps do it, and a live
+        // range of more than one warp
+        g.track = want_track && g.WP <= 24 && g.RS >= 64 && 2 * T <= 2 * (g.RS - 32) ? 1 : 0;
         if (T == 1 || ChunkSmem(g).bytes <= kMaxSmemBytes) break;
     }
     g.n_chunks = P > 0 ? (P + T - 1) / T : 0;
@@ -447,7 +447,7 @@ apsm_status train_run(const apsm_params *p, const float *rx_in, const float *sym
     const ChunkSmem layout(g);
     // the extended instantiation only for the modes that need it
     const bool ext_modes = decide || soft != nullptr || hard != nullptr || p->weights == APSM_Q_VIOLATED;
-    const ChunkLauncher chunk = chunk_launcher(g.RS / 32, g.WP, ext_modes);
+    const ChunkLauncher chunk = chunk_launcher(chunk_warps(g.RS, g.WP), g.WP, ext_modes);
     if (!chunk) return APSM_ERR_UNSUPPORTED;
 
     // phase A: the partial Gaussian sums of f, at the extended pilots [q0, q0 + nq), over the

@@ -43,7 +43,7 @@ struct TrainGeom {
     int T;         // pilots per chunk
     int n_chunks;
     int RMAX;      // 2T + W: live-range capacity
-    int RS;        // row stride of the per-chunk kernel tables: RMAX rounded up to 32
+    int RS;        // row stride of the per-chunk kernel tables in the workspace: RMAX rounded up to 32
     int WP;        // window W rounded up to a supported multiple of 4
     int slice;     // entries per phase-A slice
     int KXS;       // row stride of the next-chunk table: 2T rounded up to 32
@@ -135,11 +135,17 @@ constexpr int kBlockMin = 8;  // shortest step block of the blocked form (padded
 // row sets of a block that may end past it.
 __host__ __device__ constexpr int chunk_zero_rows(int WP) { return WP + kBlockMin <= 32 ? 32 - WP : 0; }
 
+// Warps of the phase-B CTA for a live-range table stride RS: one thread per live-range sample, in
+// the blocked form at least one warp besides the window warp.
+__host__ __device__ constexpr int chunk_warps(int RS, int WP) {
+    return WP + kBlockMin <= 32 && RS < 64 ? 2 : RS / 32;
+}
+
 // Shared-memory layout of phase B (bytes; every region 16-byte aligned).
 struct ChunkSmem {
     int bar, kmat, gev, egam, beta, dg, tgt, clin, pil, trk, bytes;
     __host__ __device__ ChunkSmem(const TrainGeom &g) {
-        const int RS = g.RS;
+        const int RS = chunk_warps(g.RS, g.WP) * 32;
         const int npil = g.T + (g.W + 1) / 2 + 1;
         bar = 0;
         kmat = 16;                                   // WP zero rows, RS rows of RS, the zero rows after them
@@ -166,10 +172,8 @@ template <int S, int WP, bool kExt>
 __global__ void __launch_bounds__(32 * S, 1) train_chunk_kernel(const ChunkArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int RS = 32 * S;
-    if (a.pdl_mode == 0) {
-        pdl_wait();
-        pdl_trigger();
-    }
+    constexpr bool kBlocked = WP + kBlockMin - 1 <= 32;
+    static_assert(!kBlocked || S > 1, "the blocked form has warps beside the window warp");
     const TrainGeom &g = a.g;
     const ChunkSmem L(g);
     uint64_t *bar = reinterpret_cast<uint64_t *>(smem + L.bar);
@@ -197,17 +201,13 @@ __global__ void __launch_bounds__(32 * S, 1) train_chunk_kernel(const ChunkArgs 
     const int n_first = 2 * g.nc0;  // first sample this call trains on (case log / outputs index from it)
     const bool evict = (tb + t0 + Tc - 1) >= D;
 
-    // ---- stage the chunk's kernel tables and pilots with the bulk-copy engine ---------------
     if (u == 0) {
         mbar_init(bar, 1);
         fence_mbar_init();
-        const uint32_t kb = (uint32_t)R * RS * 4, gb = evict ? (uint32_t)Tc * 2 * RS * 4 : 0u,
-                       pb = (uint32_t)npil * M * 8;
-        mbar_arrive_expect_tx(bar, kb + gb + pb);
-        bulk_g2s(s_kmat, a.kmat + (size_t)a.chunk * RS * RS, kb, bar);
-        if (evict) bulk_g2s(s_gev, a.gev + (size_t)a.chunk * g.T * 2 * RS, gb, bar);
-        bulk_g2s(s_pil, a.rx + (size_t)pa0 * M, pb, bar);
     }
+    for (int i = u; i < 2 * (WP + RS); i += RS) s_beta[i] = 0.f;
+    for (int i = u; i < WP * RS; i += RS) s_kmat[i - WP * RS] = 0.f;
+    for (int i = u; i < chunk_zero_rows(WP) * RS; i += RS) s_kmat[R * RS + i] = 0.f;
     __syncthreads();  // the barrier's initialisation is visible before any thread waits on it
     const bool valid = u < R;
     const int m = l0 + u, pa = m >> 1, l = m & 1;
@@ -220,10 +220,25 @@ __global__ void __launch_bounds__(32 * S, 1) train_chunk_kernel(const ChunkArgs 
             b = l ? sy.y : sy.x;  // b_{2t} = Re b(t), b_{2t+1} = Im b(t)
         }
     };
-    if (!a.decide) read_target();
-    for (int i = u; i < 2 * (WP + RS); i += RS) s_beta[i] = 0.f;
-    for (int i = u; i < WP * RS; i += RS) s_kmat[i - WP * RS] = 0.f;
-    for (int i = u; i < chunk_zero_rows(WP) * RS; i += RS) s_kmat[R * RS + i] = 0.f;
+    // ---- the chunk's kernel tables and pilots, staged with the bulk-copy engine ---------------
+    auto stage = [&]() {
+        if (u == 0) {
+            const uint32_t kb = (uint32_t)R * g.RS * 4, gb = evict ? (uint32_t)Tc * 2 * g.RS * 4 : 0u,
+                           pb = (uint32_t)npil * M * 8;
+            mbar_arrive_expect_tx(bar, kb + gb + pb);
+            const float *km = a.kmat + (size_t)a.chunk * g.RS * g.RS, *ge = a.gev + (size_t)a.chunk * g.T * 2 * g.RS;
+            if (g.RS == RS) {
+                bulk_g2s(s_kmat, km, kb, bar);
+                if (evict) bulk_g2s(s_gev, ge, gb, bar);
+            } else {  // a live range of one warp in the blocked form: rows of 32 into rows of 64
+                for (int r = 0; r < R; ++r) bulk_g2s(s_kmat + r * RS, km + r * g.RS, g.RS * 4, bar);
+                for (int r = 0; evict && r < 2 * Tc; ++r) bulk_g2s(s_gev + r * RS, ge + r * g.RS, g.RS * 4, bar);
+            }
+            bulk_g2s(s_pil, a.rx + (size_t)pa0 * M, pb, bar);
+        }
+        if (!a.decide) read_target();
+    };
+    if (a.pdl_mode != 0) stage();  // (mode 0: the previous launch may still be writing the tables)
     float rk = 0.f;  // 1 / kappa(x_j, x_j)
     // Every thread reaches this wait; the CTA votes on its outcome so that either all threads
     // go on or all leave together (no thread may skip a later barrier the others wait at).
@@ -238,88 +253,98 @@ __global__ void __launch_bounds__(32 * S, 1) train_chunk_kernel(const ChunkArgs 
         }
         return true;
     };
-    if (a.pdl_mode == 1) {  // the staged tables do not depend on the previous chunk
-        if (!tables_ready()) return;
-        pdl_wait();
-        pdl_trigger();
-    }
-    // every global load of the prologue is issued before the first use (one round trip)
-    if (a.decide) read_target();
-    float2 clin_r[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};  // M <= 64 <= 2 RS
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-        if (u + i * RS < M) clin_r[i] = __ldcg(a.clin + (u + i * RS) * K + k);
-    // coefficients of the entries dropped in this chunk (entry t0+e-D at step 2(t0+e))
-    // (the dropped entry and the arriving one share the slot (tb + t0 + e) mod D)
-    float egam_r = 0.f;
-    if (evict && u < 2 * Tc && tb + t0 + (u >> 1) >= D)
-        egam_r = __ldcg(a.gamma + ((size_t)((tb + t0 + (u >> 1)) % D) * 2 + (u & 1)) * K + k);
-
-    // ---- this thread's sample: target, coefficient, prediction at chunk start ---------------
-    float p = 0.f, gam = 0.f;
-    if (valid) {
-        if (m < s0) {
-            if (!a.fresh_carry) p = __ldcg(a.carry + u * K + k);
-            gam = __ldcg(a.gamma + ((size_t)((tb + pa) % D) * 2 + l) * K + k);
-        } else if (a.track_in) {
-            p = __ldcg(a.track_in + (m - s0) * K + k);
-        }
-    }
-    const float gam0 = gam;
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-        if (u + i * RS < M) s_clin[u + i * RS] = clin_r[i];
-    if (evict && u < 2 * Tc) s_egam[u] = egam_r;
-    // carried gamma at the chunk start (zero past the carried samples), for the tracking threads
     const bool track = a.track_out != nullptr;  // (the region exists only in the tracked form)
-    if (track && u < 32) s_gcar[u] = (valid && m < s0) ? gam : 0.f;
-    __syncthreads();
-    if (a.pdl_mode != 1 && !tables_ready()) return;
-    // samples whose prediction starts from phase A: the chunk's new ones (untracked form), and
-    // in the first chunk of a continuation also the carried ones
-    const bool from_a = valid && ((m >= s0 && !a.track_in) || (m < s0 && a.fresh_carry));
-    if (from_a) {  // linear part w_L <w, x_m> = w_L Re / Im (c^H r) at chunk start
-        // each pilot starts at its own antenna so the lanes of a warp hit distinct banks
-        const float2 *rv = s_pil + (pa - pa0) * M;
-        float lin0 = 0.f, lin1 = 0.f;
-        int mm = pa % M;
-        for (int i = 0; i < M; i += 2) {
-            const int mb = mm + 1 == M ? 0 : mm + 1;
-            const float2 c = s_clin[mm], x = rv[mm], cb = s_clin[mb], xb = rv[mb];
-            lin0 = l ? fmaf(c.x, x.y, fmaf(-c.y, x.x, lin0)) : fmaf(c.x, x.x, fmaf(c.y, x.y, lin0));
-            lin1 = l ? fmaf(cb.x, xb.y, fmaf(-cb.y, xb.x, lin1)) : fmaf(cb.x, xb.x, fmaf(cb.y, xb.y, lin1));
-            mm = mb + 1 == M ? 0 : mb + 1;
+    const int nc = s0 - l0;                     // carried samples (rows 0 .. nc-1 of the tables)
+    float p = 0.f, gam = 0.f, gam0 = 0.f;
+    // What the previous launches wrote: this thread's sample (coefficient, prediction at the chunk
+    // start), the filter, the dropped entries' coefficients.  False: the tables never arrived.
+    auto prologue = [&]() -> bool {
+        if (a.pdl_mode != 2) {
+            pdl_wait();
+            pdl_trigger();
         }
-        p = a.wL * (lin0 + lin1);
-    }
-    // In mode 2 everything above reads only what the previous chunk's phase B (complete before
-    // this kernel could launch) and the kernel tables wrote; the phase-A sums need phase A itself.
-    if (a.pdl_mode == 2) {
-        pdl_wait();
-        pdl_trigger();
-    }
-    if (valid && (m >= s0 || a.fresh_carry)) {
-        // Gaussian part of f_{s0}(x_m) from the phase-A slices: 32 loads in flight at a time,
-        // summed into eight partial sums (slice i into sum i mod 8) combined in a fixed order
-        const float *src = a.partial + (size_t)(pa - a.part_p0) * 2 * K + l * K + k;
+        if (a.pdl_mode == 0) stage();
+        // every global load is issued before the first use (one round trip)
+        if (a.decide) read_target();
+        float2 clin_r[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};  // M <= 64 <= 2 RS
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+            if (u + i * RS < M) clin_r[i] = __ldcg(a.clin + (u + i * RS) * K + k);
+        // coefficients of the entries dropped in this chunk (entry t0+e-D at step 2(t0+e))
+        // (the dropped entry and the arriving one share the slot (tb + t0 + e) mod D)
+        float egam_r = 0.f;
+        if (evict && u < 2 * Tc && tb + t0 + (u >> 1) >= D)
+            egam_r = __ldcg(a.gamma + ((size_t)((tb + t0 + (u >> 1)) % D) * 2 + (u & 1)) * K + k);
+        if (valid) {
+            if (m < s0) {
+                if (!a.fresh_carry) p = __ldcg(a.carry + u * K + k);
+                gam = __ldcg(a.gamma + ((size_t)((tb + pa) % D) * 2 + l) * K + k);
+            } else if (a.track_in) {
+                p = __ldcg(a.track_in + (m - s0) * K + k);
+            }
+        }
+        // Gaussian part of f_{s0}(x_m) from the phase-A slices: 32 loads in flight at a time (the
+        // first ones with the loads above, unless phase A may still run), summed into eight partial
+        // sums (slice i into sum i mod 8) combined in a fixed order
+        const bool from_part = valid && (m >= s0 || a.fresh_carry);
+        const float *src = a.partial + (from_part ? (size_t)(pa - a.part_p0) * 2 * K + l * K + k : 0);
         const size_t stride = (size_t)a.part_rows * 2 * K;
-        float gs[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        for (int sl = 0; sl < a.n_slices; sl += 32) {
-            float v[32];
+        float pv[32];
+        auto part_fetch = [&](int sl) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) v[j] = sl + j < a.n_slices ? __ldcg(src + (sl + j) * stride) : 0.f;
+            for (int j = 0; j < 32; ++j) pv[j] = from_part && sl + j < a.n_slices ? __ldcg(src + (sl + j) * stride) : 0.f;
+        };
+        if (a.pdl_mode != 2) part_fetch(0);
+        gam0 = gam;
 #pragma unroll
-            for (int j = 0; j < 32; ++j) gs[j & 7] += v[j];
+        for (int i = 0; i < 2; ++i)
+            if (u + i * RS < M) s_clin[u + i * RS] = clin_r[i];
+        if (evict && u < 2 * Tc) s_egam[u] = egam_r;
+        // carried gamma at the chunk start (zero past the carried samples), for the tracking threads
+        if (track && u < 32) s_gcar[u] = (valid && m < s0) ? gam : 0.f;
+        __syncthreads();
+        if (a.pdl_mode != 1 && !tables_ready()) return false;
+        // samples whose prediction starts from phase A: the chunk's new ones (untracked form), and
+        // in the first chunk of a continuation also the carried ones
+        const bool from_a = valid && ((m >= s0 && !a.track_in) || (m < s0 && a.fresh_carry));
+        if (from_a) {  // linear part w_L <w, x_m> = w_L Re / Im (c^H r) at chunk start
+            // each pilot starts at its own antenna so the lanes of a warp hit distinct banks
+            const float2 *rv = s_pil + (pa - pa0) * M;
+            float lin0 = 0.f, lin1 = 0.f;
+            int mm = pa % M;
+            for (int i = 0; i < M; i += 2) {
+                const int mb = mm + 1 == M ? 0 : mm + 1;
+                const float2 c = s_clin[mm], x = rv[mm], cb = s_clin[mb], xb = rv[mb];
+                lin0 = l ? fmaf(c.x, x.y, fmaf(-c.y, x.x, lin0)) : fmaf(c.x, x.x, fmaf(c.y, x.y, lin0));
+                lin1 = l ? fmaf(cb.x, xb.y, fmaf(-cb.y, xb.x, lin1)) : fmaf(cb.x, xb.x, fmaf(cb.y, xb.y, lin1));
+                mm = mb + 1 == M ? 0 : mb + 1;
+            }
+            p = a.wL * (lin0 + lin1);
         }
-        p = fmaf(a.wG, ((gs[0] + gs[1]) + (gs[2] + gs[3])) + ((gs[4] + gs[5]) + (gs[6] + gs[7])), p);
-    }
-    const int nc = s0 - l0;  // carried samples (rows 0 .. nc-1 of the tables)
+        // In mode 2 everything above reads only what the previous chunk's phase B (complete before
+        // this kernel could launch) and the kernel tables wrote; the phase-A sums need phase A itself.
+        if (a.pdl_mode == 2) {
+            pdl_wait();
+            pdl_trigger();
+            part_fetch(0);
+        }
+        if (from_part) {
+            float gs[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            for (int sl = 0; sl < a.n_slices; sl += 32) {
+                if (sl > 0) part_fetch(sl);
+#pragma unroll
+                for (int j = 0; j < 32; ++j) gs[j & 7] += pv[j];
+            }
+            p = fmaf(a.wG, ((gs[0] + gs[1]) + (gs[2] + gs[3])) + ((gs[4] + gs[5]) + (gs[6] + gs[7])), p);
+        }
+        return true;
+    };
+    if (a.pdl_mode == 1 && !tables_ready()) return;  // the staged tables do not depend on the previous chunk
+    if (!prologue()) return;
 
     // ---- the recurrence over the chunk's samples -----------------------------------------------
     // Blocked form with more than one warp: the idle warps also accumulate the filter change
     // c_k += sum_j dgamma_j x~_j block by block (thread = antenna x part of the block's lanes).
-    constexpr bool kBlocked = WP + kBlockMin - 1 <= 32;
-    static_assert(!kBlocked || S > 1, "the blocked form has warps beside the window warp");
     constexpr bool kDcInRegs = kBlocked;
     const int ntr = RS - 32, tu = u - 32;
     const int dc_parts = max(1, ntr / M);
@@ -329,338 +354,392 @@ __global__ void __launch_bounds__(32 * S, 1) train_chunk_kernel(const ChunkArgs 
     const float *kcol = s_kmat + u;          // column u of the kernel table
     if constexpr (kBlocked) {
         // Blocked form.  Over a block of B = 32 - WP steps from n0, every sample that is in a
-        // window of the block lies in [n0 - WP + 1, n0 + B - 1]: 31 samples, one per lane of warp 0,
-        // which holds each one's residual d = b - f(x) and its kernel values against the others in
-        // registers and runs the B steps alone.  A step of the window warp is one dependent chain
-        // (mu q beta = mu q (max(d, eps) + min(d, -eps)) / kappa_jj, Eq. beta; one exchange through a
-        // 32-float ring; a WP-term sum in packed FMAs), so everything else stays off it:
+        // window of the block lies in [n0 - WP + 1, n0 + B - 1]: 31 samples, one per lane of warp 0
+        // (the window warp), which holds each one's prediction and its kernel values against the
+        // others in registers and runs the B steps alone.  A step is one dependent chain (mu q beta,
+        // Eq. beta written as (clamp(p, b - eps, b + eps) - p) / kappa_jj; one exchange through a
+        // 32-float ring; a WP-term sum), so everything else stays off it:
         //  * a block's summed coefficient changes move every later sample at once
         //    (kappa(x_j, x_m) does not depend on the step); the window warp does that itself for the
         //    next block's B new samples, the other warps for all later ones while the next block
-        //    runs, so that a block ends with a single CTA barrier nobody is waited for at;
+        //    runs, so that a block ends with a single CTA barrier;
         //  * a lane's kernel values of its next block are loaded, a few per step, into a second
-        //    register set (rows B.. of that set become the next block's);
+        //    register set (rows B.. of that set become the next block's); the other warps load their
+        //    columns before the barrier that publishes the changes;
         //  * outputs at arrival are kept in the lane and written at the end of the block.
+        // The other warps' code is kept short (loops, constant strides): a chunk's first two blocks
+        // run it with cold instruction caches (the launches that the wait above lets in empty them).
+        // 16 antennas, 6 users, 1024 pilots, W = 16 (16 chunks of 128 steps): a block of 16 steps takes
+        // about 2050 cycles of the window warp (128 a step; 113 in the last chunk, where the other
+        // warps have nothing to track) + 300 at its end, the first two 4000 more together; training
+        // 277 us, against 342 us with two barriers per block and every later sample moved between them.
         constexpr int B = 32 - WP;
         constexpr int NL = WP + B - 1;
         constexpr int kLater = 2 * B < 32 ? 2 * B : 32;  // samples below it are never "later" ones
-        float *s_d = s_beta, *s_g = s_d + RS, *s_b = s_g + RS, *s_rk = s_b + RS, *s_agg = s_rk + RS;  // [2][32]
+        float *s_p = s_beta, *s_g = s_p + RS, *s_b = s_g + RS, *s_rk = s_b + RS, *s_agg = s_rk + RS;  // [2][32]
         float *s_w = s_agg + 64, *s_muq = s_w + 64;
-        if (valid) {
-            s_d[u] = b - p;
-            s_g[u] = gam;
-            s_b[u] = b;
-            s_rk[u] = rk;
-        }
         float *s_muqv = s_muq + 32;
         if (u < 32) {
             s_muq[u] = a.mu / (float)(u + 1);                 // mu q while the window is filling (n < W - 1)
             s_muqv[u] = u == 0 ? 0.f : a.mu / (float)u;       // mu q with q = 1/|V_n|, |V_n| = u
         }
-        __syncthreads();
         auto block_barrier = [] { asm volatile("bar.sync 2, %0;" ::"n"(RS) : "memory"); };
         const int n_next = track ? 2 * min(g.T, g.P - (t0 + Tc)) : 0;
         int blk = 0;
-        if (u < 32) {
-            // ================= window warp =================
-            constexpr int NP = (32 + B) / 2;               // row pairs a lane loads for its next sample
-            constexpr int kPairsPerStep = (NP + B - 1) / B;
-            const int lane = u;
-            const int lw = lane - (WP - W);
-            bool lv = lane < NL && s0 - WP + 1 + lane >= l0 && s0 - WP + 1 + lane < s1;
-            int col = lv ? s0 - WP + 1 + lane - l0 : 0;
-            float d = lv ? s_d[col] : 0.f, bl = lv ? s_b[col] : 0.f, rkl = lv ? s_rk[col] : 0.f;
-            // kernel values against rows [wl0, wl0 + 32) in row pairs (row 31 meets a zero change only;
-            // rows outside the live range are zero rows)
-            uint64_t kc[16], kn[NP];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const float *kr = s_kmat + (s0 - WP + 1 - l0 + 2 * i) * RS + col;
-                kc[i] = pack2(kr[0], kr[RS]);
-            }
-            for (int n0 = s0; n0 < s1; n0 += B, ++blk) {
-                const int wl0 = n0 - WP + 1, ms = wl0 + lane;  // sample of lane 0, of this lane
-                const bool has_next = n0 + B < s1;
-                const bool lvn = has_next && lane < NL && ms + B >= l0 && ms + B < s1;
-                const int coln = lvn ? ms + B - l0 : 0;      // the sample this lane holds in the next block
-                const float *krow = s_kmat + (has_next ? (wl0 - l0) * RS + coln : 0);
-                const float nsc_full = -muq_full * rkl;      // -mu q / kappa_jj (0 in a lane without a sample)
-                float gn = 0.f, evn = 0.f, darr = 0.f;       // minus the summed change; evictions at coln
-                const float b_before = bl;
-                // kChecked: a partial last block, the filling window (n < W - 1) or case logging;
-                // kViol: weights on the violated slabs
-                auto steps = [&](auto checked_c, auto evict_c, auto viol_c) {
-                    constexpr bool kChecked = decltype(checked_c)::value, kEvict = decltype(evict_c)::value;
-                    constexpr bool kViol = decltype(viol_c)::value;
-#pragma unroll
-                    for (int s = 0; s < B; ++s) {
-                        const int n = n0 + s;
-                        if (kChecked && n >= s1) {  // (only in the last block, which loads nothing ahead)
-                            break;
-                        }
-                        if (kEvict && !(n & 1) && (n >> 1) + tb >= D) {
-                            const int e = (n >> 1) - t0;
-                            const float e0 = s_egam[2 * e], e1 = s_egam[2 * e + 1];
-                            const float *ge = s_gev + e * 2 * RS;
-                            d = fmaf(a.wG, fmaf(e0, ge[col], e1 * ge[RS + col]), d);
-                            evn = fmaf(a.wG, fmaf(e0, ge[coln], e1 * ge[RS + coln]), evn);
-                        }
-                        if constexpr (kExt) {  // sample n arrives with f_n(x_n) = b - d
-                            const bool arrives = lane == s + WP - 1;
-                            darr = arrives ? d : darr;
-                            if (a.decide) {  // its target: the decision on the filter's own output -d
-                                const float bd = a.qam_half == 1
-                                                     ? (d <= 0.f ? a.qam_a : -a.qam_a)
-                                                     : pam_value(pam_level(-d, a.qam_half, a.qam_a), a.qam_half, a.qam_a);
-                                bl = arrives ? bd : bl;
-                                d = arrives ? d + bd : d;
-                            }
-                        }
-                        // window J_n = samples [n - W + 1, n] = lanes [s + WP - W, s + WP - 1]
-                        const bool inw = (unsigned)(lw - s) < (unsigned)W;
-                        float nsc;
-                        if constexpr (kViol) {  // mu q with q = 1/|V_n| on the violated slabs
-                            const bool viol = inw && lv && fabsf(d) > a.eps;
-                            const float muq = s_muqv[__popc(__ballot_sync(0xffffffffu, viol))];  // (every lane)
-                            nsc = inw ? -muq * rkl : 0.f;
-                        } else if (kChecked && n + sb < W - 1) {  // mu q with q = 1/|J_n|
-                            nsc = inw ? -s_muq[n + sb] * rkl : 0.f;
-                        } else {
-                            nsc = inw ? nsc_full : 0.f;
-                        }
-                        const float nm = (fmaxf(d, a.eps) + fminf(d, -a.eps)) * nsc;  // -mu q beta_j
-                        float *ring = s_w + (s & 1) * 32;
-                        ring[lane] = nm;
-                        gn += nm;
-                        if (kChecked && log_cases && inw && lv)
-                            a.case_log[((size_t)(n - n_first) * W + (ms - n + W - 1)) * K + k] =
-                                (int8_t)(d > a.eps ? -1 : (d < -a.eps ? 1 : 0));
-                        __syncwarp();
-                        // lanes outside the window hold 0 in the ring: whole pairs around it
-                        uint64_t acc[4];
-                        acc[0] = pack2(d, 0.f);
-                        constexpr int kMaxPairs = WP / 2 + 1;
-                        uint64_t rv[kMaxPairs + 2];
-                        const int p0 = (s >> 1) & ~1, np = ((s + WP + 1) >> 1) - (s >> 1), off = (s >> 1) - p0;
-#pragma unroll
-                        for (int q = 0; q < kMaxPairs + 1; q += 2) {
-                            if (q < np + off) {
-                                const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(ring + 2 * (p0 + q));
-                                rv[q] = v.x;
-                                rv[q + 1] = v.y;
-                            }
-                        }
-#pragma unroll
-                        for (int q = 0; q < kPairsPerStep; ++q) {  // the next block's kernel values
-                            const int i = s * kPairsPerStep + q;
-                            if (i < NP) kn[i] = pack2(krow[2 * i * RS], krow[(2 * i + 1) * RS]);
-                        }
-#pragma unroll
-                        for (int q = 0; q < kMaxPairs; ++q) {
-                            if (q < np) {
-                                const uint64_t kv = kc[(s >> 1) + q];
-                                if (q == 0 || q >= 4) acc[q & 3] = ffma2(rv[off + q], kv, acc[q & 3]);
-                                else acc[q] = fmul2(rv[off + q], kv);
-                            }
-                        }
-                        if (np > 1) acc[0] = fadd2(acc[0], acc[1]);
-                        if (np > 3) acc[2] = fadd2(acc[2], acc[3]);
-                        if (np > 2) acc[0] = fadd2(acc[0], acc[2]);
-                        d = sum2(acc[0]);
-                    }
-                };
-                using T_ = std::true_type;
-                using F_ = std::false_type;
-                const bool checked = n0 + B > s1 || n0 + sb < W - 1 || log_cases;
-                if (kExt && a.qviol) {
-                    if constexpr (kExt) {
-                        if (evict) steps(T_{}, T_{}, T_{});
-                        else steps(T_{}, F_{}, T_{});
-                    }
-                } else if (evict) {
-                    if (checked) steps(T_{}, T_{}, F_{});
-                    else steps(F_{}, T_{}, F_{});
-                } else {
-                    if (checked) steps(T_{}, F_{}, F_{});
-                    else steps(F_{}, F_{}, F_{});
-                }
-                float *agg = s_agg + (blk & 1) * 32;
-                agg[lane] = lv ? -gn : 0.f;
+        if (valid) {
+            s_p[u] = p;
+            s_g[u] = gam;
+            s_b[u] = b;
+            s_rk[u] = rk;
+        }
+        __syncthreads();
+        {
+            if (u < 32) {
+                // ================= window warp =================
+                constexpr int NP = 32 + B;                     // rows a lane loads for its next sample
+                constexpr int kRowsPerStep = (NP + B - 1) / B;
+                const int lane = u;
+                const int lw = lane - (WP - W);
+                const int m0 = s0 - WP + 1 + lane;
+                bool lv = lane < NL && m0 >= l0 && m0 < s1;
+                int col = lv ? m0 - l0 : 0;
+                float pl = 0.f, bl = 0.f, rkl = 0.f;
                 if (lv) {
-                    s_d[col] = d;
-                    s_g[col] -= gn;
-                    if (kExt) s_b[col] = bl;
-                    if (kExt && a.soft_out && lane >= WP - 1)
-                        a.soft_out[((size_t)((ms - n_first) >> 1) * K + k) * 2 + (ms & 1)] = b_before - darr;
+                    pl = s_p[col];
+                    bl = s_b[col];
+                    rkl = s_rk[col];
                 }
-                if (has_next) {  // the block's move of this lane's next sample, if it is a new one
-                    __syncwarp();
-                    uint64_t acc[4];
+                float c1 = lv ? bl - a.eps : 0.f, c2 = lv ? bl + a.eps : 0.f;  // the hyperslab [b - eps, b + eps]
+                // kernel values against rows [wl0, wl0 + 32) (row 31 meets a zero change only; rows
+                // outside the live range are zero rows)
+                float kc[32], kn[NP];
 #pragma unroll
-                    for (int i = 0; i < 16; i += 2) {
-                        const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(agg + 2 * i);
-                        if (i < 4) {
-                            acc[i] = fmul2(v.x, kn[i]);
-                            acc[i + 1] = fmul2(v.y, kn[i + 1]);
-                        } else {
-                            acc[i & 3] = ffma2(v.x, kn[i], acc[i & 3]);
-                            acc[(i + 1) & 3] = ffma2(v.y, kn[i + 1], acc[(i + 1) & 3]);
+                for (int i = 0; i < 32; ++i) kc[i] = s_kmat[(s0 - WP + 1 - l0 + i) * RS + col];
+#pragma unroll 1
+                for (int n0 = s0; n0 < s1; n0 += B, ++blk) {
+                    const int wl0 = n0 - WP + 1, ms = wl0 + lane;  // sample of lane 0, of this lane
+                    const bool has_next = n0 + B < s1;
+                    const bool lvn = has_next && lane < NL && ms + B >= l0 && ms + B < s1;
+                    const int coln = lvn ? ms + B - l0 : 0;      // the sample this lane holds in the next block
+                    const float *krow = s_kmat + (has_next ? (wl0 - l0) * RS + coln : 0);
+                    const float sc_full = muq_full * rkl;        // mu q / kappa_jj (0 in a lane without a sample)
+                    float agg = 0.f, evn = 0.f, parr = 0.f;      // summed change; evictions at coln; output at arrival
+                    // kChecked: a partial last block, the filling window (n < W - 1) or case logging;
+                    // kViol: weights on the violated slabs
+                    auto steps = [&](auto checked_c, auto evict_c, auto viol_c) {
+                        constexpr bool kChecked = decltype(checked_c)::value, kEvict = decltype(evict_c)::value;
+                        constexpr bool kViol = decltype(viol_c)::value;
+#pragma unroll
+                        for (int s = 0; s < B; ++s) {
+                            const int n = n0 + s;
+                            if (kChecked && n >= s1) break;  // (only in the last block, which loads nothing ahead)
+                            if (kEvict && !(n & 1) && (n >> 1) + tb >= D) {
+                                const int e = (n >> 1) - t0;
+                                const float e0 = s_egam[2 * e], e1 = s_egam[2 * e + 1];
+                                const float *ge = s_gev + e * 2 * RS;
+                                pl -= a.wG * fmaf(e0, ge[col], e1 * ge[RS + col]);
+                                evn -= a.wG * fmaf(e0, ge[coln], e1 * ge[RS + coln]);
+                            }
+                            if constexpr (kExt) {  // sample n arrives: pl = f_n(x_n)
+                                const bool arrives = lane == s + WP - 1;
+                                parr = arrives ? pl : parr;
+                                if (a.decide) {  // its target: the decision on the filter's own output
+                                    const float bd = a.qam_half == 1
+                                                         ? (pl >= 0.f ? a.qam_a : -a.qam_a)
+                                                         : pam_value(pam_level(pl, a.qam_half, a.qam_a), a.qam_half, a.qam_a);
+                                    bl = arrives ? bd : bl;
+                                    c1 = arrives ? bd - a.eps : c1;
+                                    c2 = arrives ? bd + a.eps : c2;
+                                }
+                            }
+                            // window J_n = samples [n - W + 1, n] = lanes [s + WP - W, s + WP - 1]
+                            const bool inw = (unsigned)(lw - s) < (unsigned)W;
+                            float sc;
+                            if constexpr (kViol) {  // mu q with q = 1/|V_n| on the violated slabs
+                                const bool viol = inw && lv && (pl < c1 || pl > c2);
+                                const float muq = s_muqv[__popc(__ballot_sync(0xffffffffu, viol))];  // (every lane)
+                                sc = inw ? muq * rkl : 0.f;
+                            } else if (kChecked && n + sb < W - 1) {  // mu q with q = 1/|J_n|
+                                sc = inw ? s_muq[n + sb] * rkl : 0.f;
+                            } else {
+                                sc = inw ? sc_full : 0.f;
+                            }
+                            const float mb = (fminf(fmaxf(pl, c1), c2) - pl) * sc;  // mu q beta_j
+                            float *ring = s_w + (s & 1) * 32;
+                            ring[lane] = mb;
+                            agg += mb;
+                            if (kChecked && log_cases && inw && lv)
+                                a.case_log[((size_t)(n - n_first) * W + (ms - n + W - 1)) * K + k] =
+                                    (int8_t)(pl < c1 ? -1 : (pl > c2 ? 1 : 0));
+                            __syncwarp();
+                            // the window's sum in four chains, chain (j - s) mod 4, as packed pairs
+                            // of chains (a ring slot past the window holds 0)
+                            float rv[WP + 4];
+                            const int b4 = s & ~3;
+#pragma unroll
+                            for (int q4 = 0; q4 < WP + 4; q4 += 4)
+                                if (b4 + q4 <= s + WP - 1 + (s & 1))
+                                    *reinterpret_cast<float4 *>(rv + q4) = *reinterpret_cast<const float4 *>(ring + b4 + q4);
+#pragma unroll
+                            for (int q = 0; q < kRowsPerStep; ++q) {  // the next block's kernel values
+                                const int i = s * kRowsPerStep + q;
+                                if (i < NP) kn[i] = krow[i * RS];
+                            }
+                            auto rp = [&](int j) { return pack2(rv[j - b4], rv[j - b4 + 1]); };
+                            auto kp = [&](int j) { return pack2(kc[j], kc[j + 1]); };
+                            if (s & 1) {  // pairs (j, j + 1), j even: chains (1, 2) and (3, 0)
+                                uint64_t x = 0, y = pack2(0.f, fmaf(rv[s - b4], kc[s], pl));
+#pragma unroll
+                                for (int j = s + 1; j < s + WP; j += 4) {
+                                    x = ffma2(rp(j), kp(j), x);
+                                    y = ffma2(rp(j + 2), kp(j + 2), y);  // (the last pair's second ring value is 0)
+                                }
+                                float x0, x1, y0, y1;
+                                unpack2(x, x0, x1);
+                                unpack2(y, y0, y1);
+                                pl = (y1 + x0) + (x1 + y0);
+                            } else {      // chains (0, 1) and (2, 3)
+                                uint64_t x = pack2(pl, 0.f), y = 0;
+#pragma unroll
+                                for (int j = s; j < s + WP; j += 4) {
+                                    x = ffma2(rp(j), kp(j), x);
+                                    y = ffma2(rp(j + 2), kp(j + 2), y);
+                                }
+                                pl = sum2(x) + sum2(y);
+                            }
                         }
+                    };
+                    using T_ = std::true_type;
+                    using F_ = std::false_type;
+                    const bool checked = n0 + B > s1 || n0 + sb < W - 1 || log_cases;
+                    if (kExt && a.qviol) {
+                        if constexpr (kExt) {
+                            if (evict) steps(T_{}, T_{}, T_{});
+                            else steps(T_{}, F_{}, T_{});
+                        }
+                    } else if (evict) {
+                        if (checked) steps(T_{}, T_{}, F_{});
+                        else steps(F_{}, T_{}, F_{});
+                    } else {
+                        if (checked) steps(T_{}, F_{}, F_{});
+                        else steps(F_{}, F_{}, F_{});
                     }
-                    const float move = sum2(fadd2(fadd2(acc[0], acc[1]), fadd2(acc[2], acc[3])));
+                    float *s_ag = s_agg + (blk & 1) * 32;
+                    s_ag[lane] = lv ? agg : 0.f;
+                    if (lv) {
+                        s_p[col] = pl;
+                        s_g[col] += agg;
+                        if (kExt) s_b[col] = bl;
+                        if (kExt && a.soft_out && lane >= WP - 1)
+                            a.soft_out[((size_t)((ms - n_first) >> 1) * K + k) * 2 + (ms & 1)] = parr;
+                    }
                     block_barrier();  // the blocks before this one have reached the next block's samples
-                    const float d_old = __shfl_down_sync(0xffffffffu, d, B);
-                    d = lane < WP - 1 ? d_old : s_d[coln] + (evn - move);
-                    lv = lvn;
-                    col = coln;
-                    bl = lv ? s_b[col] : 0.f;
-                    rkl = lv ? s_rk[col] : 0.f;
-                    d = lv ? d : 0.f;
+                    if (has_next) {   // the block's move of this lane's next sample, if it is a new one
+                        const float pn = s_p[coln], bn = s_b[coln], rkn = s_rk[coln];
+                        uint64_t acc[2] = {0, 0};
 #pragma unroll
-                    for (int i = 0; i < 16; ++i) kc[i] = kn[i + B / 2];
-                } else {
-                    block_barrier();
+                        for (int i = 0; i < 32; i += 4) {
+                            const float4 v = *reinterpret_cast<const float4 *>(s_ag + i);
+                            acc[0] = ffma2(pack2(v.x, v.y), pack2(kn[i], kn[i + 1]), acc[0]);
+                            acc[1] = ffma2(pack2(v.z, v.w), pack2(kn[i + 2], kn[i + 3]), acc[1]);
+                        }
+                        const float p_old = __shfl_down_sync(0xffffffffu, pl, B);
+                        const float moved = (pn + (sum2(acc[0]) + sum2(acc[1]))) + evn;
+                        lv = lvn;
+                        col = coln;
+                        pl = lv ? (lane < WP - 1 ? p_old : moved) : 0.f;
+                        bl = lv ? bn : 0.f;
+                        rkl = lv ? rkn : 0.f;
+                        c1 = lv ? bl - a.eps : 0.f;
+                        c2 = lv ? bl + a.eps : 0.f;
+#pragma unroll
+                        for (int i = 0; i < 32; ++i) kc[i] = kn[i + B];
+                    }
                 }
-            }
-        } else {
-            // ================= the other warps =================
-            float tp[2] = {0.f, 0.f};  // tracked part of f at this thread's next-chunk samples
-            // filter change of one block: x~ = r(t) for r1(t) and -i r(t) for r2(t); lanes outside L
-            // carry a zero change
-            auto dc_apply = [&](const float *agg, int wl0b) {
+            } else {
+                // ================= the other warps =================
+                float tp[2] = {0.f, 0.f};  // tracked part of f at this thread's next-chunk samples
+                // filter change of one block: x~ = r(t) for r1(t) and -i r(t) for r2(t); lanes outside L
+                // carry a zero change
+                int dj0[2], dj1[2], dmm[2];  // this thread's parts of the sum: lanes [dj0, dj1), antenna
 #pragma unroll
                 for (int it = 0; it < 2; ++it) {
-                    const int idx = tu + it * ntr;
-                    if (idx >= dc_parts * M) continue;
-                    const int mm = idx % M, part = idx / M;
-                    const int j0 = part * NL / dc_parts, j1 = (part + 1) * NL / dc_parts;
-                    for (int j = j0; j < j1; ++j) {
-                        const float dg = agg[j];
-                        const int ms = wl0b + j;
-                        const int pi = min(max((ms >> 1) - pa0, 0), npil - 1);
-                        const float2 x = s_pil[pi * M + mm];
-                        if (ms & 1) { dcx[it] = fmaf(dg, x.y, dcx[it]); dcy[it] = fmaf(-dg, x.x, dcy[it]); }
-                        else        { dcx[it] = fmaf(dg, x.x, dcx[it]); dcy[it] = fmaf(dg, x.y, dcy[it]); }
-                    }
+                    const int idx = tu + it * ntr, part = idx / M;
+                    dmm[it] = idx % M;
+                    dj0[it] = part * NL / dc_parts;
+                    dj1[it] = idx < dc_parts * M ? (part + 1) * NL / dc_parts : dj0[it];
                 }
-            };
-            // At this chunk's start the entries of L hold gamma only at the carried samples (the new
-            // ones start at 0), so the tracked part of f_{s0} at a next-chunk sample x is
-            //   w_L <w, x> + w_G sum_{carried j} gamma_j kappa_G(x_j, x)
-            //     = w_L <w - sum_{carried j} gamma_j x_j, x> + sum_{carried j} gamma_j kappa(x_j, x),
-            // the second form using the tabulated sum kernel; the tracking threads form the reduced
-            // filter, meet at a named barrier of their own, then evaluate their samples.
-            auto track_init = [&]() {
-                for (int mm = tu; mm < M; mm += ntr) {
-                    float2 c = s_clin[mm];
-                    for (int j = 0; j < nc; ++j) {
-                        const float dg = -s_gcar[j];
-                        const float2 x = s_pil[(((l0 + j) >> 1) - pa0) * M + mm];
-                        if ((l0 + j) & 1) { c.x = fmaf(dg, x.y, c.x); c.y = fmaf(-dg, x.x, c.y); }
-                        else              { c.x = fmaf(dg, x.x, c.x); c.y = fmaf(dg, x.y, c.y); }
-                    }
-                    s_clinw[mm] = c;
-                }
-                asm volatile("bar.sync 1, %0;" ::"r"(ntr) : "memory");
+                auto dc_apply = [&](const float *agg, int wl0b) {
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    const int v = tu + i * ntr;
-                    if (v >= n_next) continue;
-                    const int tv = t0 + Tc + (v >> 1), lvv = v & 1;
-                    const float2 *rv = a.rx + (size_t)tv * M;
-                    float l0s = 0.f, l1s = 0.f;
-                    for (int mm = 0; mm < M; mm += 2) {
-                        const float4 x = __ldcg(reinterpret_cast<const float4 *>(rv + mm));
-                        const float2 c = s_clinw[mm], cb = s_clinw[mm + 1];
-                        l0s = lvv ? fmaf(c.x, x.y, fmaf(-c.y, x.x, l0s)) : fmaf(c.x, x.x, fmaf(c.y, x.y, l0s));
-                        l1s = lvv ? fmaf(cb.x, x.w, fmaf(-cb.y, x.z, l1s)) : fmaf(cb.x, x.z, fmaf(cb.y, x.w, l1s));
-                    }
-                    // s_gcar is zero past the carried samples; rows clamped into the table
-                    float acc4[4] = {a.wL * (l0s + l1s), 0.f, 0.f, 0.f};
-#pragma unroll
-                    for (int j = 0; j < 32; ++j)
-                        acc4[j & 3] = fmaf(s_gcar[j], __ldcg(a.kx + (size_t)min(j, R - 1) * g.KXS + v), acc4[j & 3]);
-                    tp[i] = (acc4[0] + acc4[1]) + (acc4[2] + acc4[3]);
-                }
-            };
-            auto track_apply = [&](const float *agg, int r0) {
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    const int v = tu + i * ntr;
-                    if (v >= n_next) continue;
-                    // rows outside [0, R) belong to lanes whose summed change is zero: clamp, no branch,
-                    // so that all NL loads are in flight together
-                    float kv[NL];
-#pragma unroll
-                    for (int j = 0; j < NL; ++j) kv[j] = __ldcg(a.kx + (size_t)min(max(r0 + j, 0), R - 1) * g.KXS + v);
-                    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                    for (int j = 0; j < NL; ++j) acc[j & 3] = fmaf(agg[j], kv[j], acc[j & 3]);
-                    tp[i] += (acc[0] + acc[1]) + (acc[2] + acc[3]);
-                }
-            };
-            // block bb (steps from nb): its moves of the samples from nb + 2 B on, and its dropped entries
-            auto near_apply = [&](const float *agg, int nb) {
-                const int r0 = nb - WP + 1 - l0;
-                for (int i = kLater + tu; i < R; i += ntr) {
-                    if (l0 + i < nb + 2 * B) continue;
-                    const float *kr = s_kmat + r0 * RS + i;
-                    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                    for (int j = 0; j < NL; ++j) acc[j & 3] = fmaf(agg[j], kr[j * RS], acc[j & 3]);
-                    float dv = s_d[i] - ((acc[0] + acc[1]) + (acc[2] + acc[3]));
-                    if (evict) {
-                        for (int n = nb + (nb & 1); n < nb + B; n += 2) {
-                            if ((n >> 1) + tb < D) continue;
-                            const int e = (n >> 1) - t0;
-                            dv = fmaf(a.wG, fmaf(s_egam[2 * e], s_gev[e * 2 * RS + i],
-                                                 s_egam[2 * e + 1] * s_gev[(e * 2 + 1) * RS + i]), dv);
+                    for (int it = 0; it < 2; ++it) {
+                        for (int j = dj0[it]; j < dj1[it]; ++j) {
+                            const float dg = agg[j];
+                            const int ms = wl0b + j;
+                            const int pi = min(max((ms >> 1) - pa0, 0), npil - 1);
+                            const float2 x = s_pil[pi * M + dmm[it]];
+                            const float xa = (ms & 1) ? x.y : x.x, xb = (ms & 1) ? -x.x : x.y;
+                            dcx[it] = fmaf(dg, xa, dcx[it]);
+                            dcy[it] = fmaf(dg, xb, dcy[it]);
                         }
                     }
-                    s_d[i] = dv;
-                }
-            };
-            for (int n0 = s0; n0 < s1; n0 += B, ++blk) {
-                if (blk == 0) {
-                    if (track) track_init();
-                } else {
-                    const float *agg = s_agg + ((blk - 1) & 1) * 32;
-                    near_apply(agg, n0 - B);
-                    dc_apply(agg, n0 - B - WP + 1);
-                    if (track) track_apply(agg, n0 - B - WP + 1 - l0);
-                }
-                if (n0 + B >= s1) {
-                    // beside the last block: the chunk's new dictionary entries (slot (tb + t) % D) and
-                    // their norms, spread over the K user CTAs, which all hold the chunk's pilots
-                    for (int i = k * ntr + tu; i < Tc * M; i += K * ntr) {
-                        const int t = t0 + i / M, mm = i % M;
-                        a.dict[(size_t)((tb + t) % D) * M + mm] = s_pil[(t - pa0) * M + mm];
+                };
+                // At this chunk's start the entries of L hold gamma only at the carried samples (the new
+                // ones start at 0), so the tracked part of f_{s0} at a next-chunk sample x is
+                //   w_L <w, x> + w_G sum_{carried j} gamma_j kappa_G(x_j, x)
+                //     = w_L <w - sum_{carried j} gamma_j x_j, x> + sum_{carried j} gamma_j kappa(x_j, x),
+                // the second form using the tabulated sum kernel; these warps form the reduced filter,
+                // meet at a named barrier of their own, then evaluate their samples.
+                auto track_init = [&]() {
+                    for (int mm = tu; mm < M; mm += ntr) {
+                        float2 c = s_clin[mm];
+                        for (int j = 0; j < nc; ++j) {
+                            const float dg = -s_gcar[j];
+                            const float2 x = s_pil[(((l0 + j) >> 1) - pa0) * M + mm];
+                            if ((l0 + j) & 1) { c.x = fmaf(dg, x.y, c.x); c.y = fmaf(-dg, x.x, c.y); }
+                            else              { c.x = fmaf(dg, x.x, c.x); c.y = fmaf(dg, x.y, c.y); }
+                        }
+                        s_clinw[mm] = c;
                     }
-                    for (int i = k * ntr + tu; i < Tc; i += K * ntr) {
-                        const float2 *rv = s_pil + (t0 + i - pa0) * M;
-                        float nrm = 0.f;
-                        for (int mm = 0; mm < M; ++mm) nrm = fmaf(rv[mm].x, rv[mm].x, fmaf(rv[mm].y, rv[mm].y, nrm));
-                        a.dict_norm[(tb + t0 + i) % D] = nrm;
-                    }
-                }
-                block_barrier();
-            }
-            if (blk > 0) {  // the last block's changes, then hand over
-                const float *agg = s_agg + ((blk - 1) & 1) * 32;
-                const int wl0 = s0 + (blk - 1) * B - WP + 1;
-                dc_apply(agg, wl0);
-                if (track) {
-                    track_apply(agg, wl0 - l0);
+                    asm volatile("bar.sync 1, %0;" ::"r"(ntr) : "memory");
 #pragma unroll
                     for (int i = 0; i < 2; ++i) {
                         const int v = tu + i * ntr;
-                        if (v < n_next) a.track_out[v * K + k] = tp[i];
+                        if (v >= n_next) continue;
+                        const int tv = t0 + Tc + (v >> 1), lvv = v & 1;
+                        const float2 *rv = a.rx + (size_t)tv * M;
+                        float kv[32];
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) kv[j] = __ldcg(a.kx + (size_t)min(j, R - 1) * g.KXS + v);
+                        float l0s = 0.f, l1s = 0.f;
+                        for (int m0 = 0; m0 < M; m0 += 16) {  // eight loads in flight
+                            float4 x[8];
+#pragma unroll
+                            for (int q = 0; q < 8; ++q)
+                                x[q] = m0 + 2 * q < M ? __ldcg(reinterpret_cast<const float4 *>(rv + m0 + 2 * q))
+                                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                            for (int q = 0; q < 8; ++q) {
+                                if (m0 + 2 * q < M) {
+                                    const float2 c = s_clinw[m0 + 2 * q], cb = s_clinw[m0 + 2 * q + 1];
+                                    l0s = lvv ? fmaf(c.x, x[q].y, fmaf(-c.y, x[q].x, l0s))
+                                              : fmaf(c.x, x[q].x, fmaf(c.y, x[q].y, l0s));
+                                    l1s = lvv ? fmaf(cb.x, x[q].w, fmaf(-cb.y, x[q].z, l1s))
+                                              : fmaf(cb.x, x[q].z, fmaf(cb.y, x[q].w, l1s));
+                                }
+                            }
+                        }
+                        // s_gcar is zero past the carried samples; rows clamped into the table
+                        float acc4[4] = {a.wL * (l0s + l1s), 0.f, 0.f, 0.f};
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) acc4[j & 3] = fmaf(s_gcar[j], kv[j], acc4[j & 3]);
+                        tp[i] = (acc4[0] + acc4[1]) + (acc4[2] + acc4[3]);
                     }
+                };
+                // 31-term sum of a block's changes against one column of a table whose rows are `stride`
+                // apart: sum j mod 4, as eight rows at a time
+                auto col_dot = [&](const float *agg, const float *colp, int stride) {
+                    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+                    for (int j = 0; j < 32; j += 8) {  // (row 31 meets a zero change; it is inside the table)
+                        const float4 v0 = *reinterpret_cast<const float4 *>(agg + j),
+                                     v1 = *reinterpret_cast<const float4 *>(agg + j + 4);
+                        const float av[8] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) acc[q & 3] = fmaf(av[q], colp[(j + q) * stride], acc[q & 3]);
+                    }
+                    return (acc[0] + acc[1]) + (acc[2] + acc[3]);
+                };
+                // block from step nb: its moves of the samples from nb + 2 B on, and its dropped entries
+                auto near_apply = [&](const float *agg, int nb) {
+                    for (int i = kLater + tu; i < R; i += ntr) {
+                        if (l0 + i < nb + 2 * B) continue;
+                        float v = s_p[i] + col_dot(agg, s_kmat + (nb - WP + 1 - l0) * RS + i, RS);
+                        if (evict) {
+                            for (int n = nb + (nb & 1); n < nb + B; n += 2) {
+                                if ((n >> 1) + tb < D) continue;
+                                const int e = (n >> 1) - t0;
+                                v -= a.wG * fmaf(s_egam[2 * e], s_gev[e * 2 * RS + i],
+                                                 s_egam[2 * e + 1] * s_gev[(e * 2 + 1) * RS + i]);
+                            }
+                        }
+                        s_p[i] = v;
+                    }
+                };
+                // The next chunk's samples: the first one's column is loaded from L2 before the barrier
+                // that publishes the block's changes.  Rows outside [0, R) belong to lanes whose summed
+                // change is zero: the first block of a call and the last of a chunk clamp them.
+                float kt[NL];
+                auto track_fetch = [&](int r0, int v) {
+                    const float *src = a.kx + v;
+                    if (r0 >= 0 && r0 + NL <= R && g.KXS == 128) {  // whole-length chunks: a constant stride
+#pragma unroll
+                        for (int j = 0; j < NL; ++j) kt[j] = __ldcg(src + (size_t)r0 * 128 + j * 128);
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < NL; ++j) kt[j] = __ldcg(src + (size_t)min(max(r0 + j, 0), R - 1) * g.KXS);
+                    }
+                };
+                int track_r0 = 0;
+                auto track_apply = [&](const float *agg) {
+#pragma unroll 1
+                    for (int i = 0; i < 2 && tu + i * ntr < n_next; ++i) {
+                        if (i > 0) track_fetch(track_r0, tu + i * ntr);
+                        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                        for (int j = 0; j < 32; j += 4) {
+                            const float4 v = *reinterpret_cast<const float4 *>(agg + j);
+                            acc[0] = fmaf(v.x, kt[j], acc[0]);
+                            acc[1] = fmaf(v.y, kt[j + 1], acc[1]);
+                            acc[2] = fmaf(v.z, kt[j + 2], acc[2]);
+                            if (j + 3 < NL) acc[3] = fmaf(v.w, kt[j + 3], acc[3]);
+                        }
+                        const float t = (acc[0] + acc[1]) + (acc[2] + acc[3]);
+                        if (i == 0) tp[0] += t;
+                        else tp[1] += t;
+                    }
+                };
+#pragma unroll 1
+                for (int n0 = s0; n0 < s1; n0 += B, ++blk) {
+                    if (blk == 0) {
+                        if (track) track_init();
+                    } else {
+                        const float *agg = s_agg + ((blk - 1) & 1) * 32;
+                        near_apply(agg, n0 - B);
+                        if (track) track_apply(agg);
+                    }
+                    track_r0 = n0 - WP + 1 - l0;
+                    if (tu < n_next) track_fetch(track_r0, tu);
+                    if (blk > 0) dc_apply(s_agg + ((blk - 1) & 1) * 32, n0 - B - WP + 1);
+                    if (n0 + B >= s1) {
+                        // beside the last block: the chunk's new dictionary entries (slot (tb + t) % D) and
+                        // their norms, spread over the K user CTAs, which all hold the chunk's pilots
+                        for (int i = k * ntr + tu; i < Tc * M; i += K * ntr) {
+                            const int t = t0 + i / M, mm = i % M;
+                            a.dict[(size_t)((tb + t) % D) * M + mm] = s_pil[(t - pa0) * M + mm];
+                        }
+                        for (int i = k * ntr + tu; i < Tc; i += K * ntr) {
+                            const float2 *rv = s_pil + (t0 + i - pa0) * M;
+                            float nrm = 0.f;
+                            for (int mm = 0; mm < M; ++mm) nrm = fmaf(rv[mm].x, rv[mm].x, fmaf(rv[mm].y, rv[mm].y, nrm));
+                            a.dict_norm[(tb + t0 + i) % D] = nrm;
+                        }
+                    }
+                    block_barrier();
                 }
+                // the last block's changes, then hand over
+                const float *agg = s_agg + ((blk - 1) & 1) * 32;
+                if (track) {
+                    if (tu < n_next) {
+                        track_apply(agg);
+                        a.track_out[tu * K + k] = tp[0];
+                    }
+                    if (tu + ntr < n_next) a.track_out[(tu + ntr) * K + k] = tp[1];
+                }
+                dc_apply(agg, s0 + (blk - 1) * B - WP + 1);
             }
         }
         if (valid) {
-            p = s_b[u] - s_d[u];
+            p = s_p[u];
             gam = s_g[u];
             b = s_b[u];
         }
