@@ -60,8 +60,8 @@ def measured_peaks():
 
 def detect_roofline(w, n_entries, seconds, engine="tf32x3"):
     """Roofline of one detection launch.  Algorithmic work per (query, entry) pair: the complex
-    Gram (2M x 2 MACs) -- on the tensor pipe as three TF32 products for FP32 accuracy
-    (engine "tf32x3") or one BF16/FP16 product ("half"), or on the FP32 pipe as 4M FMA ("ffma");
+    Gram (2M x 2 MACs) -- on the tensor pipe as three TF32 or FP16 products for FP32 accuracy
+    (engines "tf32x3", "f16x3") or one BF16/FP16 product ("half"), or on the FP32 pipe as 4M FMA ("ffma");
     the three exponentials on MUFU; the exponent arguments and the coefficient accumulation
     (4K + 3 FMA) on the FP32 pipe.  The bound is the resource with the largest minimum time; `frac` = that minimum time /
     measured time."""
@@ -79,7 +79,7 @@ def detect_roofline(w, n_entries, seconds, engine="tf32x3"):
                "alu": (2 * 3 * pairs, FP32_PEAK_TFLOPS * 1e12, "TFLOP/s")}
     else:
         tensor = ((3 * gram, bf16 * (1.1 / 2.25) * 1e12, "TFLOP/s") if engine == "tf32x3" else
-                  (gram, bf16 * 1e12, "TFLOP/s"))
+                  (3 * gram, bf16 * 1e12, "TFLOP/s") if engine == "f16x3" else (gram, bf16 * 1e12, "TFLOP/s"))
         res = {"tensor": tensor,
                "alu": (2 * (4 * w["K"] + 3) * pairs, FP32_PEAK_TFLOPS * 1e12, "TFLOP/s")}
     res["mufu"] = (3 * pairs, MUFU_PEAK_PER_S, "Gex2/s")
@@ -435,7 +435,7 @@ def run_precision(args):
         # FP32 has no tensor-core kernel above 32 antennas (its TF32 hi/lo operands would not fit
         # shared memory), so it runs on the FMA engine here; BF16/FP16 form the Gram and the
         # coefficient sums on the tensor cores.
-        engine = "half-tc" if dt != "fp32" else ("ffma" if M > 32 else "tf32x3")
+        engine = "half-tc" if dt != "fp32" else "f16x3"
         out[dt] = {"value": N / (ms / 1e3), "ms": ms, "pairs_per_s": pairs / (ms / 1e3), "engine": engine,
                    "roofline": detect_roofline(dict(M=M, K=K, N=N), D, ms / 1e3, engine),
                    "ser": float((h_.cpu().numpy() != x.idx_data).mean())}

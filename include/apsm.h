@@ -419,7 +419,8 @@ apsm_status apsm_batch_workspace_bytes(const apsm_instance *inst, int32_t n, siz
  *                 decisions (or no hard output) in classes the launch-choice table does not give
  *                 to the FMA engine; any other instance is detected by apsm_detect on its
  *                 branch after its training.  Per instance the outputs equal apsm_train followed
- *                 by apsm_detect bit for bit.
+ *                 by apsm_detect, bit for bit where both form the Gram in the same way (always with
+ *                 APSM_OPT_DETECT_TMA = 0), else up to FP32 rounding.
  * The descriptors (and the buffers they point to) are bound at creation: apsm_batch_launch replays
  * the same work on new data in the same buffers.  Every instance is validated before anything is
  * recorded.  workspace: apsm_batch_workspace_bytes bytes, 256-byte aligned, caller-owned, kept
@@ -458,8 +459,10 @@ apsm_status apsm_check_wait_timeout(const apsm_state *st, void *stream);
  *                         the current chunk; 0: they are evaluated between chunks (sequential)
  *   APSM_OPT_DETECT_TMA   1 (default): FP32 detection with 4, 8 or 16 antennas and an even user
  *                         count in {2, 4, 6, 8, 12, 16} stages every operand by TMA (entry rows
- *                         as stored, the real split's rotation on the query side); 0: the
- *                         tensor-core form that converts entry rows in shared memory
+ *                         as stored, the real split's rotation on the query side), and with 32
+ *                         or 64 antennas forms the Gram from three FP16 products of scaled hi and
+ *                         lo copies; 0: the tensor-core form that converts entry rows to TF32 in
+ *                         shared memory (64 antennas: the FP32 FMA engine)
  *   APSM_OPT_HALF_TC_COEF 1 (default): BF16/FP16 detection with 16, 32 or 64 antennas forms the
  *                         coefficient sums on the tensor cores too (the exponentials rounded to
  *                         BF16, the coefficients as a BF16 hi + lo pair, FP32 accumulation);

@@ -12,6 +12,7 @@
 #include "apsm_common.cuh"
 #include "detect_bwd.cuh"
 #include "detect_f32.cuh"
+#include "detect_h3.cuh"
 #include "detect_tc.cuh"
 #include "detect_tcc.cuh"
 #include "detect_tma.cuh"
@@ -27,6 +28,7 @@ TcLauncher detect_tc_launcher(int M, int K, int prec);  // detect_tc_m*.cu
 TmaLauncher detect_tma_launcher(int M, int K);         // detect_tma_m*.cu
 TccLauncher detect_tcc_launcher(int M, int K);         // detect_tc_m*.cu (BF16/FP16, coefficient sums on tcgen05)
 size_t detect_tcc_workspace(int M, int K, int D);
+H3Launcher detect_h3_launcher(int M, int K);           // detect_h3_m*.cu (FP32, 32 and 64 antennas)
 using ChunkLauncher = cudaError_t (*)(const ChunkArgs &, int, cudaStream_t);
 ChunkLauncher chunk_launcher(int S, int WP, bool ext);  // train_chunk.cu
 int padded_window(int W);                           // train_chunk.cu
@@ -648,8 +650,9 @@ apsm_status apsm_detect_ws(const apsm_params *p, const apsm_state *st, const flo
         // BF16/FP16 with a workspace: the coefficient sums on the tensor cores too
         TccLauncher tcc = (prec == kHalf && workspace && g_opt_half_tc_coef.load()) ? detect_tcc_launcher(p->M, p->K)
                                                                                      : nullptr;
+        H3Launcher h3 = (p->dtype == APSM_FP32 && g_opt_detect_tma.load()) ? detect_h3_launcher(p->M, p->K) : nullptr;
         TmaLauncher tma = (p->dtype == APSM_FP32 && g_opt_detect_tma.load()) ? detect_tma_launcher(p->M, p->K) : nullptr;
-        if (tc || tma) {
+        if (tc || tma || h3) {
             TcArgs ta{};
             ta.rx = reinterpret_cast<const float2 *>(rx);
             ta.N = N;
@@ -668,6 +671,12 @@ apsm_status apsm_detect_ws(const apsm_params *p, const apsm_state *st, const flo
             ta.hard = hard;
             ta.status = st->meta + 3;
             if (qam_pass) ta.hard = nullptr;
+            if (h3) {
+                int launches = 0;
+                if (h3(ta, &launches, strm) != cudaSuccess) return APSM_ERR_CUDA;
+                g_launches += launches;
+                return qam_pass ? qam_labels(soft, hard, N, p, strm) : APSM_OK;
+            }
             // the TMA-staged form where it applies (shape, alignment; balanced over the SMs with a
             // workspace), else the converter form
             int sms = 0;

@@ -7,6 +7,7 @@
 #include "detect_tc_batch.cuh"
 #include "detect_tma.cuh"
 #include "detect_tcc.cuh"
+#include "detect_h3.cuh"
 
 namespace apsm {
 
@@ -44,6 +45,9 @@ TcBatchLauncher detect_tc_batch_launcher_m8(int kb, int *ctas_per_sm);
 TcBatchLauncher detect_tc_batch_launcher_m16(int kb, int *ctas_per_sm);
 TcBatchLauncher detect_tc_batch_launcher_m32(int kb, int *ctas_per_sm);
 TcBatchLauncher detect_tc_batch_launcher_m64(int kb, int *ctas_per_sm);
+
+H3Launcher detect_h3_launcher_m32(int kb);
+H3Launcher detect_h3_launcher_m64(int kb);
 
 TmaLauncher detect_tma_launcher_m4(int K);
 TmaLauncher detect_tma_launcher_m8(int K);
@@ -119,6 +123,12 @@ size_t detect_tcc_workspace(int M, int K, int D) {
         case 64: return detect_tcc_workspace_m64(kb, D);
         default: return 0;
     }
+}
+
+// FP32 detection with the Gram as three FP16 products; nullptr if none.
+H3Launcher detect_h3_launcher(int M, int K) {
+    const int kb = tc_user_bucket(K);
+    return M == 32 ? detect_h3_launcher_m32(kb) : (M == 64 ? detect_h3_launcher_m64(kb) : nullptr);
 }
 
 // Batched persistent detection (FP32 accuracy) for class (M, user bucket of K); nullptr if none.
