@@ -590,127 +590,152 @@ __global__ void __launch_bounds__(kBwdThreads, 6) train_bwd_kernel(const TrainBw
 }
 
 // ---- three warps per user ----------------------------------------------------------------------
-// The same recurrence and adjoint as train_bwd_kernel, for windows of at most 32 slots.  A step has
+// The same recurrence and adjoint as train_bwd_kernel, for windows below 32 slots.  A step has
 // two phases, each a set of independent pieces that one warp ran one after the other (740 warp
 // instructions and 1700 cycles a step, a third of them issuing); three warps of a user now take
 // them side by side and meet at a barrier of their own after each phase:
 //   window warp  phase 1: the window's projections (reverse: the slots' terms), lane o = window slot o;
 //                phase 2: the carried predictions (reverse: adjoints) of the window's samples
 //   row warp     phase 1: the O(S) sum over the coefficients at the sample that arrives (reverse: the
-//                pull of the one that enters), 4 kPfV entries per lane (float4) from registers loaded
-//                a step ahead, the rest directly; phase 2: the coefficients
+//                pull of the one that enters), 4 kPfV entries per lane (float4) staged ahead, the rest
+//                directly; phase 2: the coefficients
 //   filter warp  phase 1: the arriving sample's window kernel values and components, its product with
 //                the filter; phase 2: the filter
 // Every sum keeps the order it had in one warp.  kTeamUsers users of an instance per CTA.
 // @FIGT@
 constexpr int kTeamUsers = 3;
 constexpr int kTeamThreads = 96;
-constexpr int kPfV = 4;  // float4 of a row per lane and table fetched a step ahead (512 entries)
+constexpr int kPfV = 4;    // float4 of a row per lane and table that are staged ahead (512 entries)
+constexpr int kAhead = 3;  // steps ahead that global reads are issued; a ring of kAhead + 1 slots
 
-__device__ __forceinline__ float4 ldg4_if(bool c, const float *p) {  // p 16-byte aligned
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t@q ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
-                 : "+f"(v.x), "+f"(v.y), "+f"(v.z), "+f"(v.w)
-                 : "l"(p), "r"((int)c));
-    return v;
+// Reads of a later step, copied to the lane's own slots of a shared-memory ring (cp.async: no register
+// waits for them, and a lane reads only what it copied, so its own wait orders them).  A step takes
+// less than the L2 latency, so one step ahead is not enough.
+__device__ __forceinline__ void cp16(float *dst, const float *src) {  // both 16-byte aligned
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp8(float *dst, const float *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp4(float *dst, const float *src, bool ok) {  // 0 where !ok (nothing is read)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(ok ? 4 : 0)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// the copies committed kAhead - 1 or more commits ago have landed
+__device__ __forceinline__ void cp_wait_oldest() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kAhead - 1) : "memory");
 }
 
 // Entries lo4 + 4 (lane + 32 q) + 0..3 (q < kPfV, lo4 = lo rounded down to a multiple of 4, the
 // first of the four below hi) of one or two table rows (rows are padded to a multiple of 4 floats).
-struct RowPfW {
-    float4 g[kPfV], d[kPfV];
-};
-
-__device__ __forceinline__ void row_fetch_w(RowPfW &f, const float *grow, const float *drow, int lo, int hi, int lane) {
+__device__ __forceinline__ void row_copy(float *slot, const float *grow, const float *drow, int lo, int hi, int lane) {
     const int lo4 = lo & ~3;
 #pragma unroll
     for (int q = 0; q < kPfV; ++q) {
-        const int i0 = lo4 + 4 * (lane + 32 * q);
-        f.g[q] = ldg4_if(i0 < hi, grow + i0);
-        f.d[q] = ldg4_if(drow != nullptr && i0 < hi, drow + i0);
+        const int o = 4 * (lane + 32 * q), i0 = lo4 + o;
+        if (i0 < hi) {
+            cp16(slot + o, grow + i0);
+            if (drow) cp16(slot + 128 * kPfV + o, drow + i0);
+        }
     }
 }
 
 __device__ __forceinline__ float f4(const float4 &v, int e) { return e == 0 ? v.x : e == 1 ? v.y : e == 2 ? v.z : v.w; }
 
-// band of row r, entries s0 + t for t = lane (and lane + 32 when W = 32), inside [0, S)
-template <int NQ>
-__device__ __forceinline__ void band_fetch_w(BandPf &b, const TrainBwdArgs &a, int S, int W, int r, int s0, int lane) {
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        const int t = lane + 32 * q, j = s0 + t;
-        const bool ok = r >= 0 && r < S && t <= W && j >= 0 && j < S;
-        const size_t x = ok ? (size_t)r * a.Sp + j : 0;
-        b.g[q] = ldg_if(ok, a.gtab + x);
-        b.d[q] = ldg_if(ok, a.gdtab + x);
-        b.l[q] = ldg_if(ok, a.ltab + x);
-    }
+// band of row r, entries s0 + lane up to s0 + W, inside [0, S), to a slot [table][32]
+__device__ __forceinline__ void band_copy(float *slot, const TrainBwdArgs &a, int S, int W, int r, int s0, int lane) {
+    const int j = s0 + lane;
+    const bool ok = r >= 0 && r < S && lane <= W && j >= 0 && j < S;
+    const size_t x = ok ? (size_t)r * a.Sp + j : 0;
+    cp4(slot + lane, a.gtab + x, ok);
+    cp4(slot + 32 + lane, a.gdtab + x, ok);
+    cp4(slot + 64 + lane, a.ltab + x, ok);
 }
 
-template <int NQ>
-__device__ __forceinline__ void band_store_w(const BandPf &b, float *kg, float *kd, float *kl, int S, int W, int r,
-                                             int s0, int sr, int s0r, int lane) {
-    const int WR = W + 1;
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        const int t = lane + 32 * q, j = s0 + t;
-        if (r >= 0 && r < S && t <= W && j >= 0 && j < S) {
-            const int sj = ring_slot(s0r, t, WR);
-            const int u = sr * WR + sj, v = sj * WR + sr;
-            kg[u] = b.g[q];
-            kg[v] = b.g[q];
-            kd[u] = b.d[q];
-            kd[v] = b.d[q];
-            kl[u] = b.l[q];
-            kl[v] = b.l[q];
-        }
-    }
+// floats of one user's region: gamma / R [S rounded up to 4, zero padded], ca, cb [32], kg, kd, kl
+// [RB][RB], xw [RB][2M], py, pd, pw, pb [RB], w / wbar [2M], the step's sums [4], RB = bwd_ring(W);
+// then the rings of kAhead + 1 slots: rows [2][128 kPfV], bands and components [3][32] + [128] + a target
+// [4], tape [32][6] + a final adjoint [32]
+constexpr int kRowSlot = 2 * 128 * kPfV, kBandSlot = 3 * 32 + 128 + 4, kTapeSlot = 32 * 6 + 32;
+// samples of the window and the one entering or leaving it, by their low bits
+__host__ __device__ constexpr int bwd_ring(int W) { return W < 16 ? 16 : 32; }
+__host__ __device__ inline int bwd_team_rings(int S, int W, int L2) {
+    const int RB = bwd_ring(W);
+    return (((S + 3) & ~3) + 64 + 3 * RB * RB + RB * L2 + 4 * RB + L2 + 4 + 3) & ~3;
 }
-
-// floats of one user's region: gamma / R [S rounded up to 4, zero padded], kg, kd, kl [(W+1)^2],
-// xw [(W+1)][2M], py, pd, pw, pb, ca, cb [W], w / wbar [2M], the step's sums [4]
 __host__ __device__ inline int bwd_team_floats(int S, int W, int L2) {
-    const int WR = W + 1;
-    return (((S + 3) & ~3) + 3 * WR * WR + WR * L2 + 6 * W + L2 + 4 + 3) & ~3;
+    return bwd_team_rings(S, W, L2) + (kAhead + 1) * (kRowSlot + kBandSlot + kTapeSlot);
 }
 
-// WM: a bound on the window (8, 16 or 32) over which the O(W) loops are unrolled, so that their
-// shared-memory loads are independent of one another.
+// WM: a bound on the window (8, 16 or 31) over which the O(W) loops are unrolled: their operands are
+// loaded first, all in flight, and slots at or past |J_n| take a zero coefficient (the rings start at
+// zero, so every product is finite).
 template <int WM>
 __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kernel(const TrainBwdArgs a0) {
     extern __shared__ __align__(16) float sm[];
     const TrainBwdArgs a = for_instance(a0, blockIdx.y);
-    constexpr int NQ = WM >= 32 ? 2 : 1;  // band entries per lane (W + 1 <= 32 NQ)
     const int lane = threadIdx.x & 31, team = threadIdx.x / kTeamThreads, tl = threadIdx.x % kTeamThreads;
     const int role = tl >> 5;  // 0: window warp, 1: row warp, 2: filter warp
     const int k = blockIdx.x * kTeamUsers + team;
-    const int M = a.M, K = a.K, W = a.W, D = a.D, P = a.P, S = 2 * P, L2 = 2 * M, WR = W + 1;
-    float *nrm = sm, *rk = nrm + ((S + 3) & ~3);  // ||x_j||^2 and 1 / kappa_jj, shared by the users
-    float *gam = rk + ((S + 3) & ~3) + team * bwd_team_floats(S, W, L2);
+    const int M = a.M, K = a.K, W = a.W, D = a.D, P = a.P, S = 2 * P, L2 = 2 * M;
+    const int RB = bwd_ring(W), RM = RB - 1;  // sample j sits in ring slot j & RM
     const int S4 = (S + 3) & ~3;
-    float *kg = gam + S4, *kd = kg + WR * WR, *kl = kd + WR * WR, *xw = kl + WR * WR;
-    float *py = xw + WR * L2, *pd = py + W, *pw = pd + W, *pb = pw + W, *ca = pb + W, *cb = ca + W, *w = cb + W, *sums = w + L2;
+    float *nrm = sm, *rk = nrm + S4;  // ||x_j||^2 and 1 / kappa_jj, shared by the users
+    float *gam = rk + S4 + team * bwd_team_floats(S, W, L2);
+    float *ca = gam + S4, *cb = ca + 32, *kg = cb + 32, *kd = kg + RB * RB, *kl = kd + RB * RB, *xw = kl + RB * RB;
+    float *py = xw + RB * L2, *pd = py + RB, *pw = pd + RB, *pb = pw + RB, *w = pb + RB, *sums = w + L2;
+    constexpr int kRing = kAhead + 1;
+    static_assert((kRing & (kRing - 1)) == 0, "ring slots by mask");
+    float *rows = gam + bwd_team_rings(S, W, L2), *bands = rows + kRing * kRowSlot, *tapes = bands + kRing * kBandSlot;
+    auto row_slot = [&](int j) { return rows + (j & (kRing - 1)) * kRowSlot; };
+    auto band_slot = [&](int j) { return bands + (j & (kRing - 1)) * kBandSlot; };
+    auto tape_slot = [&](int n) { return tapes + (n & (kRing - 1)) * kTapeSlot; };
     Tape *tape = a.tape + (size_t)k * S * W;
     float *snap = a.snap + (size_t)k * (P > D ? P - D : 0) * W;
     const float inv_s3 = 1.f / (a.sigma * a.sigma * a.sigma);
     const float mqW = a.mu / (float)W, qW = 1.f / (float)W;
-    auto pmod = [](int x, int R) { return ((x % R) + R) % R; };
-    int sW = 0, sR = 0;  // slots of the reference sample n - W - 1 (mod W, mod W + 1)
-    auto slotW = [&](int n, int j) { return ring_slot(sW, j - (n - W - 1), W); };
-    auto slotR = [&](int n, int j) { return ring_slot(sR, j - (n - W - 1), WR); };
     auto first_centre = [&](int n) { return 2 * max(0, (n >> 1) - D + 1); };
     auto evict_step = [&](int i) { return 2 * ((i >> 1) + D); };
-    // component m of sample j as stored, and its sign (x_{2t+1}'s upper half is -Re r)
-    auto xc = [&](int j, int m) {
+    // component m of sample j as stored, to its place in a band slot, and its sign (x_{2t+1}'s upper
+    // half is -Re r)
+    auto x_copy = [&](float *slot, int j, int m) {
         const bool ok = m < L2 && j >= 0 && j < S;
         const bool up = m >= M, odd = j & 1;
         const int mm = up ? m - M : m, comp = up ? (odd ? 0 : 1) : (odd ? 1 : 0);
-        return ldg_if(ok, reinterpret_cast<const float *>(a.rx + (ok ? (size_t)(j >> 1) * M + mm : 0)) + comp);
+        cp4(slot + 96 + m, reinterpret_cast<const float *>(a.rx + (ok ? (size_t)(j >> 1) * M + mm : 0)) + comp, ok);
     };
     auto xsign = [&](int j, int m, float v) { return (m >= M && (j & 1)) ? -v : v; };
-    auto wrap = [&](int x) { return x >= WR ? x - WR : x; };  // x < 2 (W + 1)
-    auto target_at = [&](bool ok, int j) {
-        return ldg_if(ok, reinterpret_cast<const float *>(a.sym + (ok ? (size_t)(j >> 1) * K + k : 0)) + (j & 1));
+    // the band a slot holds, into the window rings at (r, s0 + t) and (s0 + t, r): the tables are
+    // exactly symmetric
+    auto band_store = [&](const float *slot, int r, int s0) {
+        const int j = s0 + lane;
+        if (r >= 0 && r < S && lane <= W && j >= 0 && j < S) {
+            const int u = (r & RM) * RB + (j & RM), v = (j & RM) * RB + (r & RM);
+            const float g = slot[lane], d = slot[32 + lane], l = slot[64 + lane];
+            kg[u] = g;
+            kg[v] = g;
+            kd[u] = d;
+            kd[v] = d;
+            kl[u] = l;
+            kl[v] = l;
+        }
+    };
+    // w += sum_o ca_o x_{jlo+o}, component by component in slot order
+    auto filter_update = [&](int jlo, int nJ) {
+        float c[WM];
+#pragma unroll
+        for (int o = 0; o < WM; ++o) c[o] = ca[o];
+#pragma unroll
+        for (int o = 0; o < WM; ++o) c[o] = o < nJ ? c[o] : 0.f;
+        for (int m = lane; m < L2; m += 32) {
+            float x[WM], acc = w[m];
+#pragma unroll
+            for (int o = 0; o < WM; ++o) x[o] = xw[((jlo + o) & RM) * L2 + m];
+#pragma unroll
+            for (int o = 0; o < WM; ++o) acc = fmaf(c[o], x[o], acc);
+            w[m] = acc;
+        }
     };
 
     for (int i = threadIdx.x; i < S; i += blockDim.x) {
@@ -721,99 +746,108 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
     __syncthreads();  // the only block barrier: nrm and rk are shared by the users
     if (k >= K) return;
     auto team_sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(kTeamThreads) : "memory"); };
-    for (int i = tl; i < S4; i += kTeamThreads) gam[i] = 0.f;
+    for (int i = tl; i < S4 + 64 + 3 * RB * RB + RB * L2 + 4 * RB; i += kTeamThreads) gam[i] = 0.f;  // and every ring
     for (int m = tl; m < M; m += kTeamThreads) {
         const float2 c = a.clin0 ? a.clin0[m * K + k] : make_float2(0.f, 0.f);
         w[m] = c.x;
         w[M + m] = c.y;
     }
-    RowPfW pf;
-    BandPf bp;
-    float xn[4];
     if (a.mode & 1) {
-        sW = pmod(-W - 1, W);
-        sR = pmod(-W - 1, WR);
-        float bn = 0.f;  // the next arrival's target, a step early
-        if (role == 2) {
-            band_fetch_w<NQ>(bp, a, S, W, 0, -W, lane);
-            band_store_w<NQ>(bp, kg, kd, kl, S, W, 0, -W, slotR(0, 0), slotR(0, -W), lane);
-            band_fetch_w<NQ>(bp, a, S, W, 1, 1 - W, lane);
+        // what arrival j needs: its rows (row warp), its band, components and target (filter warp)
+        auto fetch_row = [&](int j) {
+            if (j < S)
+                row_copy(row_slot(j), a.gtab + (size_t)j * a.Sp, a.gdtab + (size_t)j * a.Sp, first_centre(j), j, lane);
+            cp_commit();
+        };
+        auto fetch_arrival = [&](int j) {
+            float *slot = band_slot(j);
+            band_copy(slot, a, S, W, j, j - W, lane);
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int m = lane + 32 * c;
-                if (m < L2) xw[slotR(0, 0) * L2 + m] = xcomp(a.rx, M, 0, m);
-                xn[c] = xc(1, m);
-            }
-            bn = target_at(lane == 0 && S > 1, 1);
-            if (lane == 0) pb[0] = target_at(true, 0);
-        } else if (role == 1) {
-            if (S > 1) row_fetch_w(pf, a.gtab + a.Sp, a.gdtab + a.Sp, first_centre(1), 1, lane);
-        }
+            for (int c = 0; c < 4; ++c)
+                if (32 * c < L2) x_copy(slot, j, lane + 32 * c);
+            if (lane == 0)
+                cp4(slot + 224, reinterpret_cast<const float *>(a.sym + (j < S ? (size_t)(j >> 1) * K + k : 0)) + (j & 1), j < S);
+            cp_commit();
+        };
         team_sync();
         if (role == 2) {
+            for (int j = 0; j < kAhead; ++j) fetch_arrival(j);
+            cp_wait_oldest();
+            const float *slot = band_slot(0);
+            band_store(slot, 0, -W);
             float ws = 0.f;
-            for (int m = lane; m < L2; m += 32) ws = fmaf(w[m], xw[slotR(0, 0) * L2 + m], ws);
+            for (int m = lane; m < L2; m += 32) {
+                const float x = xsign(0, m, slot[96 + m]);
+                xw[m] = x;
+                ws = fmaf(w[m], x, ws);
+            }
             ws = warp_sum(ws);
             if (lane == 0) {
+                pb[0] = slot[224];
                 py[0] = 0.f;
                 pd[0] = 0.f;
                 pw[0] = ws;
             }
+            fetch_arrival(kAhead);
+        } else if (role == 1) {
+            for (int j = 1; j <= kAhead; ++j) fetch_row(j);
         }
         team_sync();
 
         // ---- forward ---------------------------------------------------------------------------------------
-        for (int n = 0; n < S; ++n, sW = ring_slot(sW, 1, W), sR = ring_slot(sR, 1, WR)) {
+        for (int n = 0; n < S; ++n) {
             const int jlo = max(0, n - W + 1), nJ = n - jlo + 1, jn = n + 1;
-            const float mq = nJ == W ? mqW : a.mu / (float)nJ;
-            float b_jn = 0.f;
             // phase 1, from the state before this step
             if (role == 0) {
                 if (lane < nJ) {  // the window's projections (Eq. beta), all from f_n
-                    const int j = jlo + lane, r = slotW(n, j);
-                    const float dw = pw[r], yg = py[r], gd = pd[r];
+                    const float mq = nJ == W ? mqW : a.mu / (float)nJ;
+                    const int j = jlo + lane, r = j & RM;
+                    const float dw = pw[r], yg = py[r], gd = pd[r], r_k = rk[j], gj = gam[j], bj = pb[r];
+                    const float kap = fmaf(a.wL, nrm[j], a.wG);
                     const float y = fmaf(a.wL, dw, a.wG * yg);
-                    const float e = y - pb[r];
-                    const float kap = fmaf(a.wL, nrm[j], a.wG), r_k = rk[j];
+                    const float e = y - bj;
                     float beta = 0.f, s = 0.f;
                     if (kap != 0.f) {
                         if (e < -a.eps) { s = 1.f; beta = (-e - a.eps) * r_k; }
                         else if (e > a.eps) { s = -1.f; beta = (-e + a.eps) * r_k; }
                     }
-                    tape[(size_t)n * W + lane] = Tape{beta, s, kap, dw, yg, gd};
                     ca[lane] = mq * beta;
-                    cb[lane] = gam[j] + mq * beta;  // the coefficient after the step
+                    cb[lane] = gj + mq * beta;  // the coefficient after the step
+                    tape[(size_t)n * W + lane] = Tape{beta, s, kap, dw, yg, gd};
                 }
             } else if (role == 1) {
                 if (jn < S) {
-                    float ys = 0.f, ds = 0.f;  // the arrival's sums
+                    cp_wait_oldest();
+                    const float *pg = row_slot(jn) + 4 * lane, *pdv = pg + 128 * kPfV;  // this lane's entries
                     const int lo = first_centre(jn), lo4 = lo & ~3;
+                    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+                    float4 gm[kPfV], gv[kPfV], dv[kPfV];
+#pragma unroll
+                    for (int q = 0; q < kPfV; ++q) {
+                        const int i0 = lo4 + 4 * (lane + 32 * q);
+                        const bool in = i0 < jn;
+                        gm[q] = in ? *reinterpret_cast<const float4 *>(gam + i0) : z4;
+                        gv[q] = in ? *reinterpret_cast<const float4 *>(pg + 128 * q) : z4;
+                        dv[q] = in ? *reinterpret_cast<const float4 *>(pdv + 128 * q) : z4;
+                    }
                     float y2[2] = {0.f, 0.f}, d2[2] = {0.f, 0.f};  // two chains of sums
                     if (lo == 0) {  // nothing evicted yet: gamma is zero from jn on (padding included)
 #pragma unroll
                         for (int q = 0; q < kPfV; ++q) {
-                            const int i0 = 4 * (lane + 32 * q);
-                            if (i0 < jn) {
-                                const float4 gm = *reinterpret_cast<const float4 *>(gam + i0);
-                                y2[0] = fmaf(gm.x, pf.g[q].x, fmaf(gm.z, pf.g[q].z, y2[0]));
-                                y2[1] = fmaf(gm.y, pf.g[q].y, fmaf(gm.w, pf.g[q].w, y2[1]));
-                                d2[0] = fmaf(gm.x, pf.d[q].x, fmaf(gm.z, pf.d[q].z, d2[0]));
-                                d2[1] = fmaf(gm.y, pf.d[q].y, fmaf(gm.w, pf.d[q].w, d2[1]));
-                            }
+                            y2[0] = fmaf(gm[q].x, gv[q].x, fmaf(gm[q].z, gv[q].z, y2[0]));
+                            y2[1] = fmaf(gm[q].y, gv[q].y, fmaf(gm[q].w, gv[q].w, y2[1]));
+                            d2[0] = fmaf(gm[q].x, dv[q].x, fmaf(gm[q].z, dv[q].z, d2[0]));
+                            d2[1] = fmaf(gm[q].y, dv[q].y, fmaf(gm[q].w, dv[q].w, d2[1]));
                         }
                     } else {
 #pragma unroll
                         for (int q = 0; q < kPfV; ++q) {
-                            const int i0 = lo4 + 4 * (lane + 32 * q);
-                            if (i0 < jn) {
-                                const float4 gm = *reinterpret_cast<const float4 *>(gam + i0);
 #pragma unroll
-                                for (int e = 0; e < 4; ++e) {
-                                    const int i = i0 + e;
-                                    if (i >= lo && i < jn) {
-                                        y2[e & 1] = fmaf(f4(gm, e), f4(pf.g[q], e), y2[e & 1]);
-                                        d2[e & 1] = fmaf(f4(gm, e), f4(pf.d[q], e), d2[e & 1]);
-                                    }
+                            for (int e = 0; e < 4; ++e) {
+                                const int i = lo4 + 4 * (lane + 32 * q) + e;
+                                if (i >= lo && i < jn) {
+                                    y2[e & 1] = fmaf(f4(gm[q], e), f4(gv[q], e), y2[e & 1]);
+                                    d2[e & 1] = fmaf(f4(gm[q], e), f4(dv[q], e), d2[e & 1]);
                                 }
                             }
                         }
@@ -823,82 +857,61 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
                         y2[0] = fmaf(gam[i], __ldg(grow + i), y2[0]);
                         d2[0] = fmaf(gam[i], __ldg(drow + i), d2[0]);
                     }
-                    ys = y2[0] + y2[1];
-                    ds = d2[0] + d2[1];
-                    if (jn + 1 < S)
-                        row_fetch_w(pf, a.gtab + (size_t)(jn + 1) * a.Sp, a.gdtab + (size_t)(jn + 1) * a.Sp,
-                                    first_centre(jn + 1), jn + 1, lane);
-                    ys = warp_sum(ys);
-                    ds = warp_sum(ds);
+                    const float ys = warp_sum(y2[0] + y2[1]), ds = warp_sum(d2[0] + d2[1]);
                     if (lane == 0) {
                         sums[0] = ys;
                         sums[1] = ds;
                     }
                 }
-            } else {
-                b_jn = bn;
-                bn = target_at(lane == 0 && jn + 1 < S, jn + 1);
-                if (jn < S) {
-                    float ws = 0.f;
-                    band_store_w<NQ>(bp, kg, kd, kl, S, W, jn, jn - W, slotR(n, jn), slotR(n, jn - W), lane);
-                    band_fetch_w<NQ>(bp, a, S, W, jn + 1, jn + 1 - W, lane);
-                    const int sx = slotR(n, jn) * L2;
+            } else if (jn < S) {
+                cp_wait_oldest();
+                const float *slot = band_slot(jn);
+                band_store(slot, jn, jn - W);
+                float ws = 0.f;
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const int m = lane + 32 * c;
-                        if (m < L2) {
-                            const float x = xsign(jn, m, xn[c]);
-                            xw[sx + m] = x;
-                            ws = fmaf(w[m], x, ws);
-                            xn[c] = xc(jn + 1, m);
-                        }
+                for (int c = 0; c < 4; ++c) {
+                    const int m = lane + 32 * c;
+                    if (m < L2) {
+                        const float x = xsign(jn, m, slot[96 + m]);
+                        xw[(jn & RM) * L2 + m] = x;
+                        ws = fmaf(w[m], x, ws);
                     }
-                    ws = warp_sum(ws);
-                    if (lane == 0) sums[2] = ws;
                 }
+                ws = warp_sum(ws);
+                if (lane == 0) sums[2] = ws;
             }
             team_sync();
             // phase 2, Eq. apsm: coefficients, linear part, carried predictions of J_{n+1} (2D = W + 1: the
             // oldest centre of J_n leaves before step n+1)
-            const int s_lo = slotR(n, jlo);
             if (role == 1) {
                 if (lane < nJ) gam[jlo + lane] = cb[lane];
+                if (jn < S) fetch_row(jn + kAhead);
             } else if (role == 2) {
-                if (lane == 0 && jn < S) pb[slotW(n, jn)] = b_jn;
-                for (int m = lane; m < L2; m += 32) {
-                    float acc = w[m];
-#pragma unroll
-                    for (int o = 0; o < WM; ++o)
-                        if (o < nJ) acc = fmaf(ca[o], xw[wrap(s_lo + o) * L2 + m], acc);
-                    w[m] = acc;
-                }
+                if (lane == 0 && jn < S) pb[jn & RM] = band_slot(jn)[224];
+                filter_update(jlo, nJ);
+                if (jn < S) fetch_arrival(jn + kAhead);
             } else {
                 const int t_lo = max(0, n - W + 2), n_t = jn < S ? jn - t_lo + 1 : 0;
                 const int e_lo = first_centre(n), e_hi = jn < S ? first_centre(jn) : e_lo;
                 if (lane < n_t) {
-                    const int j = t_lo + lane, r = slotW(n, j), sj = slotR(n, j) * WR;
-                    float ay, ad, aw;
-                    if (j == jn) {
-                        ay = sums[0];
-                        ad = sums[1];
-                        aw = sums[2];
-                    } else {
-                        ay = py[r];
-                        ad = pd[r];
-                        aw = pw[r];
+                    const int j = t_lo + lane, r = j & RM;
+                    float c[WM], vg[WM], vd[WM], vl[WM];
+#pragma unroll
+                    for (int o = 0; o < WM; ++o) {
+                        const int x = ((jlo + o) & RM) * RB + r;
+                        c[o] = ca[o];
+                        vg[o] = kg[x];
+                        vd[o] = kd[x];
+                        vl[o] = kl[x];
                     }
+                    float ay = j == jn ? sums[0] : py[r], ad = j == jn ? sums[1] : pd[r], aw = j == jn ? sums[2] : pw[r];
                     const int o_lo = j == jn ? max(0, e_hi - jlo) : 0;
 #pragma unroll
                     for (int o = 0; o < WM; ++o) {
-                        if (o < nJ) {
-                            const int si = sj + wrap(s_lo + o);
-                            const float c = ca[o];
-                            aw = fmaf(c, kl[si], aw);
-                            if (o >= o_lo) {
-                                ay = fmaf(c, kg[si], ay);
-                                ad = fmaf(c, kd[si], ad);
-                            }
-                        }
+                        const float cl = o < nJ ? c[o] : 0.f, cg = o >= o_lo ? cl : 0.f;
+                        aw = fmaf(cl, vl[o], aw);
+                        ay = fmaf(cg, vg[o], ay);
+                        ad = fmaf(cg, vd[o], ad);
                     }
                     if (j != jn) {
                         const float *grow = a.gtab + (size_t)j * a.Sp, *drow = a.gdtab + (size_t)j * a.Sp;
@@ -920,18 +933,19 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
     if (!(a.mode & 2)) return;
 
     // ---- reverse sweep ---------------------------------------------------------------------------------
+    asm volatile("cp.async.wait_all;" ::: "memory");  // the rings of slots are free
+    team_sync();
     {  // kernel values and components of the last W + 1 samples (as the forward left them)
         const int j0 = max(0, S - W - 1), nr = S - j0;
         for (int t = tl; t < nr * nr; t += kTeamThreads) {
             const int i = j0 + t / nr, j = j0 + t % nr;
             const size_t x = (size_t)i * a.Sp + j;
-            const int u = (i % WR) * WR + j % WR;
-            kg[u] = a.gtab[x];
-            kl[u] = a.ltab[x];
+            kg[(i & RM) * RB + (j & RM)] = a.gtab[x];
+            kl[(i & RM) * RB + (j & RM)] = a.ltab[x];
         }
         for (int t = tl; t < nr * L2; t += kTeamThreads) {
             const int j = j0 + t / L2, m = t % L2;
-            xw[(j % WR) * L2 + m] = xcomp(a.rx, M, j, m);
+            xw[(j & RM) * L2 + m] = xcomp(a.rx, M, j, m);
         }
     }
     for (int i = tl; i < S4; i += kTeamThreads) gam[i] = 0.f;  // R
@@ -941,69 +955,83 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
         w[M + m] = d.y;
     }
     const int alive0 = max(0, P - D);
-    auto final_at = [&](int j) {
-        const bool ok = j >= 0 && (j >> 1) >= alive0;
+    auto final_src = [&](int j, bool &ok) {
+        ok = j >= 0 && (j >> 1) >= alive0;
         int t = j >> 1;  // its ring slot: t mod D (t < D unless entries were evicted)
         if (P > D) t %= D;
-        return ldg_if(ok, a.dgamma + (ok ? ((size_t)t * 2 + (j & 1)) * K + k : 0));
+        return a.dgamma + (ok ? ((size_t)t * 2 + (j & 1)) * K + k : 0);
     };
     auto pull_hi = [&](int n) {
         const int e = evict_step(n - W);
         return e > n + 1 ? min(e, S) : n - W + 2;
     };
-    team_sync();
-    const int je0 = S - 1 - W;
-    float fa = 0.f;  // window warp: the entrant's final adjoint, a step early
-    Tape tnext;
-    auto tape_at = [&](Tape &t, bool ok, int n) {
-        const float *f = reinterpret_cast<const float *>(tape + (ok ? (size_t)n * W + lane : 0));
-        const float2 u0 = ld2_if(ok, f), u1 = ld2_if(ok, f + 2), u2 = ld2_if(ok, f + 4);
-        t = Tape{u0.x, u0.y, u1.x, u1.y, u2.x, u2.y};
+    // what step n of the sweep needs: its tape, the final adjoint of its entrant n - W and that entrant's
+    // row (row warp), the entrant's band and components (filter warp)
+    auto fetch_step = [&](int n) {
+        float *slot = tape_slot(n);
+        const int j = n - W;
+        if (n >= 0 && lane < min(n + 1, W)) {
+            const float *f = reinterpret_cast<const float *>(tape + (size_t)n * W + lane);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) cp8(slot + 6 * lane + 2 * i, f + 2 * i);
+        }
+        bool ok;
+        const float *fs = final_src(j, ok);
+        if (lane == 0) cp4(slot + 192, fs, ok);
+        if (j >= 0) row_copy(row_slot(n), a.gtab + (size_t)j * a.Sp, nullptr, j + 2, pull_hi(n), lane);
+        cp_commit();
     };
+    auto fetch_entrant = [&](int n) {
+        float *slot = band_slot(n);
+        band_copy(slot, a, S, W, n - W, n - W, lane);
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+            if (32 * c < L2) x_copy(slot, n - W, lane + 32 * c);
+        cp_commit();
+    };
+    team_sync();
     if (role == 0) {
         for (int j = max(0, S - W) + lane; j < S; j += 32) {  // abar of the last window (xw holds them)
             float d = 0.f;
-            const int sx = pmod(j, WR) * L2;
-            for (int m = 0; m < L2; ++m) d = fmaf(w[m], xw[sx + m], d);
-            py[j % W] = d + final_at(j);
+            for (int m = 0; m < L2; ++m) d = fmaf(w[m], xw[(j & RM) * L2 + m], d);
+            bool ok;
+            const float *fs = final_src(j, ok);
+            py[j & RM] = d + (ok ? __ldg(fs) : 0.f);
         }
-        fa = final_at(je0);
-        tape_at(tnext, lane < S - max(0, S - W), S - 1);
     } else if (role == 1) {
-        if (je0 >= 0) row_fetch_w(pf, a.gtab + (size_t)je0 * a.Sp, nullptr, je0 + 2, pull_hi(S - 1), lane);
+        for (int i = 0; i < kAhead; ++i) fetch_step(S - 1 - i);
+        cp_wait_oldest();
     } else {
-        band_fetch_w<NQ>(bp, a, S, W, je0, je0, lane);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) xn[c] = xc(je0, lane + 32 * c);
+        for (int i = 0; i < kAhead; ++i) fetch_entrant(S - 1 - i);
     }
-    sW = pmod(S - 1 - W - 1, W);
-    sR = pmod(S - 1 - W - 1, WR);
     team_sync();
     float sig_bar = 0.f, mu_bar = 0.f, eps_bar = 0.f, wl_bar = 0.f;  // lane o: window slot o's terms
-    for (int n = S - 1; n >= 0; --n, sW = ring_slot(sW, W - 1, W), sR = ring_slot(sR, WR - 1, WR)) {
+    for (int n = S - 1; n >= 0; --n) {
         const int jlo = max(0, n - W + 1), nJ = n - jlo + 1, je = n - W;
-        const float q = nJ == W ? qW : 1.f / (float)nJ;
         float fa_je = 0.f;
         // phase 1, from the adjoint of S_{n+1}
         if (role == 0) {
-            fa_je = fa;
-            fa = final_at(je - 1);
+            const float *slot = tape_slot(n);  // (landed before the last barrier)
+            fa_je = slot[192];
             if (lane < nJ) {
-                const Tape tp = tnext;
-                tape_at(tnext, n > 0 && lane < n - max(0, n - W), n - 1);
+                const float q = nJ == W ? qW : 1.f / (float)nJ;
+                const float2 u0 = *reinterpret_cast<const float2 *>(slot + 6 * lane),
+                             u1 = *reinterpret_cast<const float2 *>(slot + 6 * lane + 2),
+                             u2 = *reinterpret_cast<const float2 *>(slot + 6 * lane + 4);
+                const Tape tp{u0.x, u0.y, u1.x, u1.y, u2.x, u2.y};
                 const int j = jlo + lane;
-                const float ab = py[slotW(n, j)];
+                const float ab = py[j & RM], r_k = rk[j], nj = nrm[j];
                 mu_bar += q * tp.beta * ab;
                 const float bbar = a.mu * q * ab;
                 float cwo = 0.f, cgo = 0.f;
                 if (tp.s != 0.f) {
-                    const float ybar = -bbar * rk[j];
-                    eps_bar += tp.s * ybar;
-                    wl_bar += (ybar * tp.beta) * (nrm[j] - 1.f);
-                    wl_bar += ybar * (tp.dotw - tp.gauss);
-                    sig_bar += ybar * a.wG * tp.gd2 * inv_s3;
+                    const float ybar = -bbar * r_k;
                     cwo = ybar * a.wL;
                     cgo = ybar * a.wG;
+                    eps_bar += tp.s * ybar;
+                    wl_bar += (ybar * tp.beta) * (nj - 1.f);
+                    wl_bar += ybar * (tp.dotw - tp.gauss);
+                    sig_bar += ybar * a.wG * tp.gd2 * inv_s3;
                 }
                 ca[lane] = cwo;
                 cb[lane] = cgo;
@@ -1014,60 +1042,58 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
                 snap[(size_t)((e >> 1) - D) * W + lane] = gam[e - W + 1 + lane];
             }
             if (je >= 0) {
-                float gs = 0.f;
+                const float *pg = row_slot(n) + 4 * lane;
                 const int lo = je + 2, hi = pull_hi(n), e = evict_step(je);
                 const int s_lo = e <= S - 1 ? e - W + 1 : S;
                 const float *sv = snap + (size_t)((e >> 1) - D) * W;
                 const float *grow = a.gtab + (size_t)je * a.Sp;
                 const int lo4 = lo & ~3;
+                const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
+                float4 rm[kPfV], gv[kPfV];
+#pragma unroll
+                for (int q = 0; q < kPfV; ++q) {
+                    const int i0 = lo4 + 4 * (lane + 32 * q);
+                    const bool in = i0 < hi;
+                    rm[q] = in ? *reinterpret_cast<const float4 *>(gam + i0) : z4;
+                    gv[q] = in ? *reinterpret_cast<const float4 *>(pg + 128 * q) : z4;
+                }
                 float g2[2] = {0.f, 0.f};
                 if (hi == S && s_lo >= S) {  // no eviction after the entrant: R is zero below lo and past S
 #pragma unroll
-                    for (int qq = 0; qq < kPfV; ++qq) {
-                        const int i0 = lo4 + 4 * (lane + 32 * qq);
-                        if (i0 < hi) {
-                            const float4 rm = *reinterpret_cast<const float4 *>(gam + i0);
-                            g2[0] = fmaf(rm.x, pf.g[qq].x, fmaf(rm.z, pf.g[qq].z, g2[0]));
-                            g2[1] = fmaf(rm.y, pf.g[qq].y, fmaf(rm.w, pf.g[qq].w, g2[1]));
-                        }
+                    for (int q = 0; q < kPfV; ++q) {
+                        g2[0] = fmaf(rm[q].x, gv[q].x, fmaf(rm[q].z, gv[q].z, g2[0]));
+                        g2[1] = fmaf(rm[q].y, gv[q].y, fmaf(rm[q].w, gv[q].w, g2[1]));
                     }
                 } else {
 #pragma unroll
-                    for (int qq = 0; qq < kPfV; ++qq) {
-                        const int i0 = lo4 + 4 * (lane + 32 * qq);
-                        if (i0 < hi) {
-                            const float4 rm = *reinterpret_cast<const float4 *>(gam + i0);
+                    for (int q = 0; q < kPfV; ++q) {
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const int i = i0 + e;
-                                if (i >= lo && i < hi) {
-                                    const float r = i >= s_lo ? f4(rm, e) - sv[i - s_lo] : f4(rm, e);
-                                    g2[e & 1] = fmaf(r, f4(pf.g[qq], e), g2[e & 1]);
-                                }
+                        for (int c = 0; c < 4; ++c) {
+                            const int i = lo4 + 4 * (lane + 32 * q) + c;
+                            if (i >= lo && i < hi) {
+                                const float r = i >= s_lo ? f4(rm[q], c) - sv[i - s_lo] : f4(rm[q], c);
+                                g2[c & 1] = fmaf(r, f4(gv[q], c), g2[c & 1]);
                             }
                         }
                     }
                 }
                 for (int i = max(lo, lo4 + 4 * 32 * kPfV) + lane; i < hi; i += 32)
                     g2[0] = fmaf(i >= s_lo ? gam[i] - sv[i - s_lo] : gam[i], __ldg(grow + i), g2[0]);
-                gs = g2[0] + g2[1];
-                if (je - 1 >= 0) row_fetch_w(pf, a.gtab + (size_t)(je - 1) * a.Sp, nullptr, je + 1, pull_hi(n - 1), lane);
-                gs = warp_sum(gs);
+                const float gs = warp_sum(g2[0] + g2[1]);
                 if (lane == 0) sums[0] = gs;
             }
         } else if (je >= 0) {
+            cp_wait_oldest();
+            const float *slot = band_slot(n);
+            band_store(slot, je, je);
             float ls = 0.f;
-            band_store_w<NQ>(bp, kg, kd, kl, S, W, je, je, slotR(n, je), slotR(n, je), lane);
-            band_fetch_w<NQ>(bp, a, S, W, je - 1, je - 1, lane);
-            const int sx = slotR(n, je) * L2;
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 const int m = lane + 32 * c;
                 if (m < L2) {
-                    const float x = xsign(je, m, xn[c]);
-                    xw[sx + m] = x;
+                    const float x = xsign(je, m, slot[96 + m]);
+                    xw[(je & RM) * L2 + m] = x;
                     ls = fmaf(w[m], x, ls);
-                    xn[c] = xc(je - 1, m);
                 }
             }
             ls = warp_sum(ls);
@@ -1075,36 +1101,32 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
         }
         team_sync();
         // phase 2: the adjoint of S_n
-        const int s_lo = slotR(n, jlo);
         if (role == 1) {
             if (lane < nJ) gam[jlo + lane] += cb[lane];
+            fetch_step(n - kAhead);
+            cp_wait_oldest();  // step n - 1's copies, for the window warp too
         } else if (role == 2) {
-            for (int m = lane; m < L2; m += 32) {
-                float acc = w[m];
-#pragma unroll
-                for (int o = 0; o < WM; ++o)
-                    if (o < nJ) acc = fmaf(ca[o], xw[wrap(s_lo + o) * L2 + m], acc);
-                w[m] = acc;
-            }
+            filter_update(jlo, nJ);
+            fetch_entrant(n - kAhead);
         } else {
             const int t_lo = max(0, n - W), n_t = n - t_lo;
             if (lane < n_t) {
-                const int j = t_lo + lane, r = slotW(n, j), sj = slotR(n, j) * WR;
-                float acc;
-                bool alive = true;
-                if (j == je) {
-                    acc = fa_je + sums[0] + sums[1];
-                    alive = n < evict_step(j);
-                } else {
-                    acc = py[r];
-                }
+                const int j = t_lo + lane, r = j & RM;
+                float c[WM], b[WM], vg[WM], vl[WM];
 #pragma unroll
                 for (int o = 0; o < WM; ++o) {
-                    if (o < nJ) {
-                        const int si = sj + wrap(s_lo + o);
-                        acc = fmaf(ca[o], kl[si], acc);
-                        if (alive) acc = fmaf(cb[o], kg[si], acc);
-                    }
+                    const int x = ((jlo + o) & RM) * RB + r;
+                    c[o] = ca[o];
+                    b[o] = cb[o];
+                    vg[o] = kg[x];
+                    vl[o] = kl[x];
+                }
+                const bool alive = j != je || n < evict_step(j);
+                float acc = j == je ? fa_je + sums[0] + sums[1] : py[r];
+#pragma unroll
+                for (int o = 0; o < WM; ++o) {
+                    acc = fmaf(o < nJ ? c[o] : 0.f, vl[o], acc);
+                    acc = fmaf(o < nJ && alive ? b[o] : 0.f, vg[o], acc);
                 }
                 py[r] = acc;
             }
@@ -1115,7 +1137,7 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
     if (role == 2)
         for (int m = lane; m < M; m += 32) a.dclin0[m * K + k] = make_float2(w[m], w[M + m]);
     // slot partials combined in slot order
-    float *red = py;  // py, pd, pw, pb: 4 W floats
+    float *red = kg;
     if (role == 0) {
         if (lane < W) {
             red[4 * lane + 0] = sig_bar;
@@ -1204,7 +1226,7 @@ apsm_status train_bwd_run(const apsm_params *p, int n, const float *rx_pilot, co
     const size_t smem_w =
         sizeof(float) * (2 * (size_t)((2 * P + 3) & ~3) +
                          (size_t)std::min(p->K, kTeamUsers) * bwd_team_floats(2 * P, p->window, 2 * p->M));
-    const bool team_form = p->window <= 32 && smem_w <= 227 * 1024;
+    const bool team_form = p->window < 32 && smem_w <= 227 * 1024;
     if (!team_form && smem > 227 * 1024) return APSM_ERR_UNSUPPORTED;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) {
@@ -1255,7 +1277,7 @@ apsm_status train_bwd_run(const apsm_params *p, int n, const float *rx_pilot, co
     if (mode & 1) train_bwd_tables_kernel<<<dim3(blocks, n), 256, 0, strm>>>(a);
     if (team_form) {
         auto kern = p->window <= 8 ? train_bwd_team_kernel<8>
-                    : p->window <= 16 ? train_bwd_team_kernel<16> : train_bwd_team_kernel<32>;
+                    : p->window <= 16 ? train_bwd_team_kernel<16> : train_bwd_team_kernel<31>;
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_w) != cudaSuccess)
             return APSM_ERR_CUDA;
         const int users = std::min(p->K, kTeamUsers);
