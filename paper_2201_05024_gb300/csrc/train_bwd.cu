@@ -589,22 +589,25 @@ __global__ void __launch_bounds__(kBwdThreads, 6) train_bwd_kernel(const TrainBw
     }
 }
 
-// ---- three warps per user ----------------------------------------------------------------------
-// The same recurrence and adjoint as train_bwd_kernel, for windows below 32 slots.  A step has
+// ---- four warps per user -----------------------------------------------------------------------
+// The same recurrence and adjoint as train_bwd_kernel, for windows of at most 30 slots.  A step has
 // two phases, each a set of independent pieces that one warp ran one after the other (740 warp
-// instructions and 1700 cycles a step, a third of them issuing); three warps of a user now take
+// instructions and 1700 cycles a step, a third of them issuing); four warps of a user now take
 // them side by side and meet at a barrier of their own after each phase:
-//   window warp  phase 1: the window's projections (reverse: the slots' terms), lane o = window slot o;
-//                phase 2: the carried predictions (reverse: adjoints) of the window's samples
-//   row warp     phase 1: the O(S) sum over the coefficients at the sample that arrives (reverse: the
-//                pull of the one that enters), 4 kPfV entries per lane (float4) staged ahead, the rest
-//                directly; phase 2: the coefficients
-//   filter warp  phase 1: the arriving sample's window kernel values and components, its product with
-//                the filter; phase 2: the filter
-// Every sum keeps the order it had in one warp.  kTeamUsers users of an instance per CTA.
-// @FIGT@
+//   window warp   phase 1: the window's projections (reverse: the slots' terms), lane o = window slot o;
+//                 phase 2: the carried predictions (reverse: adjoints) of the window's samples
+//   row warp      phase 1: the O(S) sum over the coefficients at the sample that arrives (reverse: the
+//                 pull of the one that enters), 4 kPfV entries per lane (float4) staged ahead, the rest
+//                 directly; phase 2: the coefficients
+//   filter warp   phase 1: the arriving sample's product with the filter; phase 2: the filter
+//   staging warp  phase 1: the next arrival's kernel values and components into the window rings;
+//                 phase 2: the copies of the one kAhead steps later
+// Every sum keeps the order it had in one warp.  A step is bound by the instructions and latencies
+// of its longest warp in each phase.  kTeamUsers users of an instance per CTA.
+// 16 antennas, 6 users, 256 pilots, W = 8: one call 1.71 ms as one warp per user, about 0.75 ms here
+// (cycle stamps per real-split step: forward 600 + 950, reverse 580 + 780).
 constexpr int kTeamUsers = 3;
-constexpr int kTeamThreads = 96;
+constexpr int kTeamThreads = 128;
 constexpr int kPfV = 4;    // float4 of a row per lane and table that are staged ahead (512 entries)
 constexpr int kAhead = 3;  // steps ahead that global reads are issued; a ring of kAhead + 1 slots
 
@@ -654,21 +657,22 @@ __device__ __forceinline__ void band_copy(float *slot, const TrainBwdArgs &a, in
 }
 
 // floats of one user's region: gamma / R [S rounded up to 4, zero padded], ca, cb [32], kg, kd, kl
-// [RB][RB], xw [RB][2M], py, pd, pw, pb [RB], w / wbar [2M], the step's sums [4], RB = bwd_ring(W);
+// [RB][RB], xw [RB][2M], py, pd, pw, pb [RB], w / wbar [2M], the step's sums [4], four zeros, RB = bwd_ring(W);
 // then the rings of kAhead + 1 slots: rows [2][128 kPfV], bands and components [3][32] + [128] + a target
 // [4], tape [32][6] + a final adjoint [32]
 constexpr int kRowSlot = 2 * 128 * kPfV, kBandSlot = 3 * 32 + 128 + 4, kTapeSlot = 32 * 6 + 32;
-// samples of the window and the one entering or leaving it, by their low bits
-__host__ __device__ constexpr int bwd_ring(int W) { return W < 16 ? 16 : 32; }
+// samples of the window, the one entering or leaving it and the one staged for the next step, by
+// their low bits
+__host__ __device__ constexpr int bwd_ring(int W) { return W + 2 <= 16 ? 16 : 32; }
 __host__ __device__ inline int bwd_team_rings(int S, int W, int L2) {
     const int RB = bwd_ring(W);
-    return (((S + 3) & ~3) + 64 + 3 * RB * RB + RB * L2 + 4 * RB + L2 + 4 + 3) & ~3;
+    return (((S + 3) & ~3) + 64 + 3 * RB * RB + RB * L2 + 4 * RB + ((L2 + 3) & ~3) + 4 + 4 + 3) & ~3;
 }
 __host__ __device__ inline int bwd_team_floats(int S, int W, int L2) {
     return bwd_team_rings(S, W, L2) + (kAhead + 1) * (kRowSlot + kBandSlot + kTapeSlot);
 }
 
-// WM: a bound on the window (8, 16 or 31) over which the O(W) loops are unrolled: their operands are
+// WM: a bound on the window (8, 16 or 30) over which the O(W) loops are unrolled: their operands are
 // loaded first, all in flight, and slots at or past |J_n| take a zero coefficient (the rings start at
 // zero, so every product is finite).
 template <int WM>
@@ -676,7 +680,7 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
     extern __shared__ __align__(16) float sm[];
     const TrainBwdArgs a = for_instance(a0, blockIdx.y);
     const int lane = threadIdx.x & 31, team = threadIdx.x / kTeamThreads, tl = threadIdx.x % kTeamThreads;
-    const int role = tl >> 5;  // 0: window warp, 1: row warp, 2: filter warp
+    const int role = tl >> 5;  // 0: window warp, 1: row warp, 2: filter warp, 3: staging warp
     const int k = blockIdx.x * kTeamUsers + team;
     const int M = a.M, K = a.K, W = a.W, D = a.D, P = a.P, S = 2 * P, L2 = 2 * M;
     const int RB = bwd_ring(W), RM = RB - 1;  // sample j sits in ring slot j & RM
@@ -684,7 +688,7 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
     float *nrm = sm, *rk = nrm + S4;  // ||x_j||^2 and 1 / kappa_jj, shared by the users
     float *gam = rk + S4 + team * bwd_team_floats(S, W, L2);
     float *ca = gam + S4, *cb = ca + 32, *kg = cb + 32, *kd = kg + RB * RB, *kl = kd + RB * RB, *xw = kl + RB * RB;
-    float *py = xw + RB * L2, *pd = py + RB, *pw = pd + RB, *pb = pw + RB, *w = pb + RB, *sums = w + L2;
+    float *py = xw + RB * L2, *pd = py + RB, *pw = pd + RB, *pb = pw + RB, *w = pb + RB, *sums = w + L2, *zero4 = sums + 4;
     constexpr int kRing = kAhead + 1;
     static_assert((kRing & (kRing - 1)) == 0, "ring slots by mask");
     float *rows = gam + bwd_team_rings(S, W, L2), *bands = rows + kRing * kRowSlot, *tapes = bands + kRing * kBandSlot;
@@ -721,13 +725,11 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
             kl[v] = l;
         }
     };
-    // w += sum_o ca_o x_{jlo+o}, component by component in slot order
-    auto filter_update = [&](int jlo, int nJ) {
+    // w += sum_o ca_o x_{jlo+o}, component by component in slot order (ca is zero past the window)
+    auto filter_update = [&](int jlo) {
         float c[WM];
 #pragma unroll
         for (int o = 0; o < WM; ++o) c[o] = ca[o];
-#pragma unroll
-        for (int o = 0; o < WM; ++o) c[o] = o < nJ ? c[o] : 0.f;
         for (int m = lane; m < L2; m += 32) {
             float x[WM], acc = w[m];
 #pragma unroll
@@ -746,51 +748,57 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
     __syncthreads();  // the only block barrier: nrm and rk are shared by the users
     if (k >= K) return;
     auto team_sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(kTeamThreads) : "memory"); };
-    for (int i = tl; i < S4 + 64 + 3 * RB * RB + RB * L2 + 4 * RB; i += kTeamThreads) gam[i] = 0.f;  // and every ring
+    for (int i = tl; i < bwd_team_floats(S, W, L2); i += kTeamThreads) gam[i] = 0.f;  // and every ring
     for (int m = tl; m < M; m += kTeamThreads) {
         const float2 c = a.clin0 ? a.clin0[m * K + k] : make_float2(0.f, 0.f);
         w[m] = c.x;
         w[M + m] = c.y;
     }
     if (a.mode & 1) {
-        // what arrival j needs: its rows (row warp), its band, components and target (filter warp)
-        auto fetch_row = [&](int j) {
-            if (j < S)
+        // what arrival j needs: its rows, its band, components and target
+        auto stage_issue = [&](int j) {
+            if (j < S) {
+                float *slot = band_slot(j);
                 row_copy(row_slot(j), a.gtab + (size_t)j * a.Sp, a.gdtab + (size_t)j * a.Sp, first_centre(j), j, lane);
+                band_copy(slot, a, S, W, j, j - W, lane);
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (32 * c < L2) x_copy(slot, j, lane + 32 * c);
+                if (lane == 0) cp4(slot + 224, reinterpret_cast<const float *>(a.sym + (size_t)(j >> 1) * K + k) + (j & 1), true);
+            }
             cp_commit();
         };
-        auto fetch_arrival = [&](int j) {
-            float *slot = band_slot(j);
-            band_copy(slot, a, S, W, j, j - W, lane);
+        auto stage_finish = [&](int j) {  // landed: band and components into the window rings
+            cp_wait_oldest();
+            if (j < S) {
+                const float *slot = band_slot(j);
+                band_store(slot, j, j - W);
 #pragma unroll
-            for (int c = 0; c < 4; ++c)
-                if (32 * c < L2) x_copy(slot, j, lane + 32 * c);
-            if (lane == 0)
-                cp4(slot + 224, reinterpret_cast<const float *>(a.sym + (j < S ? (size_t)(j >> 1) * K + k : 0)) + (j & 1), j < S);
-            cp_commit();
+                for (int c = 0; c < 4; ++c) {
+                    const int m = lane + 32 * c;
+                    if (m < L2) xw[(j & RM) * L2 + m] = xsign(j, m, slot[96 + m]);
+                }
+                if (lane == 0) pb[j & RM] = slot[224];
+            }
         };
         team_sync();
-        if (role == 2) {
-            for (int j = 0; j < kAhead; ++j) fetch_arrival(j);
-            cp_wait_oldest();
-            const float *slot = band_slot(0);
-            band_store(slot, 0, -W);
-            float ws = 0.f;
-            for (int m = lane; m < L2; m += 32) {
-                const float x = xsign(0, m, slot[96 + m]);
-                xw[m] = x;
-                ws = fmaf(w[m], x, ws);
+        if (role == 3) {
+            for (int j = 0; j < kAhead; ++j) stage_issue(j);
+            for (int j = 0; j < 2; ++j) {
+                stage_finish(j);
+                stage_issue(j + kAhead);
             }
+        }
+        team_sync();
+        if (role == 2) {  // sample 0 arrives with no live centre
+            float ws = 0.f;
+            for (int m = lane; m < L2; m += 32) ws = fmaf(w[m], xw[m], ws);
             ws = warp_sum(ws);
             if (lane == 0) {
-                pb[0] = slot[224];
                 py[0] = 0.f;
                 pd[0] = 0.f;
                 pw[0] = ws;
             }
-            fetch_arrival(kAhead);
-        } else if (role == 1) {
-            for (int j = 1; j <= kAhead; ++j) fetch_row(j);
         }
         team_sync();
 
@@ -817,27 +825,28 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
                 }
             } else if (role == 1) {
                 if (jn < S) {
-                    cp_wait_oldest();
                     const float *pg = row_slot(jn) + 4 * lane, *pdv = pg + 128 * kPfV;  // this lane's entries
                     const int lo = first_centre(jn), lo4 = lo & ~3;
-                    const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
                     float4 gm[kPfV], gv[kPfV], dv[kPfV];
 #pragma unroll
                     for (int q = 0; q < kPfV; ++q) {
-                        const int i0 = lo4 + 4 * (lane + 32 * q);
-                        const bool in = i0 < jn;
-                        gm[q] = in ? *reinterpret_cast<const float4 *>(gam + i0) : z4;
-                        gv[q] = in ? *reinterpret_cast<const float4 *>(pg + 128 * q) : z4;
-                        dv[q] = in ? *reinterpret_cast<const float4 *>(pdv + 128 * q) : z4;
+                        if (lo4 + 128 * q < jn) {  // (an entry at or past jn meets a zero coefficient)
+                            const int i0 = lo4 + 4 * (lane + 32 * q);
+                            gm[q] = *reinterpret_cast<const float4 *>(i0 < jn ? gam + i0 : zero4);
+                            gv[q] = *reinterpret_cast<const float4 *>(pg + 128 * q);
+                            dv[q] = *reinterpret_cast<const float4 *>(pdv + 128 * q);
+                        }
                     }
                     float y2[2] = {0.f, 0.f}, d2[2] = {0.f, 0.f};  // two chains of sums
                     if (lo == 0) {  // nothing evicted yet: gamma is zero from jn on (padding included)
 #pragma unroll
                         for (int q = 0; q < kPfV; ++q) {
-                            y2[0] = fmaf(gm[q].x, gv[q].x, fmaf(gm[q].z, gv[q].z, y2[0]));
-                            y2[1] = fmaf(gm[q].y, gv[q].y, fmaf(gm[q].w, gv[q].w, y2[1]));
-                            d2[0] = fmaf(gm[q].x, dv[q].x, fmaf(gm[q].z, dv[q].z, d2[0]));
-                            d2[1] = fmaf(gm[q].y, dv[q].y, fmaf(gm[q].w, dv[q].w, d2[1]));
+                            if (128 * q < jn) {
+                                y2[0] = fmaf(gm[q].x, gv[q].x, fmaf(gm[q].z, gv[q].z, y2[0]));
+                                y2[1] = fmaf(gm[q].y, gv[q].y, fmaf(gm[q].w, gv[q].w, y2[1]));
+                                d2[0] = fmaf(gm[q].x, dv[q].x, fmaf(gm[q].z, dv[q].z, d2[0]));
+                                d2[1] = fmaf(gm[q].y, dv[q].y, fmaf(gm[q].w, dv[q].w, d2[1]));
+                            }
                         }
                     } else {
 #pragma unroll
@@ -863,33 +872,29 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
                         sums[1] = ds;
                     }
                 }
-            } else if (jn < S) {
-                cp_wait_oldest();
-                const float *slot = band_slot(jn);
-                band_store(slot, jn, jn - W);
-                float ws = 0.f;
+            } else if (role == 2) {
+                if (jn < S) {
+                    float ws = 0.f;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const int m = lane + 32 * c;
-                    if (m < L2) {
-                        const float x = xsign(jn, m, slot[96 + m]);
-                        xw[(jn & RM) * L2 + m] = x;
-                        ws = fmaf(w[m], x, ws);
+                    for (int c = 0; c < 4; ++c) {
+                        const int m = lane + 32 * c;
+                        if (m < L2) ws = fmaf(w[m], xw[(jn & RM) * L2 + m], ws);
                     }
+                    ws = warp_sum(ws);
+                    if (lane == 0) sums[2] = ws;
                 }
-                ws = warp_sum(ws);
-                if (lane == 0) sums[2] = ws;
+            } else {
+                stage_finish(jn + 1);
             }
             team_sync();
             // phase 2, Eq. apsm: coefficients, linear part, carried predictions of J_{n+1} (2D = W + 1: the
             // oldest centre of J_n leaves before step n+1)
             if (role == 1) {
                 if (lane < nJ) gam[jlo + lane] = cb[lane];
-                if (jn < S) fetch_row(jn + kAhead);
             } else if (role == 2) {
-                if (lane == 0 && jn < S) pb[jn & RM] = band_slot(jn)[224];
-                filter_update(jlo, nJ);
-                if (jn < S) fetch_arrival(jn + kAhead);
+                filter_update(jlo);
+            } else if (role == 3) {
+                stage_issue(jn + 1 + kAhead);
             } else {
                 const int t_lo = max(0, n - W + 2), n_t = jn < S ? jn - t_lo + 1 : 0;
                 const int e_lo = first_centre(n), e_hi = jn < S ? first_centre(jn) : e_lo;
@@ -907,9 +912,9 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
                     float ay = j == jn ? sums[0] : py[r], ad = j == jn ? sums[1] : pd[r], aw = j == jn ? sums[2] : pw[r];
                     const int o_lo = j == jn ? max(0, e_hi - jlo) : 0;
 #pragma unroll
-                    for (int o = 0; o < WM; ++o) {
-                        const float cl = o < nJ ? c[o] : 0.f, cg = o >= o_lo ? cl : 0.f;
-                        aw = fmaf(cl, vl[o], aw);
+                    for (int o = 0; o < WM; ++o) {  // (ca is zero past the window)
+                        const float cg = o >= o_lo ? c[o] : 0.f;
+                        aw = fmaf(c[o], vl[o], aw);
                         ay = fmaf(cg, vg[o], ay);
                         ad = fmaf(cg, vd[o], ad);
                     }
@@ -965,29 +970,42 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
         const int e = evict_step(n - W);
         return e > n + 1 ? min(e, S) : n - W + 2;
     };
-    // what step n of the sweep needs: its tape, the final adjoint of its entrant n - W and that entrant's
-    // row (row warp), the entrant's band and components (filter warp)
-    auto fetch_step = [&](int n) {
-        float *slot = tape_slot(n);
-        const int j = n - W;
-        if (n >= 0 && lane < min(n + 1, W)) {
-            const float *f = reinterpret_cast<const float *>(tape + (size_t)n * W + lane);
+    // what step n of the sweep needs: its tape, and its entrant n - W's final adjoint, row, band and
+    // components
+    auto stage_issue = [&](int n) {
+        if (n >= 0) {
+            float *slot = tape_slot(n);
+            const int j = n - W;
+            if (lane < min(n + 1, W)) {
+                const float *f = reinterpret_cast<const float *>(tape + (size_t)n * W + lane);
 #pragma unroll
-            for (int i = 0; i < 3; ++i) cp8(slot + 6 * lane + 2 * i, f + 2 * i);
+                for (int i = 0; i < 3; ++i) cp8(slot + 6 * lane + 2 * i, f + 2 * i);
+            }
+            if (j >= 0) {
+                bool ok;
+                const float *fs = final_src(j, ok);
+                if (lane == 0) cp4(slot + 192, fs, ok);
+                row_copy(row_slot(n), a.gtab + (size_t)j * a.Sp, nullptr, j + 2, pull_hi(n), lane);
+                band_copy(band_slot(n), a, S, W, j, j, lane);
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (32 * c < L2) x_copy(band_slot(n), j, lane + 32 * c);
+            }
         }
-        bool ok;
-        const float *fs = final_src(j, ok);
-        if (lane == 0) cp4(slot + 192, fs, ok);
-        if (j >= 0) row_copy(row_slot(n), a.gtab + (size_t)j * a.Sp, nullptr, j + 2, pull_hi(n), lane);
         cp_commit();
     };
-    auto fetch_entrant = [&](int n) {
-        float *slot = band_slot(n);
-        band_copy(slot, a, S, W, n - W, n - W, lane);
+    auto stage_finish = [&](int n) {
+        cp_wait_oldest();
+        const int j = n - W;
+        if (j >= 0) {
+            const float *slot = band_slot(n);
+            band_store(slot, j, j);
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-            if (32 * c < L2) x_copy(slot, n - W, lane + 32 * c);
-        cp_commit();
+            for (int c = 0; c < 4; ++c) {
+                const int m = lane + 32 * c;
+                if (m < L2) xw[(j & RM) * L2 + m] = xsign(j, m, slot[96 + m]);
+            }
+        }
     };
     team_sync();
     if (role == 0) {
@@ -998,12 +1016,12 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
             const float *fs = final_src(j, ok);
             py[j & RM] = d + (ok ? __ldg(fs) : 0.f);
         }
-    } else if (role == 1) {
-        for (int i = 0; i < kAhead; ++i) fetch_step(S - 1 - i);
-        cp_wait_oldest();
-    } else {
-        for (int i = 0; i < kAhead; ++i) fetch_entrant(S - 1 - i);
+    } else if (role == 3) {
+        for (int i = 0; i < kAhead; ++i) stage_issue(S - 1 - i);
+        stage_finish(S - 1);
+        stage_issue(S - 1 - kAhead);
     }
+    if (lane >= W && role == 0) ca[lane] = cb[lane] = 0.f;  // (and past |J_n| below: zero coefficients)
     team_sync();
     float sig_bar = 0.f, mu_bar = 0.f, eps_bar = 0.f, wl_bar = 0.f;  // lane o: window slot o's terms
     for (int n = S - 1; n >= 0; --n) {
@@ -1035,6 +1053,8 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
                 }
                 ca[lane] = cwo;
                 cb[lane] = cgo;
+            } else {
+                ca[lane] = cb[lane] = 0.f;
             }
         } else if (role == 1) {
             if (((n + 1) & 1) == 0 && n + 1 <= S - 1 && ((n + 1) >> 1) >= D && lane < W - 1) {
@@ -1048,21 +1068,23 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
                 const float *sv = snap + (size_t)((e >> 1) - D) * W;
                 const float *grow = a.gtab + (size_t)je * a.Sp;
                 const int lo4 = lo & ~3;
-                const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
                 float4 rm[kPfV], gv[kPfV];
 #pragma unroll
                 for (int q = 0; q < kPfV; ++q) {
-                    const int i0 = lo4 + 4 * (lane + 32 * q);
-                    const bool in = i0 < hi;
-                    rm[q] = in ? *reinterpret_cast<const float4 *>(gam + i0) : z4;
-                    gv[q] = in ? *reinterpret_cast<const float4 *>(pg + 128 * q) : z4;
+                    if (lo4 + 128 * q < hi) {
+                        const int i0 = lo4 + 4 * (lane + 32 * q);
+                        rm[q] = *reinterpret_cast<const float4 *>(i0 < hi ? gam + i0 : zero4);
+                        gv[q] = *reinterpret_cast<const float4 *>(pg + 128 * q);
+                    }
                 }
                 float g2[2] = {0.f, 0.f};
                 if (hi == S && s_lo >= S) {  // no eviction after the entrant: R is zero below lo and past S
 #pragma unroll
                     for (int q = 0; q < kPfV; ++q) {
-                        g2[0] = fmaf(rm[q].x, gv[q].x, fmaf(rm[q].z, gv[q].z, g2[0]));
-                        g2[1] = fmaf(rm[q].y, gv[q].y, fmaf(rm[q].w, gv[q].w, g2[1]));
+                        if (lo4 + 128 * q < hi) {
+                            g2[0] = fmaf(rm[q].x, gv[q].x, fmaf(rm[q].z, gv[q].z, g2[0]));
+                            g2[1] = fmaf(rm[q].y, gv[q].y, fmaf(rm[q].w, gv[q].w, g2[1]));
+                        }
                     }
                 } else {
 #pragma unroll
@@ -1082,32 +1104,28 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
                 const float gs = warp_sum(g2[0] + g2[1]);
                 if (lane == 0) sums[0] = gs;
             }
-        } else if (je >= 0) {
-            cp_wait_oldest();
-            const float *slot = band_slot(n);
-            band_store(slot, je, je);
-            float ls = 0.f;
+        } else if (role == 2) {
+            if (je >= 0) {
+                float ls = 0.f;
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int m = lane + 32 * c;
-                if (m < L2) {
-                    const float x = xsign(je, m, slot[96 + m]);
-                    xw[(je & RM) * L2 + m] = x;
-                    ls = fmaf(w[m], x, ls);
+                for (int c = 0; c < 4; ++c) {
+                    const int m = lane + 32 * c;
+                    if (m < L2) ls = fmaf(w[m], xw[(je & RM) * L2 + m], ls);
                 }
+                ls = warp_sum(ls);
+                if (lane == 0) sums[1] = ls;
             }
-            ls = warp_sum(ls);
-            if (lane == 0) sums[1] = ls;
+        } else {
+            stage_finish(n - 1);
         }
         team_sync();
         // phase 2: the adjoint of S_n
         if (role == 1) {
             if (lane < nJ) gam[jlo + lane] += cb[lane];
-            fetch_step(n - kAhead);
-            cp_wait_oldest();  // step n - 1's copies, for the window warp too
         } else if (role == 2) {
-            filter_update(jlo, nJ);
-            fetch_entrant(n - kAhead);
+            filter_update(jlo);
+        } else if (role == 3) {
+            stage_issue(n - 1 - kAhead);
         } else {
             const int t_lo = max(0, n - W), n_t = n - t_lo;
             if (lane < n_t) {
@@ -1125,8 +1143,8 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
                 float acc = j == je ? fa_je + sums[0] + sums[1] : py[r];
 #pragma unroll
                 for (int o = 0; o < WM; ++o) {
-                    acc = fmaf(o < nJ ? c[o] : 0.f, vl[o], acc);
-                    acc = fmaf(o < nJ && alive ? b[o] : 0.f, vg[o], acc);
+                    acc = fmaf(c[o], vl[o], acc);
+                    acc = fmaf(alive ? b[o] : 0.f, vg[o], acc);
                 }
                 py[r] = acc;
             }
@@ -1222,11 +1240,11 @@ apsm_status train_bwd_run(const apsm_params *p, int n, const float *rx_pilot, co
     if (!workspace || workspace_bytes < b.total * (size_t)n) return APSM_ERR_WORKSPACE;
     if (reinterpret_cast<uintptr_t>(workspace) & 255) return APSM_ERR_INVALID_ARG;
     const size_t smem = train_bwd_smem(p->M, p->window, P);
-    // three warps per user when the window fits the lanes and the rings of a CTA's users its shared memory
+    // four warps per user when the window fits the lanes and the rings of a CTA's users its shared memory
     const size_t smem_w =
         sizeof(float) * (2 * (size_t)((2 * P + 3) & ~3) +
                          (size_t)std::min(p->K, kTeamUsers) * bwd_team_floats(2 * P, p->window, 2 * p->M));
-    const bool team_form = p->window < 32 && smem_w <= 227 * 1024;
+    const bool team_form = p->window <= 30 && smem_w <= 227 * 1024;
     if (!team_form && smem > 227 * 1024) return APSM_ERR_UNSUPPORTED;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) {
@@ -1277,7 +1295,7 @@ apsm_status train_bwd_run(const apsm_params *p, int n, const float *rx_pilot, co
     if (mode & 1) train_bwd_tables_kernel<<<dim3(blocks, n), 256, 0, strm>>>(a);
     if (team_form) {
         auto kern = p->window <= 8 ? train_bwd_team_kernel<8>
-                    : p->window <= 16 ? train_bwd_team_kernel<16> : train_bwd_team_kernel<31>;
+                    : p->window <= 16 ? train_bwd_team_kernel<16> : train_bwd_team_kernel<30>;
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_w) != cudaSuccess)
             return APSM_ERR_CUDA;
         const int users = std::min(p->K, kTeamUsers);
