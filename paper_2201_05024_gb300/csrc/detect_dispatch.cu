@@ -46,6 +46,7 @@ TcBatchLauncher detect_tc_batch_launcher_m16(int kb, int *ctas_per_sm);
 TcBatchLauncher detect_tc_batch_launcher_m32(int kb, int *ctas_per_sm);
 TcBatchLauncher detect_tc_batch_launcher_m64(int kb, int *ctas_per_sm);
 
+H3Launcher detect_h3_launcher_m16(int kb);
 H3Launcher detect_h3_launcher_m32(int kb);
 H3Launcher detect_h3_launcher_m64(int kb);
 
@@ -128,7 +129,12 @@ size_t detect_tcc_workspace(int M, int K, int D) {
 // FP32 detection with the Gram as three FP16 products; nullptr if none.
 H3Launcher detect_h3_launcher(int M, int K) {
     const int kb = tc_user_bucket(K);
-    return M == 32 ? detect_h3_launcher_m32(kb) : (M == 64 ? detect_h3_launcher_m64(kb) : nullptr);
+    switch (M) {
+        case 16: return detect_h3_launcher_m16(kb);
+        case 32: return detect_h3_launcher_m32(kb);
+        case 64: return detect_h3_launcher_m64(kb);
+        default: return nullptr;
+    }
 }
 
 // Batched persistent detection (FP32 accuracy) for class (M, user bucket of K); nullptr if none.

@@ -36,7 +36,10 @@
 // the MMAs 3000, beside it; ncu: FMA pipe 66 % active).
 // Measured (FP32, 64 antennas, 16 users, 4096 entries, 100003 vectors): 8025 us on the FMA engine
 // (323 FMA per pair), 1288 us here.  32 antennas, 11 users, 1500 entries, 10001 vectors: 110 us in the
-// TF32 x3 converter form (79 CTAs of 128 queries for 152 SMs), 64 us here.
+// TF32 x3 converter form (79 CTAs of 128 queries for 152 SMs), 64 us here.  16 antennas, 6 users, 1024
+// entries: an entry tile takes 3340 cycles (1800 of FMAs) against 3950 per 32 entries and 256 queries in
+// the TMA-staged TF32 x3 form; resting the converters, dropping the exponentials or the coefficient reads
+// saves 5, 5 and 10 %, four epilogue groups instead of two nothing: warps wait for the FMA pipe.
 #pragma once
 
 #include <algorithm>
@@ -52,6 +55,13 @@ constexpr int kH3Epi = 256;       // epilogue threads
 constexpr int kH3Conv = 96;       // converter threads
 constexpr int kH3Threads = kH3Epi + kH3Conv + 32;
 constexpr int kH3MaxSplit = 8;    // CTAs per cluster
+// 16 antennas: dictionaries up to here keep the TMA-staged form and with it the last bit of their
+// outputs, which the gradient of a training-sized dictionary is taken of in FP64 (results compared at
+// 1e-9).  Above, this form is the faster one at every size measured (us of device time, TMA-staged form
+// and this): 6 users, 260 entries: 64 vectors 16.2 and 10.6, 16384: 34.8 and 17.1, 100000: 84.6 and 70.9;
+// 1024 entries: 64 vectors 25.7 and 13.8, 4000: 33.1 and 19.0, 65536: 138.6 and 128.0.  (2 users, 1024
+// entries, 65536 vectors: 93.1 and 84.5; 16 users: 258.8 and 236.9.)
+constexpr int kH3MinEntries16 = 256;
 constexpr int kH3Devices = 16;    // devices whose cluster counts are kept
 
 template <int M, int KB>
@@ -418,11 +428,12 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const TcArgs a
         // ================= epilogue =================
         // ---- this warp's 32 query rows as scaled hi and lo copies, by pieces of eight antennas (eight
         // consecutive lanes write eight consecutive rows of one k-column)
+        constexpr int kBatch = P8 < 4 ? P8 : 4;
 #pragma unroll 1
-        for (int i0 = 0; i0 < 32 * P8; i0 += 128) {  // sixteen loads in flight per lane
-            float4 va[4][4];
+        for (int i0 = 0; i0 < 32 * P8; i0 += 32 * kBatch) {  // up to sixteen loads in flight per lane
+            float4 va[kBatch][4];
 #pragma unroll
-            for (int n = 0; n < 4; ++n) {
+            for (int n = 0; n < kBatch; ++n) {
                 const int i = i0 + 32 * n + lane, r = 32 * warp + ((i & 7) | (i / (8 * P8) << 3)), p = (i >> 3) % P8;
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
@@ -430,7 +441,7 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const TcArgs a
                                             : make_float4(0.f, 0.f, 0.f, 0.f);
             }
 #pragma unroll
-            for (int n = 0; n < 4; ++n) {
+            for (int n = 0; n < kBatch; ++n) {
                 const int i = i0 + 32 * n + lane, r = 32 * warp + ((i & 7) | (i / (8 * P8) << 3)), p = (i >> 3) % P8;
                 float inv;
                 const float s = h3_scale(s_nq[r], inv);
