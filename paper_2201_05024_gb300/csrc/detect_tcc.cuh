@@ -30,8 +30,13 @@
 namespace apsm {
 
 constexpr int kTccChunk = 16;     // entries per exponential chunk
-constexpr int kTccXBuf = 2;       // exponential buffers
-constexpr int kTccThreads = 192;
+constexpr int kTccGroups = 4;     // epilogue groups of 128 threads, one chunk of a 64-entry tile each
+constexpr int kTccXBuf = kTccGroups;  // exponential buffers, one per group
+constexpr int kTccAcc = 3;        // Gram accumulators
+constexpr int kTccGStages = 3;    // coefficient stages: a tile's are free only after its last GEMM
+constexpr int kTccEpi = 128 * kTccGroups;
+constexpr int kTccThreads = kTccEpi + 64;
+static_assert(kTcEntries / kTccChunk % kTccGroups == 0, "every group the same chunks of each tile");
 
 // Shared-memory matrix descriptor, K-major, no swizzle, with an explicit leading byte offset
 // (bytes between k-adjacent core matrices) and stride byte offset (between 8-row groups).
@@ -44,6 +49,23 @@ __device__ __forceinline__ uint64_t umma_sdesc_lbo(uint32_t addr, uint32_t lbo, 
     return d;
 }
 
+// 32 accumulator columns of this warp's 32 lanes.
+__device__ __forceinline__ void tcc_tmem_ld32(uint32_t taddr, float (&v)[32]) {
+    uint32_t r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr)
+        : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+}
+
 template <int M, int KB>
 struct TccSmem {
     using Sh = TcShape<M, kHalf>;
@@ -53,14 +75,17 @@ struct TccSmem {
     static constexpr int kXBytes = kTcRows * KX * 2;              // one exponential buffer
     static constexpr int kGBytes = NY * 3 * E * 2;                // one copy of G for a tile
     // a packed tile (the same layout in the workspace and in a shared-memory stage)
-    static constexpr int kOG = Sh::kBytesB;                       // G hi, then G lo
+    static constexpr int kOG = Sh::kBytesB;                       // G, 2 NY rows: hi, then lo
     static constexpr int kOH = kOG + 2 * kGBytes;                 // -k2 n_t [E]
     static constexpr int kTile = round_up(kOH + E * 4, 1024);
     static constexpr int kA = 0;
-    static constexpr int kS = round_up(Sh::kBytesA, 1024);        // 2 tile stages
-    static constexpr int kX = kS + 2 * kTile;                     // exponential buffers
+    static constexpr int kS = round_up(Sh::kBytesA, 1024);        // 2 stages of the Gram operand
+    static constexpr int kGBytesAll = 2 * kGBytes + E * 4;        // G and norms of a tile
+    static constexpr int kGPart = round_up(kGBytesAll, 128);      // kTccGStages stages of them
+    static constexpr int kG = kS + 2 * kOG;
+    static constexpr int kX = kG + kTccGStages * kGPart;          // exponential buffers
     static constexpr int kBar = kX + kTccXBuf * kXBytes;          // mbarriers
-    static constexpr int kTmem = kBar + 16 * 8;
+    static constexpr int kTmem = kBar + 24 * 8;
     static constexpr int kBytes = kTmem + 16;
     static_assert(kBytes <= 227 * 1024, "one CTA per SM");
     static_assert(Sh::kBytesB % 16 == 0 && kGBytes % 16 == 0, "bulk-copy granules");
@@ -142,9 +167,9 @@ __global__ void __launch_bounds__(128) tcc_pack_kernel(const TcArgs a, unsigned 
             hp[i] = *reinterpret_cast<const uint32_t *>(&h2);
             lp[i] = *reinterpret_cast<const uint32_t *>(&l2);
         }
-        const int off = L::kOG + (kc * NY + n) * 16;
+        const int off = L::kOG + (kc * 2 * NY + n) * 16;  // rows n (hi) and NY + n (lo)
         *reinterpret_cast<uint4 *>(blk + off) = hi;
-        *reinterpret_cast<uint4 *>(blk + L::kGBytes + off) = lo;
+        *reinterpret_cast<uint4 *>(blk + off + NY * 16) = lo;
     }
 }
 
@@ -158,12 +183,18 @@ __global__ void __launch_bounds__(kTccThreads, 1) detect_tcc_kernel(const TcArgs
     extern __shared__ __align__(1024) unsigned char smem[];
     unsigned char *sA = smem + L::kA;
     unsigned char *sS = smem + L::kS;
+    unsigned char *sG = smem + L::kG;
     unsigned char *sX = smem + L::kX;
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L::kBar);
-    uint64_t *s_full = bars, *mma_done = bars + 2, *epi_done = bars + 4, *g_free = bars + 6, *x_full = bars + 8,
-             *x_free = bars + 8 + kTccXBuf;
+    uint64_t *b_full = bars, *mma_done = bars + 2, *epi_done = mma_done + kTccAcc, *x_full = epi_done + kTccAcc,
+             *x_free = x_full + kTccXBuf, *g_full = x_free + kTccXBuf, *y_done = g_full + kTccGStages;
+    static_assert(2 + 2 * kTccAcc + 2 * kTccXBuf + kTccGStages + 1 <= 24, "barriers");
     uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + L::kTmem);
-    constexpr uint32_t kCols = 512;  // Gram accumulators at [0, 2 NB), Y at [2 NB, 2 NB + NY)
+    __shared__ float s_nq[kTccEpi];
+    __shared__ int s_some;  // some pair of the CTA went to the direct differences
+    constexpr uint32_t kYCol = kTccAcc * NB;  // Gram accumulators below it, Y at it: 2 NY columns, hi and lo
+    constexpr uint32_t kCols = 512;
+    static_assert(kYCol + 2 * NY <= kCols, "TMEM columns");
 
     const int tid = threadIdx.x, warp = tid >> 5;
     const int q0 = blockIdx.x * kTcRows;
@@ -180,12 +211,14 @@ __global__ void __launch_bounds__(kTccThreads, 1) detect_tcc_kernel(const TcArgs
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (tid == 0) {
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(&s_full[i], 1);
+        s_some = 0;
+        for (int i = 0; i < 2; ++i) mbar_init(&b_full[i], 1);
+        for (int i = 0; i < kTccAcc; ++i) {
             mbar_init(&mma_done[i], 1);
-            mbar_init(&epi_done[i], kTcRows);
-            mbar_init(&g_free[i], 1);
+            mbar_init(&epi_done[i], kTccEpi);
         }
+        for (int i = 0; i < kTccGStages; ++i) mbar_init(&g_full[i], 1);
+        mbar_init(y_done, 1);
         for (int i = 0; i < kTccXBuf; ++i) {
             mbar_init(&x_full[i], kTcRows);
             mbar_init(&x_free[i], 1);
@@ -194,148 +227,174 @@ __global__ void __launch_bounds__(kTccThreads, 1) detect_tcc_kernel(const TcArgs
     }
     // the first two tiles' copies go out before the query operand is built
     __syncthreads();
-    if (tid == 128) {
-        for (int t = 0; t < 2 && t < n_tiles; ++t) {
-            mbar_arrive_expect_tx(&s_full[t], (uint32_t)L::kTile);
-            bulk_g2s(sS + t * L::kTile, packed + (size_t)t * L::kTile, (uint32_t)L::kTile, &s_full[t]);
+    auto copy_b = [&](int t) {  // tile t's Gram operand; its coefficients and norms
+        mbar_arrive_expect_tx(&b_full[t & 1], (uint32_t)L::kOG);
+        bulk_g2s(sS + (t & 1) * L::kOG, packed + (size_t)t * L::kTile, (uint32_t)L::kOG, &b_full[t & 1]);
+    };
+    auto copy_g = [&](int t) {
+        const int sg = t % kTccGStages;
+        mbar_arrive_expect_tx(&g_full[sg], (uint32_t)L::kGBytesAll);
+        bulk_g2s(sG + sg * L::kGPart, packed + (size_t)t * L::kTile + L::kOG, (uint32_t)L::kGBytesAll, &g_full[sg]);
+    };
+    if (tid == kTccEpi) {
+        for (int t = 0; t < kTccGStages && t < n_tiles; ++t) {
+            if (t < 2) copy_b(t);
+            copy_g(t);
         }
     }
     // ---- the query operand (as detect_tc.cuh) -------------------------------------------------
-    float nq = 0.f;
-    if (warp < 4) {
-        const int s = q0 + tid;
+    // (a group takes every kTccGroups-th piece of eight antennas of its rows)
+    static_assert(tc_core_rows<M, kHalf>(), "whole core rows");
+    if (warp < 4 * kTccGroups) {
+        constexpr int C = Sh::kCoreK;
+        const int row = tid & (kTcRows - 1), s = q0 + row;
         const float2 *rq = a.rx + (size_t)s * M;
-        if constexpr (tc_core_rows<M, kHalf>()) {
-            constexpr int C = Sh::kCoreK;
-#pragma unroll 2
-            for (int p = 0; p < M / C; ++p) {
-                float re[C], im[C];
-                if (s < a.N) {
-                    const float4 *src = reinterpret_cast<const float4 *>(rq + p * C);
+        float np = 0.f;
 #pragma unroll
-                    for (int q = 0; q < C / 2; ++q) {
-                        const float4 v = __ldg(src + q);
-                        re[2 * q] = v.x; im[2 * q] = v.y; re[2 * q + 1] = v.z; im[2 * q + 1] = v.w;
-                    }
-                } else {
+        for (int p = tid / kTcRows; p < M / C; p += kTccGroups) {
+            float re[C], im[C];
+            if (s < a.N) {
+                const float4 *src = reinterpret_cast<const float4 *>(rq + p * C);
 #pragma unroll
-                    for (int c = 0; c < C; ++c) re[c] = im[c] = 0.f;
+                for (int q = 0; q < C / 2; ++q) {
+                    const float4 v = __ldg(src + q);
+                    re[2 * q] = v.x; im[2 * q] = v.y; re[2 * q + 1] = v.z; im[2 * q + 1] = v.w;
                 }
+            } else {
 #pragma unroll
-                for (int c = 0; c < C; ++c) {
-                    nq = fmaf(re[c], re[c], fmaf(im[c], im[c], nq));
-                    re[c] *= g2;
-                    im[c] *= g2;
-                }
-                put_core<kHalf, C>(sA, Sh::kBytesA, Sh::off(tid, p * C), re, a.half_fmt);
-                put_core<kHalf, C>(sA, Sh::kBytesA, Sh::off(tid, M + p * C), im, a.half_fmt);
+                for (int c = 0; c < C; ++c) re[c] = im[c] = 0.f;
             }
-        } else {
-            for (int m = 0; m < M; ++m) {
-                const float2 v = s < a.N ? __ldg(rq + m) : make_float2(0.f, 0.f);
-                nq = fmaf(v.x, v.x, fmaf(v.y, v.y, nq));
-                put_elem<kHalf>(sA, Sh::kBytesA, Sh::off(tid, m), g2 * v.x, a.half_fmt);
-                put_elem<kHalf>(sA, Sh::kBytesA, Sh::off(tid, M + m), g2 * v.y, a.half_fmt);
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                np = fmaf(re[c], re[c], fmaf(im[c], im[c], np));
+                re[c] *= g2;
+                im[c] *= g2;
             }
-            for (int k = 2 * M; k < Sh::KD; ++k) put_elem<kHalf>(sA, Sh::kBytesA, Sh::off(tid, k), 0.f, a.half_fmt);
+            put_core<kHalf, C>(sA, Sh::kBytesA, Sh::off(row, p * C), re, a.half_fmt);
+            put_core<kHalf, C>(sA, Sh::kBytesA, Sh::off(row, M + p * C), im, a.half_fmt);
         }
+        s_nq[tid] = np;
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     tc_fence_before();
-    const bool cta_in_range = __syncthreads_and(warp >= 4 || a.k2 * nq <= kFactorLimit);
+    __syncthreads();
+    float nq = 0.f;  // this row's squared norm
+    if (warp < 4 * kTccGroups) {
+#pragma unroll
+        for (int i = 0; i < kTccGroups; ++i) nq += s_nq[i * kTcRows + (tid & (kTcRows - 1))];
+    }
+    const bool cta_in_range = __syncthreads_and(a.k2 * nq <= kFactorLimit);
     tc_fence_after();
     const uint32_t tmem = *s_tmem;
     bool ok = true;
 
-    if (warp == 4) {
+    if (warp == 4 * kTccGroups) {
         // ================= tile copies and Gram MMAs (one thread) =================
-        if (tid == 128) {
+        if (tid == kTccEpi) {
             const uint32_t idesc = (1u << 4) | ((a.half_fmt ? 1u : 0u) << 7) | ((a.half_fmt ? 1u : 0u) << 10) |
                                    ((uint32_t)(NB >> 3) << 17) | ((uint32_t)(kTcRows >> 4) << 24);
-            const uint32_t a0 = smem_u32(sA);
+            const uint64_t ad = umma_sdesc(smem_u32(sA), Sh::SBO);
             int issued = min(2, n_tiles), committed = -1;
             for (int t = 0; t < n_tiles; ++t) {
-                const int st = t & 1;
-                // tile t has landed; the epilogue of tile t-2 freed TMEM stage st
-                if (!mbar_wait_bounded(&s_full[st], (t >> 1) & 1) ||
-                    (t >= 2 && !mbar_wait_sleepy(&epi_done[st], ((t - 2) >> 1) & 1))) {
+                const int sb = t & 1, st = t % kTccAcc;
+                // tile t's operand has landed; the epilogue of tile t - kTccAcc freed TMEM stage st
+                if (!mbar_wait_bounded(&b_full[sb], (t >> 1) & 1) ||
+                    (t >= kTccAcc && !mbar_wait_bounded(&epi_done[st], (t / kTccAcc - 1) & 1))) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
-                const uint32_t d = tmem + (uint32_t)(st * NB), b0 = smem_u32(sS + st * L::kTile);
+                const uint32_t d = tmem + (uint32_t)(st * NB);
+                const uint64_t bd = umma_sdesc(smem_u32(sS + sb * L::kOG), Sh::SBO);
 #pragma unroll
-                for (int s = 0; s < Sh::kSteps; ++s) {
-                    const uint64_t ah = umma_sdesc(a0 + s * 256, Sh::SBO), bh = umma_sdesc(b0 + s * 256, Sh::SBO);
-                    umma_f16(d, ah, bh, idesc, s > 0);
-                }
+                for (int s = 0; s < Sh::kSteps; ++s) umma_f16(d, ad + s * 16, bd + s * 16, idesc, s > 0);
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                                  smem_u32(&mma_done[st]))
                              : "memory");
                 committed = t;
-                // the stage of tile t-1 is free once its epilogue and its coefficient GEMMs are done
-                if (t >= 1 && t + 1 < n_tiles) {
-                    const int so = (t - 1) & 1;
-                    if (!mbar_wait_sleepy(&epi_done[so], ((t - 1) >> 1) & 1) ||
-                        !mbar_wait_sleepy(&g_free[so], ((t - 1) >> 1) & 1)) {
+                if (t + 2 < n_tiles) {  // its stage is free once the Gram has read it
+                    if (!mbar_wait_bounded(&mma_done[st], (t / kTccAcc) & 1)) {
                         ok = false;
                         break;
                     }
-                    mbar_arrive_expect_tx(&s_full[so], (uint32_t)L::kTile);
-                    bulk_g2s(sS + so * L::kTile, packed + (size_t)(t + 1) * L::kTile, (uint32_t)L::kTile, &s_full[so]);
-                    issued = t + 2;
+                    copy_b(t + 2);
+                    issued = t + 3;
                 }
             }
             // every copy and MMA issued here has landed before the CTA may exit
-            for (int t = max(0, issued - 2); t < issued; ++t) mbar_wait_sleepy(&s_full[t & 1], (t >> 1) & 1);
-            if (committed >= 0) mbar_wait_sleepy(&mma_done[committed & 1], (committed >> 1) & 1);
+            for (int t = max(0, issued - 2); t < issued; ++t) mbar_wait_sleepy(&b_full[t & 1], (t >> 1) & 1);
+            if (committed >= 0) mbar_wait_sleepy(&mma_done[committed % kTccAcc], (committed / kTccAcc) & 1);
         }
-    } else if (warp == 5) {
-        // ================= coefficient-GEMM issue (one thread) =================
-        if (tid == 160) {
-            const uint32_t coef_idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(NY >> 3) << 17) |
+    } else if (warp == 4 * kTccGroups + 1) {
+        // ================= coefficient copies and GEMM issue (one thread) =================
+        if (tid == kTccEpi + 32) {
+            const uint32_t coef_idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(2 * NY >> 3) << 17) |
                                         ((uint32_t)(kTcRows >> 4) << 24);
-            const uint32_t y = tmem + 2 * NB;
-            for (int g = 0; g < n_chunks; ++g) {
-                const int xb = g % kTccXBuf, t = g / kChunks, c = g % kChunks, st = t & 1;
-                if (!mbar_wait_bounded(&x_full[xb], (g / kTccXBuf) & 1)) {
+            const uint32_t y = tmem + kYCol;
+            const uint64_t xd0 = umma_sdesc_lbo(smem_u32(sX), kTcRows * 16, 128);
+            const uint64_t gd0 = umma_sdesc_lbo(smem_u32(sG), 2 * NY * 16, 128);
+            int issued = min(kTccGStages, n_tiles);
+            for (int t = 0; t < n_tiles && ok; ++t) {
+                const int sg = t % kTccGStages;
+                if (!mbar_wait_bounded(&g_full[sg], (t / kTccGStages) & 1)) {
                     ok = false;
                     break;
                 }
-                tc_fence_after();
-                // X chunk: [k-chunk of 8][128 rows][16 B]; G: [k-chunk of 8][NY rows][16 B], this
-                // chunk's k-chunks are 6c .. 6c + 5
-                const uint32_t x0 = smem_u32(sX + xb * L::kXBytes);
-                const uint32_t gh = smem_u32(sS + st * L::kTile + L::kOG) + c * 6 * NY * 16;
-                const uint32_t gl = gh + L::kGBytes;
 #pragma unroll
-                for (int ks = 0; ks < L::KX / 16; ++ks) {
-                    const uint64_t xd = umma_sdesc_lbo(x0 + ks * 2 * kTcRows * 16, kTcRows * 16, 128);
-                    const uint64_t hd = umma_sdesc_lbo(gh + ks * 2 * NY * 16, NY * 16, 128);
-                    const uint64_t ld = umma_sdesc_lbo(gl + ks * 2 * NY * 16, NY * 16, 128);
-                    umma_f16(y, xd, hd, coef_idesc, (g > 0 || ks > 0) ? 1u : 0u);
-                    umma_f16(y, xd, ld, coef_idesc, 1u);
-                }
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                                 smem_u32(&x_free[xb]))
-                             : "memory");
-                if (c == kChunks - 1)  // the tile's last reader of its G
+                for (int c = 0; c < kChunks; ++c) {
+                    const int g = t * kChunks + c, xb = g % kTccXBuf;
+                    if (!mbar_wait_bounded(&x_full[xb], (g / kTccXBuf) & 1)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    // X chunk: [k-chunk of 8][128 rows][16 B]; G: [k-chunk of 8][2 NY rows][16 B], this
+                    // chunk's k-chunks are 6c .. 6c + 5
+                    const uint64_t xd = xd0 + xb * (L::kXBytes >> 4);
+                    const uint64_t gd = gd0 + (sg * L::kGPart >> 4) + c * 6 * 2 * NY;
+#pragma unroll
+                    for (int ks = 0; ks < L::KX / 16; ++ks)
+                        umma_f16(y, xd + ks * 2 * kTcRows, gd + ks * 2 * 2 * NY, coef_idesc, (c > 0 || ks > 0 || t > 0) ? 1u : 0u);
                     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                                     smem_u32(&g_free[st]))
+                                     smem_u32(&x_free[xb]))
                                  : "memory");
+                    // the coefficient stage of tile t-1 is free once its last chunk's GEMM is done (whose
+                    // x_full also says that every epilogue thread has read the norms); by now it is
+                    if (c == kChunks - 2 && t >= 1 && t - 1 + kTccGStages < n_tiles) {
+                        const int gp = t * kChunks - 1;
+                        if (!mbar_wait_bounded(&x_free[gp % kTccXBuf], (gp / kTccXBuf) & 1)) {
+                            ok = false;
+                            break;
+                        }
+                        copy_g(t - 1 + kTccGStages);
+                        issued = t + kTccGStages;
+                    }
+                }
             }
+            // Y's own barrier (its one phase cannot be taken for another, as a group's wait for a chunk that
+            // is not its own could); reached on errors too, when the MMAs issued so far are done
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                             smem_u32(y_done))
+                         : "memory");
+            for (int t = max(0, issued - kTccGStages); t < issued; ++t)
+                mbar_wait_sleepy(&g_full[t % kTccGStages], (t / kTccGStages) & 1);
+            mbar_wait_sleepy(y_done, 0);
         }
-    } else if (warp < 4) {
+    } else {
         // ================= epilogue: exponentials into X, exact pairs in FP32 =================
+        const int grp = warp >> 2, row = tid & (kTcRows - 1);
         const float hq = cta_in_range ? 0.f : -a.k2 * nq;
-        const uint32_t lane_base = (uint32_t)(32 * warp) << 16;
-        const int s_row = q0 + tid;
+        const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
+        const int s_row = q0 + row;
         const float one_m_theta = 1.f - kGuardHalf;
         const float thr_q = one_m_theta * a.k2 * nq;
         const float base_q = a.k2 * nq + hq;
-        float acc1[KB], acc2[KB];  // direct-difference pairs only
-#pragma unroll
-        for (int k = 0; k < KB; ++k) acc1[k] = acc2[k] = 0.f;
+        // direct-difference pairs only: indexed in loops that stay loops, so that the sums live in local
+        // memory and leave the registers to the exponentials
+        float acc[2 * KB];
+#pragma unroll 1
+        for (int k = 0; k < 2 * KB; ++k) acc[k] = 0.f;
+        bool exact = false;
         auto exact_pair = [&](int t) {
             if (t >= n_ent || s_row >= a.N) return;
             const float2 *rq = a.rx + (size_t)s_row * M;
@@ -352,127 +411,181 @@ __global__ void __launch_bounds__(kTccThreads, 1) detect_tcc_kernel(const TcArgs
                 dC = fmaf(cx, cx, fmaf(cy, cy, dC));
             }
             const float eA = ex2(base_q - a.k2 * dA), eB = ex2(base_q - a.k2 * dB), eC = ex2(base_q - a.k2 * dC);
-#pragma unroll
-            for (int k = 0; k < KB; ++k) {
-                const float g1 = k < a.K ? __ldg(a.gamma + ((size_t)t * 2) * a.K + k) : 0.f;
-                const float gg = k < a.K ? __ldg(a.gamma + ((size_t)t * 2 + 1) * a.K + k) : 0.f;
-                acc1[k] = fmaf(g1, eA, fmaf(gg, eC, acc1[k]));
-                acc2[k] = fmaf(g1, eB, fmaf(gg, eA, acc2[k]));
+            exact = true;
+#pragma unroll 1
+            for (int k = 0; k < a.K; ++k) {
+                const float g1 = __ldg(a.gamma + ((size_t)t * 2) * a.K + k);
+                const float gg = __ldg(a.gamma + ((size_t)t * 2 + 1) * a.K + k);
+                acc[k] = fmaf(g1, eA, fmaf(gg, eC, acc[k]));
+                acc[KB + k] = fmaf(g1, eB, fmaf(gg, eA, acc[KB + k]));
             }
         };
         for (int tile = 0; tile < n_tiles && ok; ++tile) {
-            const int st = tile & 1;
-            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&s_full[st], (tile >> 1) & 1) &&
-                                             mbar_wait_bounded(&mma_done[st], (tile >> 1) & 1))) {
+            const int st = tile % kTccAcc, sg = tile % kTccGStages;
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&g_full[sg], (tile / kTccGStages) & 1) &&
+                                             mbar_wait_bounded(&mma_done[st], (tile / kTccAcc) & 1))) {
                 ok = false;
                 break;
             }
             tc_fence_after();
-            const float *hh = reinterpret_cast<const float *>(sS + st * L::kTile + L::kOH);
+            const float *hh = reinterpret_cast<const float *>(sG + sg * L::kGPart + 2 * L::kGBytes);
 #pragma unroll 1
-            for (int c = 0; c < kChunks; ++c) {
+            for (int c = grp; c < kChunks; c += kTccGroups) {
                 const int g = tile * kChunks + c, xb = g % kTccXBuf;
+                float vr[32];  // (Re z, Im z) of the chunk's 16 entries
+                tcc_tmem_ld32(tmem + lane_base + (uint32_t)(st * NB + 32 * c), vr);
                 // the coefficient GEMM of chunk g - kTccXBuf has read buffer xb
                 if (g >= kTccXBuf &&
                     !__all_sync(0xffffffffu, mbar_wait_bounded(&x_free[xb], ((g - kTccXBuf) / kTccXBuf) & 1))) {
                     ok = false;
                     break;
                 }
-                float vr[32];  // (Re z, Im z) of the chunk's 16 entries
-                tmem_ld16(tmem + lane_base + (uint32_t)(st * NB + 32 * c), *reinterpret_cast<float(*)[16]>(vr));
-                tmem_ld16(tmem + lane_base + (uint32_t)(st * NB + 32 * c + 16), *reinterpret_cast<float(*)[16]>(vr + 16));
-                float hv[CE];
-#pragma unroll
-                for (int q = 0; q < CE / 4; ++q)
-                    *reinterpret_cast<float4 *>(hv + 4 * q) = *reinterpret_cast<const float4 *>(hh + CE * c + 4 * q);
-                float xA[CE], xB[CE], xC[CE];
-                uint32_t fbits = 0;
-#pragma unroll
-                for (int j = 0; j < CE; ++j) {
-                    const float re = vr[2 * j], im = vr[2 * j + 1];
-                    float h = hv[j] + hq;
-                    // flagged: max(v_re, |v_im|) > (1 - theta) k2 (n_s + n_t)
-                    const bool f = fmaxf(re, fabsf(im)) > fmaf(-one_m_theta, hv[j], thr_q);
-                    h = f ? -INFINITY : h;
-                    fbits |= f ? (1u << j) : 0u;
-                    float a2 = re, b2 = im;
-                    add2_bcast(a2, b2, h);
-                    xA[j] = ex2(a2);
-                    xB[j] = ex2(b2);
-                    xC[j] = ex2(h - im);
-                }
                 // X row: k-chunk 2 kind + (j / 8) holds entries 8 (j / 8) .. of one kind
-                unsigned char *xrow = sX + xb * L::kXBytes + tid * 16;
-                const float *src[3] = {xA, xB, xC};
+                unsigned char *xrow = sX + xb * L::kXBytes + row * 16;
+                bool any = false;
 #pragma unroll
-                for (int kind = 0; kind < 3; ++kind) {
+                for (int h8 = 0; h8 < 2; ++h8) {
+                    float hv[8], xA[8], xB[8], xC[8];
+                    *reinterpret_cast<float4 *>(hv) = *reinterpret_cast<const float4 *>(hh + CE * c + 8 * h8);
+                    *reinterpret_cast<float4 *>(hv + 4) = *reinterpret_cast<const float4 *>(hh + CE * c + 8 * h8 + 4);
 #pragma unroll
-                    for (int h8 = 0; h8 < 2; ++h8) {
+                    for (int j = 0; j < 8; ++j) {
+                        const float re = vr[16 * h8 + 2 * j], im = vr[16 * h8 + 2 * j + 1], h = hv[j] + hq;
+                        any |= fmaxf(re, fabsf(im)) > fmaf(-one_m_theta, hv[j], thr_q);
+                        float a2 = re, b2 = im;
+                        add2_bcast(a2, b2, h);
+                        xA[j] = ex2(a2);
+                        xB[j] = ex2(b2);
+                        xC[j] = ex2(h - im);
+                    }
+                    const float *src[3] = {xA, xB, xC};
+#pragma unroll
+                    for (int kind = 0; kind < 3; ++kind) {
                         uint4 v;
                         uint32_t *vp = &v.x;
 #pragma unroll
                         for (int i = 0; i < 4; ++i) {
-                            const __nv_bfloat162 b2 =
-                                __floats2bfloat162_rn(src[kind][8 * h8 + 2 * i], src[kind][8 * h8 + 2 * i + 1]);
+                            const __nv_bfloat162 b2 = __floats2bfloat162_rn(src[kind][2 * i], src[kind][2 * i + 1]);
                             vp[i] = *reinterpret_cast<const uint32_t *>(&b2);
                         }
                         *reinterpret_cast<uint4 *>(xrow + (2 * kind + h8) * kTcRows * 16) = v;
                     }
                 }
+                // flagged: max(v_re, |v_im|) > (1 - theta) k2 (n_s + n_t); such a pair's exponentials leave X
+                uint32_t fbits = 0;
+                const bool slow = __any_sync(0xffffffffu, any);
+                if (slow) {
+#pragma unroll
+                    for (int j = 0; j < CE; ++j) {
+                        const bool f = fmaxf(vr[2 * j], fabsf(vr[2 * j + 1])) > fmaf(-one_m_theta, hh[CE * c + j], thr_q);
+                        if (f) {
+                            fbits |= 1u << j;
+#pragma unroll
+                            for (int kind = 0; kind < 3; ++kind)
+                                *reinterpret_cast<uint16_t *>(xrow + (2 * kind + j / 8) * kTcRows * 16 + (j & 7) * 2) = 0;
+                        }
+                    }
+                }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 mbar_arrive(&x_full[xb]);
-                if (__any_sync(0xffffffffu, fbits != 0)) {
+                if (slow) {
 #pragma unroll 1
                     while (fbits) {
                         const int j = __ffs(fbits) - 1;
                         fbits &= fbits - 1;
                         exact_pair(tile * E + CE * c + j);
                     }
+                    __syncwarp();
                 }
             }
             tc_fence_before();
             mbar_arrive(&epi_done[st]);
         }
         // ---- Y (complete once the last chunk's GEMM has committed) plus the exact pairs -----------
-        if (ok && n_chunks > 0) {
-            const int gl = n_chunks - 1;
-            ok = __all_sync(0xffffffffu, mbar_wait_bounded(&x_free[gl % kTccXBuf], (gl / kTccXBuf) & 1));
-            tc_fence_after();
+        if (!__all_sync(0xffffffffu, mbar_wait_bounded(y_done, 0))) ok = false;
+        tc_fence_after();
+        // the groups' exact sums meet in the tile stages, which nothing reads any more; each group then
+        // writes its share of the users
+        float *s_acc = reinterpret_cast<float *>(sS);  // [group][2KB][128 rows]
+        static_assert(kTccGroups * 2 * KB * kTcRows * 4 <= L::kX - L::kS, "exact sums fit the tile stages");
+        // the filter as [antenna][KB] behind them, for the linear part
+        float2 *s_clin = reinterpret_cast<float2 *>(sX);
+        static_assert(M * KB * 8 <= kTccXBuf * L::kXBytes, "filter fits the exponential buffers");
+        for (int i = tid; i < M * KB; i += kTccEpi)
+            s_clin[i] = i % KB < a.K ? __ldg(a.clin + (size_t)(i / KB) * a.K + i % KB) : make_float2(0.f, 0.f);
+        const bool warp_exact = __any_sync(0xffffffffu, exact);
+        if (warp_exact) s_some = 1;
+        __syncwarp();
+        asm volatile("bar.sync 1, %0;" ::"n"(kTccEpi) : "memory");
+        const bool some = *reinterpret_cast<volatile int *>(&s_some) != 0;
+        if (some) {
+#pragma unroll 1
+            for (int n = 0; n < 2 * KB; ++n) s_acc[(grp * 2 * KB + n) * kTcRows + row] = acc[n];
+            asm volatile("bar.sync 1, %0;" ::"n"(kTccEpi) : "memory");
         }
+        constexpr int KG = (KB + kTccGroups - 1) / kTccGroups;  // users per group
         float y[NY];
 #pragma unroll
         for (int n = 0; n < NY; ++n) y[n] = 0.f;
         if (ok && n_chunks > 0) {
 #pragma unroll
-            for (int n0 = 0; n0 < NY; n0 += 16)
-                tmem_ld16(tmem + lane_base + (uint32_t)(2 * NB + n0), *reinterpret_cast<float(*)[16]>(y + n0));
+            for (int n0 = 0; n0 < NY; n0 += 16) {
+                float lo[16];
+                tmem_ld16(tmem + lane_base + (uint32_t)(kYCol + n0), *reinterpret_cast<float(*)[16]>(y + n0));
+                tmem_ld16(tmem + lane_base + (uint32_t)(kYCol + NY + n0), lo);
+#pragma unroll
+                for (int n = 0; n < 16; ++n) y[n0 + n] += lo[n];
+            }
         }
-        const int s = s_row;
+        const int s = s_row, k0 = grp * KG;
         if (ok && s < a.N) {
             const float fq = cta_in_range ? ex2(-a.k2 * nq) : 1.f;
             const float2 *rq = a.rx + (size_t)s * M;
-            for (int k = 0; k < a.K && k < KB; ++k) {
-                float l1 = 0.f, l2 = 0.f;
-                for (int m = 0; m < M; ++m) {
-                    const float2 cl = __ldg(a.clin + m * a.K + k), r = __ldg(rq + m);
-                    l1 = fmaf(cl.x, r.x, fmaf(cl.y, r.y, l1));
-                    l2 = fmaf(cl.x, r.y, fmaf(-cl.y, r.x, l2));
-                }
-                float y1 = 0.f, y2 = 0.f;
+            float l1[KG], l2[KG], y1[KG], y2[KG];
 #pragma unroll
-                for (int kk = 0; kk < KB; ++kk)
-                    if (kk == k) {
-                        y1 = y[kk] + acc1[kk];
-                        y2 = y[KB + kk] + acc2[kk];
+            for (int u = 0; u < KG; ++u) {
+                l1[u] = l2[u] = y1[u] = y2[u] = 0.f;
+#pragma unroll
+                for (int gi = 0; gi < kTccGroups; ++gi)
+                    if (gi == grp && gi * KG + u < KB) {
+                        y1[u] = y[gi * KG + u];
+                        y2[u] = y[KB + gi * KG + u];
                     }
-                y1 = fmaf(a.wL, l1, a.wG * fq * y1);
-                y2 = fmaf(a.wL, l2, a.wG * fq * y2);
-                a.soft[(size_t)s * a.K + k] = make_float2(y1, y2);
-                if (a.hard) a.hard[(size_t)s * a.K + k] = (uint8_t)((y1 < 0.f ? 1 : 0) | (y2 < 0.f ? 2 : 0));
+            }
+#pragma unroll 2
+            for (int m = 0; m < M; m += 8) {
+                float4 v[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) v[q] = __ldg(reinterpret_cast<const float4 *>(rq + m) + q);
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const float x = c & 1 ? v[c / 2].z : v[c / 2].x, z = c & 1 ? v[c / 2].w : v[c / 2].y;
+#pragma unroll
+                    for (int u = 0; u < KG; ++u) {
+                        const float2 cl = s_clin[(m + c) * KB + min(k0 + u, KB - 1)];
+                        l1[u] = fmaf(cl.x, x, fmaf(cl.y, z, l1[u]));
+                        l2[u] = fmaf(cl.x, z, fmaf(-cl.y, x, l2[u]));
+                    }
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < KG; ++u) {
+                const int k = k0 + u;
+                if (k >= a.K || k >= KB) continue;
+                float e1 = 0.f, e2 = 0.f;
+                if (some)
+                    for (int gi = 0; gi < kTccGroups; ++gi) {
+                        e1 += s_acc[(gi * 2 * KB + k) * kTcRows + row];
+                        e2 += s_acc[(gi * 2 * KB + KB + k) * kTcRows + row];
+                    }
+                const float v1 = fmaf(a.wL, l1[u], a.wG * fq * (y1[u] + e1));
+                const float v2 = fmaf(a.wL, l2[u], a.wG * fq * (y2[u] + e2));
+                a.soft[(size_t)s * a.K + k] = make_float2(v1, v2);
+                if (a.hard) a.hard[(size_t)s * a.K + k] = (uint8_t)((v1 < 0.f ? 1 : 0) | (v2 < 0.f ? 2 : 0));
             }
         }
     }
-    if (!ok && (tid == 0 || tid == 128 || tid == 160)) report(a.status, APSM_ERR_TIMEOUT);
+    if (!ok && (tid & 31) == 0) report(a.status, APSM_ERR_TIMEOUT);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
