@@ -9,34 +9,61 @@
 // entry t): X = the exponentials in BF16, written by the epilogue threads into shared memory a
 // chunk of 16 entries at a time, and G the coefficients arranged per output column (n = k:
 // g1 against E_A, g2 against E_C; n = KB + k: g2 against E_A, g1 against E_B) as a BF16 hi + lo
-// pair, so that their rounding does not count.  Y (128 rows x NY columns, FP32) accumulates in
-// TMEM over the whole dictionary; the FP32 pipe then only forms the exponent arguments.
-// Pairs flagged by the cancellation guard (theta = 2^-4, see detect_tc.cuh) enter X as zero
-// and are recomputed by direct differences into FP32 register sums.
+// pair (rows n and NY + n of one operand), so that their rounding does not count.  Y (128 rows x 2 NY
+// columns, FP32) accumulates in TMEM over the whole dictionary, its halves added at the end; the FP32
+// pipe then only forms the exponent arguments.  Pairs flagged by the cancellation guard (theta = 2^-4,
+// see detect_tc.cuh) enter X as zero and are recomputed by direct differences into FP32 sums, one set
+// per epilogue group, added in group order.
 //
 // Both operands that depend on the dictionary alone -- the Gram's entry operand and G -- are
 // packed once per call by tcc_pack_kernel into the caller's workspace, one contiguous block per
-// 64-entry tile [Gram entry operand | G hi | G lo | -k2 n_t] in exactly the shared-memory layout
-// the MMAs read; the detection CTAs then fetch each tile with one bulk copy.
+// 64-entry tile [Gram entry operand | G | -k2 n_t] in exactly the shared-memory layout the MMAs read;
+// the detection CTAs fetch a tile with two bulk copies, each into its own ring: the Gram operand's
+// stage is free as soon as the Gram has read it, a tile's coefficients only after its last GEMM.
 //
-// Roles (192 threads): warps 0-3 epilogue (query row = thread), warp 4 lane 0 issues the tile
-// copies and the Gram MMAs, warp 5 lane 0 the coefficient MMAs (each as soon as all four
-// epilogue warps have written an exponential chunk).  Two tile stages, two Gram accumulators,
-// two exponential buffers.  All waits are bounded.
+// Roles: epilogue groups of four warps (query row = thread mod 128; group g takes the chunks g,
+// g + groups, .. of every tile, into its own exponential buffer), which also build the query operand and,
+// each for a share of the users, the linear part; one thread that copies and issues the Gram; one that
+// copies the coefficients and issues the coefficient GEMMs (each as soon as a chunk is written).  All
+// waits are bounded.
+//
+// What bounds it: the thread that issues the coefficient GEMMs, 12 small MMAs and 4 waits per tile, some
+// 390 cycles per chunk of which 270 the three MMAs (stamps: a tile every 1900 cycles; an epilogue chunk
+// takes 1200, four at a time).  Measured (BF16, 64 antennas, 16 users, 4096 entries, 262144 vectors):
+// 2717 us with one group of four warps, two stages of whole tiles and hi and lo as MMAs of their own;
+// 2034 with four groups; 1859 with the rings apart and descriptors made once; 1380 with hi and lo as one
+// operand; 1186 with the linear part's rows read once per group (it took 44000 of a CTA's 190000
+// cycles) and the coefficient refill two chunks later.
 #pragma once
+
+#include <type_traits>
 
 #include "detect_tc.cuh"
 
 namespace apsm {
 
 constexpr int kTccChunk = 16;     // entries per exponential chunk
-constexpr int kTccGroups = 4;     // epilogue groups of 128 threads, one chunk of a 64-entry tile each
-constexpr int kTccXBuf = kTccGroups;  // exponential buffers, one per group
-constexpr int kTccAcc = 3;        // Gram accumulators
-constexpr int kTccGStages = 3;    // coefficient stages: a tile's are free only after its last GEMM
-constexpr int kTccEpi = 128 * kTccGroups;
-constexpr int kTccThreads = kTccEpi + 64;
-static_assert(kTcEntries / kTccChunk % kTccGroups == 0, "every group the same chunks of each tile");
+// The two shapes of a CTA: the wide one (one per SM), and a half one for small dictionaries,
+// two of which share an SM, so that one's set-up and output run beside the other's tiles.
+template <bool kHalfCta>
+struct TccCfg {
+    static constexpr int kGroups = kHalfCta ? 2 : 4;   // epilogue groups of 128 threads, a chunk of a tile each in turn
+    static constexpr int kXBuf = kGroups;              // exponential buffers, one per group
+    static constexpr int kEpi = 128 * kGroups;
+    static constexpr int kThreads = kEpi + 64;
+    static constexpr int kAcc = kHalfCta ? 1 : 3;      // Gram accumulators
+    static constexpr int kGStages = kHalfCta ? 2 : 3;  // coefficient stages: a tile's are free only after its last GEMM
+    static constexpr int kCols = kHalfCta ? 256 : 512; // TMEM columns
+    static constexpr int kCtas = kHalfCta ? 2 : 1;     // per SM
+    static_assert(kTcEntries / kTccChunk % kGroups == 0, "every group the same chunks of each tile");
+};
+// The half CTA where there are more query tiles than SMs and the set-up counts: dictionaries of up to 8
+// tiles, and up to 24 where its waves of two per SM round up to no more than the wide one's.  us of
+// device time, wide and half (16 antennas, 6 users, BF16): 128 entries 38900 vectors 24.1 and 18.5,
+// 262144: 122.7 and 79.0; 512 entries 50000 vectors 49.4 and 46.7; 1024 entries 50000 vectors (three waves
+// or two double ones) 72.5 and 76.0, 65536: 93.8 and 85.8; 4096 entries 262144: 951 and 957.  32 antennas,
+// 11 users, 1500 entries: 38900 vectors 80.1 and 76.3, 50000: 113 and 122.
+constexpr int kTccSms = 152, kTccHalfTiles = 8, kTccHalfTilesEven = 24;
 
 // Shared-memory matrix descriptor, K-major, no swizzle, with an explicit leading byte offset
 // (bytes between k-adjacent core matrices) and stride byte offset (between 8-row groups).
@@ -66,8 +93,9 @@ __device__ __forceinline__ void tcc_tmem_ld32(uint32_t taddr, float (&v)[32]) {
     for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
 }
 
-template <int M, int KB>
+template <int M, int KB, bool kHalfCta = false>
 struct TccSmem {
+    using C = TccCfg<kHalfCta>;
     using Sh = TcShape<M, kHalf>;
     static constexpr int E = kTcEntries;
     static constexpr int NY = round_up(2 * KB, 16);               // coefficient GEMM N
@@ -79,12 +107,13 @@ struct TccSmem {
     static constexpr int kOH = kOG + 2 * kGBytes;                 // -k2 n_t [E]
     static constexpr int kTile = round_up(kOH + E * 4, 1024);
     static constexpr int kA = 0;
-    static constexpr int kS = round_up(Sh::kBytesA, 1024);        // 2 stages of the Gram operand
+    static constexpr int kS = round_up(Sh::kBytesA, 1024);        // kBS stages of the Gram operand
     static constexpr int kGBytesAll = 2 * kGBytes + E * 4;        // G and norms of a tile
-    static constexpr int kGPart = round_up(kGBytesAll, 128);      // kTccGStages stages of them
-    static constexpr int kG = kS + 2 * kOG;
-    static constexpr int kX = kG + kTccGStages * kGPart;          // exponential buffers
-    static constexpr int kBar = kX + kTccXBuf * kXBytes;          // mbarriers
+    static constexpr int kGPart = round_up(kGBytesAll, 128);      // C::kGStages stages of them
+    static constexpr int kBS = kHalfCta && M == 32 && NY == 32 ? 1 : 2;  // (one where two would take the SM's second CTA)
+    static constexpr int kG = kS + kBS * kOG;
+    static constexpr int kX = kG + C::kGStages * kGPart;          // exponential buffers
+    static constexpr int kBar = kX + C::kXBuf * kXBytes;          // mbarriers
     static constexpr int kTmem = kBar + 24 * 8;
     static constexpr int kBytes = kTmem + 16;
     static_assert(kBytes <= 227 * 1024, "one CTA per SM");
@@ -173,10 +202,12 @@ __global__ void __launch_bounds__(128) tcc_pack_kernel(const TcArgs a, unsigned 
     }
 }
 
-template <int M, int KB>
-__global__ void __launch_bounds__(kTccThreads, 1) detect_tcc_kernel(const TcArgs a, const unsigned char *packed) {
+template <int M, int KB, bool kHalfCta>
+__global__ void __launch_bounds__(TccCfg<kHalfCta>::kThreads, TccCfg<kHalfCta>::kCtas) detect_tcc_kernel(const TcArgs a, const unsigned char *packed) {
     using Sh = TcShape<M, kHalf>;
-    using L = TccSmem<M, KB>;
+    using L = TccSmem<M, KB, kHalfCta>;
+    using Cfg = TccCfg<kHalfCta>;
+    constexpr int kGroups = Cfg::kGroups, kXBuf = Cfg::kXBuf, kEpi = Cfg::kEpi, kAcc = Cfg::kAcc, kGStages = Cfg::kGStages;
     constexpr int E = kTcEntries, NB = 2 * kTcEntries, CE = kTccChunk, NY = L::NY;
     constexpr int kChunks = E / CE;
     static_assert(KB % 2 == 0 && 2 * KB <= NY, "users in pairs");
@@ -186,14 +217,14 @@ __global__ void __launch_bounds__(kTccThreads, 1) detect_tcc_kernel(const TcArgs
     unsigned char *sG = smem + L::kG;
     unsigned char *sX = smem + L::kX;
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L::kBar);
-    uint64_t *b_full = bars, *mma_done = bars + 2, *epi_done = mma_done + kTccAcc, *x_full = epi_done + kTccAcc,
-             *x_free = x_full + kTccXBuf, *g_full = x_free + kTccXBuf, *y_done = g_full + kTccGStages;
-    static_assert(2 + 2 * kTccAcc + 2 * kTccXBuf + kTccGStages + 1 <= 24, "barriers");
+    uint64_t *b_full = bars, *mma_done = bars + 2, *epi_done = mma_done + kAcc, *x_full = epi_done + kAcc,
+             *x_free = x_full + kXBuf, *g_full = x_free + kXBuf, *y_done = g_full + kGStages;
+    static_assert(2 + 2 * kAcc + 2 * kXBuf + kGStages + 1 <= 24, "barriers");
     uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + L::kTmem);
-    __shared__ float s_nq[kTccEpi];
+    __shared__ float s_nq[kEpi];
     __shared__ int s_some;  // some pair of the CTA went to the direct differences
-    constexpr uint32_t kYCol = kTccAcc * NB;  // Gram accumulators below it, Y at it: 2 NY columns, hi and lo
-    constexpr uint32_t kCols = 512;
+    constexpr uint32_t kYCol = kAcc * NB;  // Gram accumulators below it, Y at it: 2 NY columns, hi and lo
+    constexpr uint32_t kCols = Cfg::kCols;
     static_assert(kYCol + 2 * NY <= kCols, "TMEM columns");
 
     const int tid = threadIdx.x, warp = tid >> 5;
@@ -213,13 +244,13 @@ __global__ void __launch_bounds__(kTccThreads, 1) detect_tcc_kernel(const TcArgs
     if (tid == 0) {
         s_some = 0;
         for (int i = 0; i < 2; ++i) mbar_init(&b_full[i], 1);
-        for (int i = 0; i < kTccAcc; ++i) {
+        for (int i = 0; i < kAcc; ++i) {
             mbar_init(&mma_done[i], 1);
-            mbar_init(&epi_done[i], kTccEpi);
+            mbar_init(&epi_done[i], kEpi);
         }
-        for (int i = 0; i < kTccGStages; ++i) mbar_init(&g_full[i], 1);
+        for (int i = 0; i < kGStages; ++i) mbar_init(&g_full[i], 1);
         mbar_init(y_done, 1);
-        for (int i = 0; i < kTccXBuf; ++i) {
+        for (int i = 0; i < kXBuf; ++i) {
             mbar_init(&x_full[i], kTcRows);
             mbar_init(&x_free[i], 1);
         }
@@ -228,30 +259,30 @@ __global__ void __launch_bounds__(kTccThreads, 1) detect_tcc_kernel(const TcArgs
     // the first two tiles' copies go out before the query operand is built
     __syncthreads();
     auto copy_b = [&](int t) {  // tile t's Gram operand; its coefficients and norms
-        mbar_arrive_expect_tx(&b_full[t & 1], (uint32_t)L::kOG);
-        bulk_g2s(sS + (t & 1) * L::kOG, packed + (size_t)t * L::kTile, (uint32_t)L::kOG, &b_full[t & 1]);
+        mbar_arrive_expect_tx(&b_full[t % L::kBS], (uint32_t)L::kOG);
+        bulk_g2s(sS + t % L::kBS * L::kOG, packed + (size_t)t * L::kTile, (uint32_t)L::kOG, &b_full[t % L::kBS]);
     };
     auto copy_g = [&](int t) {
-        const int sg = t % kTccGStages;
+        const int sg = t % kGStages;
         mbar_arrive_expect_tx(&g_full[sg], (uint32_t)L::kGBytesAll);
         bulk_g2s(sG + sg * L::kGPart, packed + (size_t)t * L::kTile + L::kOG, (uint32_t)L::kGBytesAll, &g_full[sg]);
     };
-    if (tid == kTccEpi) {
-        for (int t = 0; t < kTccGStages && t < n_tiles; ++t) {
-            if (t < 2) copy_b(t);
+    if (tid == kEpi) {
+        for (int t = 0; t < kGStages && t < n_tiles; ++t) {
+            if (t < L::kBS) copy_b(t);
             copy_g(t);
         }
     }
     // ---- the query operand (as detect_tc.cuh) -------------------------------------------------
-    // (a group takes every kTccGroups-th piece of eight antennas of its rows)
+    // (a group takes every kGroups-th piece of eight antennas of its rows)
     static_assert(tc_core_rows<M, kHalf>(), "whole core rows");
-    if (warp < 4 * kTccGroups) {
+    if (warp < 4 * kGroups) {
         constexpr int C = Sh::kCoreK;
         const int row = tid & (kTcRows - 1), s = q0 + row;
         const float2 *rq = a.rx + (size_t)s * M;
         float np = 0.f;
 #pragma unroll
-        for (int p = tid / kTcRows; p < M / C; p += kTccGroups) {
+        for (int p = tid / kTcRows; p < M / C; p += kGroups) {
             float re[C], im[C];
             if (s < a.N) {
                 const float4 *src = reinterpret_cast<const float4 *>(rq + p * C);
@@ -279,27 +310,27 @@ __global__ void __launch_bounds__(kTccThreads, 1) detect_tcc_kernel(const TcArgs
     tc_fence_before();
     __syncthreads();
     float nq = 0.f;  // this row's squared norm
-    if (warp < 4 * kTccGroups) {
+    if (warp < 4 * kGroups) {
 #pragma unroll
-        for (int i = 0; i < kTccGroups; ++i) nq += s_nq[i * kTcRows + (tid & (kTcRows - 1))];
+        for (int i = 0; i < kGroups; ++i) nq += s_nq[i * kTcRows + (tid & (kTcRows - 1))];
     }
     const bool cta_in_range = __syncthreads_and(a.k2 * nq <= kFactorLimit);
     tc_fence_after();
     const uint32_t tmem = *s_tmem;
     bool ok = true;
 
-    if (warp == 4 * kTccGroups) {
+    if (warp == 4 * kGroups) {
         // ================= tile copies and Gram MMAs (one thread) =================
-        if (tid == kTccEpi) {
+        if (tid == kEpi) {
             const uint32_t idesc = (1u << 4) | ((a.half_fmt ? 1u : 0u) << 7) | ((a.half_fmt ? 1u : 0u) << 10) |
                                    ((uint32_t)(NB >> 3) << 17) | ((uint32_t)(kTcRows >> 4) << 24);
             const uint64_t ad = umma_sdesc(smem_u32(sA), Sh::SBO);
-            int issued = min(2, n_tiles), committed = -1;
+            int issued = min(L::kBS, n_tiles), committed = -1;
             for (int t = 0; t < n_tiles; ++t) {
-                const int sb = t & 1, st = t % kTccAcc;
-                // tile t's operand has landed; the epilogue of tile t - kTccAcc freed TMEM stage st
-                if (!mbar_wait_bounded(&b_full[sb], (t >> 1) & 1) ||
-                    (t >= kTccAcc && !mbar_wait_bounded(&epi_done[st], (t / kTccAcc - 1) & 1))) {
+                const int sb = t % L::kBS, st = t % kAcc;
+                // tile t's operand has landed; the epilogue of tile t - kAcc freed TMEM stage st
+                if (!mbar_wait_bounded(&b_full[sb], (t / L::kBS) & 1) ||
+                    (t >= kAcc && !mbar_wait_bounded(&epi_done[st], (t / kAcc - 1) & 1))) {
                     ok = false;
                     break;
                 }
@@ -312,38 +343,38 @@ __global__ void __launch_bounds__(kTccThreads, 1) detect_tcc_kernel(const TcArgs
                                  smem_u32(&mma_done[st]))
                              : "memory");
                 committed = t;
-                if (t + 2 < n_tiles) {  // its stage is free once the Gram has read it
-                    if (!mbar_wait_bounded(&mma_done[st], (t / kTccAcc) & 1)) {
+                if (t + L::kBS < n_tiles) {  // its stage is free once the Gram has read it
+                    if (!mbar_wait_bounded(&mma_done[st], (t / kAcc) & 1)) {
                         ok = false;
                         break;
                     }
-                    copy_b(t + 2);
-                    issued = t + 3;
+                    copy_b(t + L::kBS);
+                    issued = t + L::kBS + 1;
                 }
             }
             // every copy and MMA issued here has landed before the CTA may exit
-            for (int t = max(0, issued - 2); t < issued; ++t) mbar_wait_sleepy(&b_full[t & 1], (t >> 1) & 1);
-            if (committed >= 0) mbar_wait_sleepy(&mma_done[committed % kTccAcc], (committed / kTccAcc) & 1);
+            for (int t = max(0, issued - L::kBS); t < issued; ++t) mbar_wait_sleepy(&b_full[t % L::kBS], (t / L::kBS) & 1);
+            if (committed >= 0) mbar_wait_sleepy(&mma_done[committed % kAcc], (committed / kAcc) & 1);
         }
-    } else if (warp == 4 * kTccGroups + 1) {
+    } else if (warp == 4 * kGroups + 1) {
         // ================= coefficient copies and GEMM issue (one thread) =================
-        if (tid == kTccEpi + 32) {
+        if (tid == kEpi + 32) {
             const uint32_t coef_idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(2 * NY >> 3) << 17) |
                                         ((uint32_t)(kTcRows >> 4) << 24);
             const uint32_t y = tmem + kYCol;
             const uint64_t xd0 = umma_sdesc_lbo(smem_u32(sX), kTcRows * 16, 128);
             const uint64_t gd0 = umma_sdesc_lbo(smem_u32(sG), 2 * NY * 16, 128);
-            int issued = min(kTccGStages, n_tiles);
+            int issued = min(kGStages, n_tiles);
             for (int t = 0; t < n_tiles && ok; ++t) {
-                const int sg = t % kTccGStages;
-                if (!mbar_wait_bounded(&g_full[sg], (t / kTccGStages) & 1)) {
+                const int sg = t % kGStages;
+                if (!mbar_wait_bounded(&g_full[sg], (t / kGStages) & 1)) {
                     ok = false;
                     break;
                 }
 #pragma unroll
                 for (int c = 0; c < kChunks; ++c) {
-                    const int g = t * kChunks + c, xb = g % kTccXBuf;
-                    if (!mbar_wait_bounded(&x_full[xb], (g / kTccXBuf) & 1)) {
+                    const int g = t * kChunks + c, xb = g % kXBuf;
+                    if (!mbar_wait_bounded(&x_full[xb], (g / kXBuf) & 1)) {
                         ok = false;
                         break;
                     }
@@ -360,14 +391,15 @@ __global__ void __launch_bounds__(kTccThreads, 1) detect_tcc_kernel(const TcArgs
                                  : "memory");
                     // the coefficient stage of tile t-1 is free once its last chunk's GEMM is done (whose
                     // x_full also says that every epilogue thread has read the norms); by now it is
-                    if (c == kChunks - 2 && t >= 1 && t - 1 + kTccGStages < n_tiles) {
+                    // (with fewer buffers than chunks a later chunk's x_full has said so already)
+                    if (c == kChunks - 2 && t >= 1 && t - 1 + kGStages < n_tiles) {
                         const int gp = t * kChunks - 1;
-                        if (!mbar_wait_bounded(&x_free[gp % kTccXBuf], (gp / kTccXBuf) & 1)) {
+                        if (kXBuf == kChunks && !mbar_wait_bounded(&x_free[gp % kXBuf], (gp / kXBuf) & 1)) {
                             ok = false;
                             break;
                         }
-                        copy_g(t - 1 + kTccGStages);
-                        issued = t + kTccGStages;
+                        copy_g(t - 1 + kGStages);
+                        issued = t + kGStages;
                     }
                 }
             }
@@ -376,8 +408,8 @@ __global__ void __launch_bounds__(kTccThreads, 1) detect_tcc_kernel(const TcArgs
             asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
                              smem_u32(y_done))
                          : "memory");
-            for (int t = max(0, issued - kTccGStages); t < issued; ++t)
-                mbar_wait_sleepy(&g_full[t % kTccGStages], (t / kTccGStages) & 1);
+            for (int t = max(0, issued - kGStages); t < issued; ++t)
+                mbar_wait_sleepy(&g_full[t % kGStages], (t / kGStages) & 1);
             mbar_wait_sleepy(y_done, 0);
         }
     } else {
@@ -421,22 +453,22 @@ __global__ void __launch_bounds__(kTccThreads, 1) detect_tcc_kernel(const TcArgs
             }
         };
         for (int tile = 0; tile < n_tiles && ok; ++tile) {
-            const int st = tile % kTccAcc, sg = tile % kTccGStages;
-            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&g_full[sg], (tile / kTccGStages) & 1) &&
-                                             mbar_wait_bounded(&mma_done[st], (tile / kTccAcc) & 1))) {
+            const int st = tile % kAcc, sg = tile % kGStages;
+            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&g_full[sg], (tile / kGStages) & 1) &&
+                                             mbar_wait_bounded(&mma_done[st], (tile / kAcc) & 1))) {
                 ok = false;
                 break;
             }
             tc_fence_after();
             const float *hh = reinterpret_cast<const float *>(sG + sg * L::kGPart + 2 * L::kGBytes);
 #pragma unroll 1
-            for (int c = grp; c < kChunks; c += kTccGroups) {
-                const int g = tile * kChunks + c, xb = g % kTccXBuf;
+            for (int c = grp; c < kChunks; c += kGroups) {
+                const int g = tile * kChunks + c, xb = g % kXBuf;
                 float vr[32];  // (Re z, Im z) of the chunk's 16 entries
                 tcc_tmem_ld32(tmem + lane_base + (uint32_t)(st * NB + 32 * c), vr);
-                // the coefficient GEMM of chunk g - kTccXBuf has read buffer xb
-                if (g >= kTccXBuf &&
-                    !__all_sync(0xffffffffu, mbar_wait_bounded(&x_free[xb], ((g - kTccXBuf) / kTccXBuf) & 1))) {
+                // the coefficient GEMM of chunk g - kXBuf has read buffer xb
+                if (g >= kXBuf &&
+                    !__all_sync(0xffffffffu, mbar_wait_bounded(&x_free[xb], ((g - kXBuf) / kXBuf) & 1))) {
                     ok = false;
                     break;
                 }
@@ -507,23 +539,23 @@ __global__ void __launch_bounds__(kTccThreads, 1) detect_tcc_kernel(const TcArgs
         // the groups' exact sums meet in the tile stages, which nothing reads any more; each group then
         // writes its share of the users
         float *s_acc = reinterpret_cast<float *>(sS);  // [group][2KB][128 rows]
-        static_assert(kTccGroups * 2 * KB * kTcRows * 4 <= L::kX - L::kS, "exact sums fit the tile stages");
+        static_assert(kGroups * 2 * KB * kTcRows * 4 <= L::kX - L::kS, "exact sums fit the tile stages");
         // the filter as [antenna][KB] behind them, for the linear part
         float2 *s_clin = reinterpret_cast<float2 *>(sX);
-        static_assert(M * KB * 8 <= kTccXBuf * L::kXBytes, "filter fits the exponential buffers");
-        for (int i = tid; i < M * KB; i += kTccEpi)
+        static_assert(M * KB * 8 <= kXBuf * L::kXBytes, "filter fits the exponential buffers");
+        for (int i = tid; i < M * KB; i += kEpi)
             s_clin[i] = i % KB < a.K ? __ldg(a.clin + (size_t)(i / KB) * a.K + i % KB) : make_float2(0.f, 0.f);
         const bool warp_exact = __any_sync(0xffffffffu, exact);
         if (warp_exact) s_some = 1;
         __syncwarp();
-        asm volatile("bar.sync 1, %0;" ::"n"(kTccEpi) : "memory");
+        asm volatile("bar.sync 1, %0;" ::"n"(kEpi) : "memory");
         const bool some = *reinterpret_cast<volatile int *>(&s_some) != 0;
         if (some) {
 #pragma unroll 1
             for (int n = 0; n < 2 * KB; ++n) s_acc[(grp * 2 * KB + n) * kTcRows + row] = acc[n];
-            asm volatile("bar.sync 1, %0;" ::"n"(kTccEpi) : "memory");
+            asm volatile("bar.sync 1, %0;" ::"n"(kEpi) : "memory");
         }
-        constexpr int KG = (KB + kTccGroups - 1) / kTccGroups;  // users per group
+        constexpr int KG = (KB + kGroups - 1) / kGroups;  // users per group
         float y[NY];
 #pragma unroll
         for (int n = 0; n < NY; ++n) y[n] = 0.f;
@@ -546,7 +578,7 @@ __global__ void __launch_bounds__(kTccThreads, 1) detect_tcc_kernel(const TcArgs
             for (int u = 0; u < KG; ++u) {
                 l1[u] = l2[u] = y1[u] = y2[u] = 0.f;
 #pragma unroll
-                for (int gi = 0; gi < kTccGroups; ++gi)
+                for (int gi = 0; gi < kGroups; ++gi)
                     if (gi == grp && gi * KG + u < KB) {
                         y1[u] = y[gi * KG + u];
                         y2[u] = y[KB + gi * KG + u];
@@ -574,7 +606,7 @@ __global__ void __launch_bounds__(kTccThreads, 1) detect_tcc_kernel(const TcArgs
                 if (k >= a.K || k >= KB) continue;
                 float e1 = 0.f, e2 = 0.f;
                 if (some)
-                    for (int gi = 0; gi < kTccGroups; ++gi) {
+                    for (int gi = 0; gi < kGroups; ++gi) {
                         e1 += s_acc[(gi * 2 * KB + k) * kTcRows + row];
                         e2 += s_acc[(gi * 2 * KB + KB + k) * kTcRows + row];
                     }
@@ -598,7 +630,6 @@ __global__ void __launch_bounds__(kTccThreads, 1) detect_tcc_kernel(const TcArgs
 // detect_tc.cuh (coefficient sums on the FP32 pipe) runs instead.
 template <int M, int KB>
 cudaError_t launch_detect_tcc(const TcArgs &a, void *workspace, size_t ws_bytes, cudaStream_t stream) {
-    using L = TccSmem<M, KB>;
     const int grid = (a.N + kTcRows - 1) / kTcRows;
     if (grid == 0) return cudaSuccess;
     const int n_tiles = (a.n_entries + kTcEntries - 1) / kTcEntries;
@@ -609,11 +640,20 @@ cudaError_t launch_detect_tcc(const TcArgs &a, void *workspace, size_t ws_bytes,
     tcc_pack_kernel<M, KB><<<n_tiles, 128, 0, stream>>>(a, packed);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    auto fn = detect_tcc_kernel<M, KB>;
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kBytes);
-    if (e != cudaSuccess) return e;
-    fn<<<grid, kTccThreads, L::kBytes, stream>>>(a, packed);  // ordinary launches (see launch_detect_tc)
-    return cudaGetLastError();
+    auto run = [&](auto half) {
+        constexpr bool kHalfCta = decltype(half)::value;
+        using S = TccSmem<M, KB, kHalfCta>;
+        auto fn = detect_tcc_kernel<M, KB, kHalfCta>;
+        const cudaError_t r = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kBytes);
+        if (r != cudaSuccess) return r;
+        fn<<<grid, TccCfg<kHalfCta>::kThreads, S::kBytes, stream>>>(a, packed);  // ordinary launches (see launch_detect_tc)
+        return cudaGetLastError();
+    };
+    if constexpr (2 * (TccSmem<M, KB, true>::kBytes + 4096) <= 228 * 1024) {
+        const bool even = (grid + kTccSms - 1) / kTccSms == 2 * ((grid + 2 * kTccSms - 1) / (2 * kTccSms));
+        if (grid > kTccSms && n_tiles <= (even ? kTccHalfTilesEven : kTccHalfTiles)) return run(std::true_type{});
+    }
+    return run(std::false_type{});
 }
 
 using TccLauncher = cudaError_t (*)(const TcArgs &, void *, size_t, cudaStream_t);

@@ -1,7 +1,8 @@
 """BF16/FP16 detection with the coefficient sums on the tensor cores (detect_tcc.cuh): the edges of its
 tiles (128 queries, 64 entries in four chunks, one per epilogue group) and of its rings (two Gram
 operands, three accumulators, three coefficient stages), and pairs close enough for direct
-differences in every group, against the FP64 oracle."""
+differences in every group, against the FP64 oracle;
+the last five cases: dictionaries of one to ten tiles with more query tiles than SMs (half CTAs)."""
 import numpy as np
 import pytest
 import torch
@@ -18,7 +19,9 @@ TOL = 2e-2  # the bound of every reduced-precision detection test here: BF16 Gra
 @pytest.mark.parametrize("dtype", ["bf16", "fp16"])
 @pytest.mark.parametrize("M,K,D,N", [
     (16, 1, 1, 1), (16, 3, 16, 127), (16, 5, 17, 128), (16, 6, 64, 129), (32, 2, 65, 300), (32, 12, 193, 40),
-    (64, 16, 256, 260), (64, 7, 257, 129), (64, 4, 385, 5), (32, 8, 449, 128), (16, 16, 1025, 500)])
+    (64, 16, 256, 260), (64, 7, 257, 129), (64, 4, 385, 5), (32, 8, 449, 128), (16, 16, 1025, 500),
+    (16, 6, 128, 19457), (16, 2, 64, 19700), (32, 5, 100, 20000), (16, 12, 129, 19600),
+    (16, 2, 577, 19457)])
 def test_edges_and_direct_differences(M, K, D, N, dtype):
     ent, gam, clin = synth.random_state(M, K, D, instance=D + M)
     inst = synth.make_instance(M, K, 4, N, 10.0, instance=N + K)
