@@ -158,6 +158,12 @@ __device__ __forceinline__ float ld_cluster(uint32_t smem_addr, uint32_t rank) {
 template <int M, int KB>
 __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const TcArgs a) {
     using L = H3Smem<M, KB>;
+    // 64 antennas and few users (whose outputs average the errors of the Gram the least): hi times hi in
+    // two sums of half the antennas each, added in FP32; two such accumulators instead of four.  Error of
+    // the outputs against 64 bits (2 users, 1898 entries): 1.2e-6 with one sum and the three products
+    // interleaved, 7.5e-7 with the small products first, 3.8e-7 so, 4.4e-7 in the FP32 FMA form.
+    constexpr bool kDual = M == 64 && KB <= 6;
+    constexpr int kAcc = kDual ? 2 : 4;
     constexpr int E = kH3Entries, P8 = M / 8;  // pieces of eight antennas per row
     static_assert(M % 16 == 0 && KB % 2 == 0, "whole MMA k-steps, users in pairs");
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -397,23 +403,27 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const TcArgs a
             if (J > 0 && !mbar_wait_bounded(a_ready, 0)) ok = false;
             for (int j = 0; j < J && ok; ++j) {
                 if (!mbar_wait_bounded(&full[j & 1], (j >> 1) & 1) ||
-                    (j >= 4 && !mbar_wait_bounded(&epi_done[j & 3], ((j - 4) >> 2) & 1))) {
+                    (j >= kAcc && !mbar_wait_bounded(&epi_done[(j - kAcc) & 3], ((j - kAcc) >> 2) & 1))) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
                 const uint32_t b0 = smem_u32(smem + L::kB + (j & 1) * 2 * L::kBCopy);
-                const uint32_t d0 = tmem + (uint32_t)((j & 3) * 4 * E);
+                const uint32_t d0 = tmem + (uint32_t)(j % kAcc * (512 / kAcc));
+                // the small products first: every MMA truncates the sum it adds to, so only the 2M / 16 of
+                // hi times hi do so at the size of the result
 #pragma unroll
-                for (int ks = 0; ks < 2 * M / 16; ++ks) {
-                    const uint64_t bh = umma_sdesc(b0 + ks * 256, L::SBO), bl = umma_sdesc(b0 + L::kBCopy + ks * 256, L::SBO);
+                for (int part = 0; part < 3; ++part) {
 #pragma unroll
-                    for (int q = 0; q < 2; ++q) {
-                        const uint64_t ah = umma_sdesc(a0 + q * 2 * L::kACopy + ks * 256, L::SBO);
-                        const uint64_t al = umma_sdesc(a0 + (q * 2 + 1) * L::kACopy + ks * 256, L::SBO);
-                        umma_f16(d0 + q * 2 * E, al, bh, idesc, ks > 0);
-                        umma_f16(d0 + q * 2 * E, ah, bl, idesc, 1);
-                        umma_f16(d0 + q * 2 * E, ah, bh, idesc, 1);
+                    for (int ks = 0; ks < 2 * M / 16; ++ks) {
+                        const uint64_t bd = umma_sdesc(b0 + (part == 1 ? L::kBCopy : 0) + ks * 256, L::SBO);
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) {
+                            const uint64_t ad = umma_sdesc(a0 + (q * 2 + (part == 0 ? 1 : 0)) * L::kACopy + ks * 256, L::SBO);
+                            const bool second = kDual && part == 2 && ks >= M / 16;  // the second sum, half of hi times hi
+                            umma_f16(d0 + q * 2 * E + (second ? 4 * E : 0), ad, bd, idesc,
+                                     second ? ks > M / 16 : part > 0 || ks > 0);
+                        }
                     }
                 }
                 asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
@@ -480,10 +490,14 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const TcArgs a
             tc_fence_after();
             const float *g = sC + (s * E + 16 * hf) * 2 * KB;
             const float2 *hh = sH + s * E + 16 * hf;
-            const uint32_t col = tmem + lane_base + (uint32_t)(s * 4 * E + 32 * hf);
-            uint32_t v0[8], v1[8];
+            const uint32_t col = tmem + lane_base + (uint32_t)(j % kAcc * (512 / kAcc) + 32 * hf);
+            uint32_t v0[8], v1[8], w0[8], w1[8];
             h3_tmem_ld8(col, v0);
             h3_tmem_ld8(col + 2 * E, v1);
+            if constexpr (kDual) {
+                h3_tmem_ld8(col + 4 * E, w0);
+                h3_tmem_ld8(col + 6 * E, w1);
+            }
 #pragma unroll 1
             for (int c = 0; c < 4; ++c) {  // four entries of both rows; the next four's accumulators follow
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -492,10 +506,18 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const TcArgs a
                 for (int i = 0; i < 8; ++i) {
                     x0[i] = __uint_as_float(v0[i]);
                     x1[i] = __uint_as_float(v1[i]);
+                    if constexpr (kDual) {
+                        x0[i] += __uint_as_float(w0[i]);
+                        x1[i] += __uint_as_float(w1[i]);
+                    }
                 }
                 if (c < 3) {
                     h3_tmem_ld8(col + 8 * (c + 1), v0);
                     h3_tmem_ld8(col + 2 * E + 8 * (c + 1), v1);
+                    if constexpr (kDual) {
+                        h3_tmem_ld8(col + 4 * E + 8 * (c + 1), w0);
+                        h3_tmem_ld8(col + 6 * E + 8 * (c + 1), w1);
+                    }
                 }
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
