@@ -110,7 +110,7 @@ def code_digest(texts):
 
 def kernel_digest():
     texts = []
-    for f in ("detect_tma.cuh", "detect_tc.cuh", "detect_f32.cuh", "apsm_common.cuh"):
+    for f in ("detect_h3.cuh", "detect_tc.cuh", "detect_f32.cuh", "apsm_common.cuh"):
         with open(os.path.join(ROOT, "paper_2201_05024_gb300", "csrc", f)) as fh:
             texts.append(fh.read())
     return code_digest(texts)
@@ -432,9 +432,8 @@ def run_precision(args):
         ms = _time_events(lambda: apsm.detect(q, st, rd, soft=s_, hard=h_, workspace=dw), args.steps, args.warmup)
         soft[dt] = s_
         pairs = N * D
-        # FP32 has no tensor-core kernel above 32 antennas (its TF32 hi/lo operands would not fit
-        # shared memory), so it runs on the FMA engine here; BF16/FP16 form the Gram and the
-        # coefficient sums on the tensor cores.
+        # FP32 forms the Gram from three FP16 products and keeps the coefficient sums on the FP32
+        # pipe; BF16/FP16 form both on the tensor cores.
         engine = "half-tc" if dt != "fp32" else "f16x3"
         out[dt] = {"value": N / (ms / 1e3), "ms": ms, "pairs_per_s": pairs / (ms / 1e3), "engine": engine,
                    "roofline": detect_roofline(dict(M=M, K=K, N=N), D, ms / 1e3, engine),
@@ -646,7 +645,7 @@ def main():
         return
 
     n_entries = int(st.meta[0].item())
-    roof = detect_roofline(w, n_entries, mean_detect / 1e3)
+    roof = detect_roofline(w, n_entries, mean_detect / 1e3, "f16x3")
     roof["traffic"] = DETECT_TRAFFIC["bytes_per_launch"] if DETECT_TRAFFIC["digest"] == kernel_digest() else None
     out = {
         "metric": METRIC, "value": value, "unit": "symbol-vectors/s", "n_gpus": world, "steps": args.steps,
@@ -659,7 +658,7 @@ def main():
                    "ms": mean_detect},
         "train": {"value": world * w["P"] * w["K"] / (mean_train / 1e3), "unit": "pilot-updates/s",
                   "ms": mean_train, "us_per_pilot": mean_train * 1e3 / w["P"]},
-        "roofline": {"kernel": "detect_tma_kernel<16,6> (TF32 x3 Gram)", **roof},
+        "roofline": {"kernel": "detect_h3_kernel<16,6> (FP16 x3 Gram)", **roof},
         "gpu_launches": int(launches),
         "wall_s_timed": wall,
         "e2e": e2e,
