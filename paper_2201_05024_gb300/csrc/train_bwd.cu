@@ -609,6 +609,11 @@ __global__ void __launch_bounds__(kBwdThreads, 6) train_bwd_kernel(const TrainBw
 constexpr int kTeamUsers = 3;
 constexpr int kTeamThreads = 128;
 constexpr int kPfV = 4;    // float4 of a row per lane and table that are staged ahead (512 entries)
+// Up to two CTAs of teams per SM's turn; more users run one warp each, all resident at once (16 antennas,
+// 6 users, 256 pilots, us for n instances, teams and single warps: window 8: 64: 1383 and 2295,
+// 152 (304 CTAs): 2948 and 3020, 200: 4083 and 3603, 512: 9763 and 8021; window 16: 152: 2948 and 3568,
+// 256: 5356 and 4625.  Two team CTAs on an SM at 80 registers a thread: 256 instances 5597).
+constexpr int kTeamCtas = 2 * 152;
 constexpr int kAhead = 3;  // steps ahead that global reads are issued; a ring of kAhead + 1 slots
 
 // Reads of a later step, copied to the lane's own slots of a shared-memory ring (cp.async: no register
@@ -1172,6 +1177,8 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
     }
 }
 
+#include "train_bwd_warp.cuh"
+
 __global__ void train_bwd_sum_kernel(const TrainBwdArgs a0) {
     const TrainBwdArgs a = for_instance(a0, blockIdx.y);
     if (threadIdx.x < 4) {
@@ -1244,8 +1251,13 @@ apsm_status train_bwd_run(const apsm_params *p, int n, const float *rx_pilot, co
     const size_t smem_w =
         sizeof(float) * (2 * (size_t)((2 * P + 3) & ~3) +
                          (size_t)std::min(p->K, kTeamUsers) * bwd_team_floats(2 * P, p->window, 2 * p->M));
-    const bool team_form = p->window <= 30 && smem_w <= 227 * 1024;
-    if (!team_form && smem > 227 * 1024) return APSM_ERR_UNSUPPORTED;
+    const size_t smem_1 =
+        sizeof(float) * (2 * (size_t)((2 * P + 3) & ~3) + (size_t)p->K * bwd_warp_floats(2 * P, p->window, 2 * p->M));
+    const int users = std::min(p->K, kTeamUsers), ctas = (p->K + users - 1) / users;
+    const bool one_fits = p->window <= 32 && smem_1 <= 227 * 1024;
+    const bool team_form = p->window <= 30 && smem_w <= 227 * 1024 && (!one_fits || (long long)ctas * n <= kTeamCtas);
+    const bool one_form = !team_form && one_fits;
+    if (!team_form && !one_form && smem > 227 * 1024) return APSM_ERR_UNSUPPORTED;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) {
         cudaGetLastError();
@@ -1298,8 +1310,13 @@ apsm_status train_bwd_run(const apsm_params *p, int n, const float *rx_pilot, co
                     : p->window <= 16 ? train_bwd_team_kernel<16> : train_bwd_team_kernel<30>;
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_w) != cudaSuccess)
             return APSM_ERR_CUDA;
-        const int users = std::min(p->K, kTeamUsers);
-        kern<<<dim3((p->K + users - 1) / users, n), kTeamThreads * users, smem_w, strm>>>(a);
+        kern<<<dim3(ctas, n), kTeamThreads * users, smem_w, strm>>>(a);
+    } else if (one_form) {
+        auto kern = p->window <= 8 ? train_bwd_warp_kernel<8>
+                    : p->window <= 16 ? train_bwd_warp_kernel<16> : train_bwd_warp_kernel<32>;
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_1) != cudaSuccess)
+            return APSM_ERR_CUDA;
+        kern<<<dim3(1, n), 32 * p->K, smem_1, strm>>>(a);
     } else {
         if (cudaFuncSetAttribute(train_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
             cudaSuccess)

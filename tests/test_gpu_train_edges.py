@@ -34,7 +34,8 @@ def test_adjoint_matches_fp64_model(M, K, P, W):
     inst = synth.make_instance(M, K, P, 16, 10.0, instance=P + W)
     rng = np.random.default_rng(W)
     c0 = (0.1 * (rng.standard_normal((M, K)) + 1j * rng.standard_normal((M, K)))).astype(np.complex64)
-    p = apsm.Params(M=M, K=K, window=W, dict_cap=P, sigma=sig, mu=mu, eps=eps, w_L=wL)
+    D = max(P, (W + 2) // 2)  # (a capacity holds the window)
+    p = apsm.Params(M=M, K=K, window=W, dict_cap=D, sigma=sig, mu=mu, eps=eps, w_L=wL)
     dg = np.zeros((apsm.dict_alloc(p), 2, K), np.float32)
     dg[:P] = 0.1 * rng.standard_normal((P, 2, K))
     dc = (0.1 * (rng.standard_normal((M, K)) + 1j * rng.standard_normal((M, K)))).astype(np.complex64)
@@ -49,12 +50,29 @@ def test_adjoint_matches_fp64_model(M, K, P, W):
         b = np.empty(2 * P)
         b[0::2], b[1::2] = inst.sym_pilot[:, k].real, inst.sym_pilot[:, k].imag
         w0 = np.concatenate([c0[:, k].real, c0[:, k].imag]).astype(np.float64)
-        _, _, tape = forward_direct(X, b, W, P, sig, mu, eps, wL, w0)
+        _, _, tape = forward_direct(X, b, W, D, sig, mu, eps, wL, w0)
         gfin = dg[:P, :, k].astype(np.float64).reshape(-1)
         wfin = np.concatenate([dc[:, k].real, dc[:, k].imag]).astype(np.float64)
-        s, w = reverse_push(X, W, P, sig, mu, wL, tape, gfin, wfin)
+        s, w = reverse_push(X, W, D, sig, mu, wL, tape, gfin, wfin)
         sc += s
         wb[:, k] = w[:M] + 1j * w[M:]
     assert np.abs(dc0.cpu().numpy() - wb).max() <= 3e-3 * np.abs(wb).max()
     assert np.abs(ds.cpu().numpy() - sc).max() <= 3e-3 * np.abs(sc).max()
     assert torch.isfinite(ds).all()
+
+
+@pytest.mark.parametrize("W", [7, 16, 30])
+def test_single_warp_and_team_forms_give_the_same_bits(W):
+    """Past two team CTAs per SM an instance runs one warp per user: the same bits as its own call."""
+    M, K, P, n = 4, 2, 24, 320
+    p = apsm.Params(M=M, K=K, window=W, dict_cap=P, sigma=0.6, mu=0.7, eps=0.02, w_L=0.4)
+    xs = [synth.make_instance(M, K, P, 4, 10.0, instance=i) for i in range(3)]
+    rp = torch.stack([to_dev(xs[i % 3].rx_pilot) for i in range(n)])
+    sp = torch.stack([to_dev(xs[i % 3].sym_pilot) for i in range(n)])
+    g = torch.Generator(device="cpu").manual_seed(W)
+    dg = (0.1 * torch.randn((n, apsm.dict_alloc(p), 2, K), generator=g)).cuda()
+    dc = (0.1 * torch.randn((n, M, K), dtype=torch.complex64, generator=g)).cuda()
+    ds, dc0 = apsm.train_backward_batched(p, rp, sp, dg, dc)
+    for i in (0, 1, 151, n - 1):
+        ds1, dc1 = apsm.train_backward(p, rp[i], sp[i], dg[i], dc[i])
+        assert torch.equal(ds[i], ds1) and torch.equal(dc0[i], dc1)
