@@ -28,8 +28,10 @@
 // Roles (384 threads): warps 0-7 prepare the query operand, then are the epilogue (TMEM lanes
 // 32 (w mod 4) .., entries 16 (w / 4) .. of a tile), warps 8-10 convert entry tiles (hi and lo copies,
 // coefficients, norms; a tile's global loads are issued before the wait for its stage), warp 11
-// issues the MMAs.  Entry operand two stages, coefficients and accumulators four.  All waits are
-// bounded; a timed-out CTA still meets its cluster at both barriers.
+// issues the MMAs.  Entry operand two stages, coefficients and accumulators four.  All waits on an
+// mbarrier are bounded; a timed-out CTA still meets its cluster at both barriers.  Those and the TMEM
+// allocation are the hardware's own waits, without a limit, and end because a CTA has its SM to itself as
+// far as this kernel goes (kH3OneCta) and no other kernel waits for another CTA while it holds TMEM.
 //
 // What bounds it: the FP32 pipe, 4K + 4 FMA per pair (cycle stamps at 64 antennas and 16 users: the
 // epilogue of a tile takes 6700 cycles, 5700 while the converters rest, against 4400 of packed FMAs;
@@ -63,6 +65,13 @@ constexpr int kH3MaxSplit = 8;    // CTAs per cluster
 // entries, 65536 vectors: 93.1 and 84.5; 16 users: 258.8 and 236.9.)
 constexpr int kH3MinEntries16 = 256;
 constexpr int kH3Devices = 16;    // devices whose cluster counts are kept
+// One CTA per SM is a condition of this kernel, not a matter of occupancy: a CTA holds all 512 TMEM
+// columns while it waits for its cluster, so of two on one SM the second would wait in its allocation,
+// and two clusters that meet on two SMs in opposite order would wait for each other for ever.  (At 16
+// antennas and up to 2 users two would fit: 77 registers a thread, 53 KB.)  So every launch asks for
+// more than half of an SM's 228 KB, of which each CTA has 1 KB reserved.
+constexpr int kH3OneCta = 116 * 1024;
+static_assert(2 * (kH3OneCta + 1024) > 228 * 1024, "two CTAs of any instantiations do not fit an SM");
 
 template <int M, int KB>
 struct H3Smem {
@@ -80,9 +89,11 @@ struct H3Smem {
     static constexpr int kBar = kN + kH3Rows * 4;
     static constexpr int kTmem = kBar + 16 * 8;
     static constexpr int kBytes = kTmem + 16;
+    // what a launch asks for: more than half an SM, whatever the registers allow (kH3OneCta)
+    static constexpr int kLaunch = kBytes > kH3OneCta ? kBytes : kH3OneCta;
     // the sums [2KB][kPart] reuse the operands when every MMA is done
     static_assert(2 * KB * kPart * 4 <= kC, "partial sums fit the operand space");
-    static_assert(kBytes <= 227 * 1024, "one CTA per SM");
+    static_assert(kLaunch <= 227 * 1024, "fits an SM");
 };
 
 // Power of two that brings a vector of squared norm n to components below 2^12 (1 for n = 0), and its
@@ -672,12 +683,12 @@ template <int M, int KB>
 cudaError_t launch_detect_h3(const TcArgs &a, int *launches, cudaStream_t stream) {
     using L = H3Smem<M, KB>;
     auto fn = detect_h3_kernel<M, KB>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kBytes);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kLaunch);
     if (e != cudaSuccess) return e;
     const int nq = (a.N + kH3Rows - 1) / kH3Rows, nt = (a.n_entries + kH3Entries - 1) / kH3Entries;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(kH3Threads);
-    cfg.dynamicSmemBytes = L::kBytes;
+    cfg.dynamicSmemBytes = L::kLaunch;
     cfg.stream = stream;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
