@@ -241,7 +241,9 @@ apsm_status apsm_train_noalloc(const apsm_params *p, const float *rx_pilot, cons
  * (norm expansion).  Where that cancels -- the smallest of a pair's three distances below
  * theta k2 (||r||^2 + ||r_t||^2), theta = 2^-4 for BF16/FP16 contractions and 2^-12 for FP32 with
  * inputs outside the factored range -- the pair's distances are recomputed by direct
- * differences in FP32 (direct-difference fallback).
+ * differences in FP32 (direct-difference fallback); the FP32 form of three FP16 products (see
+ * APSM_OPT_DETECT_TMA) recomputes all pairs of a vector outside the range that has an entry so near
+ * that the expansion's error would show.
  *   rx    device [N][M] complex      data vectors
  *   N     >= 0
  *   soft  device [N][K] complex      output

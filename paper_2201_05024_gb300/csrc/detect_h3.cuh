@@ -18,7 +18,8 @@
 //
 // Inside the factor range (k2 n_s <= kFactorLimit for every query of the CTA) the Gram's error is
 // below 2^-21 of k2 (n_s + n_t) in the exponent wherever a term matters; a CTA with a query
-// outside it takes FP32 direct differences throughout.
+// outside it takes the unfactored exponent and, for the rows that need it, FP32 direct differences
+// (H3Guard).
 //
 // Work split: CTAs of a cluster share one query tile and take contiguous parts of the dictionary;
 // at the end each CTA sums the parts of its share of the rows through distributed shared memory,
@@ -46,6 +47,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <type_traits>
 
 #include "detect_tc.cuh"
 
@@ -73,6 +75,25 @@ constexpr int kH3Devices = 16;    // devices whose cluster counts are kept
 constexpr int kH3OneCta = 116 * 1024;
 static_assert(2 * (kH3OneCta + 1024) > 228 * 1024, "two CTAs of any instantiations do not fit an SM");
 
+// Outside the factor range the exponent X - S (X = 2 k2 max(Re z, |Im z|), S = k2 (n_s + n_t)) is off by up to
+// 2^-21 S and its term by as much of itself.  Where 2^(X - S) S <= 4 that is less than 2e-6 of a coefficient;
+// a row with a nearer entry (inputs that share a large offset, which the norm expansion cancels) takes direct
+// differences for all of this CTA's entries.  The test is X <= S - (A + B S) with A + B S >= log2(S) - 2, its
+// tangent at S0 = 2 k2 n_s, plus 2^-12 S for the error itself at any S.
+// Measured (us; the former TF32 x3 or FMA form, the whole CTA by direct differences, and this; 16 antennas, 6
+// users, 1024 entries, 65536 vectors / 32, 11, 1500, 10001 / 64, 16, 4096, 20000): one row in 97 outside 161, 754,
+// 151 / 120, 389, 72 / 2493, 3508, 368; every row, far from the entries, 160, 755, 150 / 119, 388, 72 / 4155, 3509,
+// 368; a common offset that cancels in every pair 160, 755, 705 / 119, 388, 361 / 4149, 3509, 3087, the former
+// forms with errors of up to 6e-5 and 2.5e-4 of the output scale at 16 and 32 antennas, this one 1e-6.
+struct H3Guard {
+    float a, b1;  // -A, B - 1: nearer if X > fmaf(b1, -S, a); never for a row inside the range
+};
+__device__ __forceinline__ H3Guard h3_guard(float k2_ns) {
+    const float s0 = 2.f * k2_ns, e = 1.442695f;
+    if (!(k2_ns > kFactorLimit)) return H3Guard{INFINITY, 0.f};
+    return H3Guard{2.f + e - __log2f(s0), e / s0 + kGuardF32 - 1.f};
+}
+
 template <int M, int KB>
 struct H3Smem {
     static constexpr int kCols = 2 * M / 8;                 // 16-byte k-columns of an operand row
@@ -89,8 +110,16 @@ struct H3Smem {
     static constexpr int kBar = kN + kH3Rows * 4;
     static constexpr int kTmem = kBar + 16 * 8;
     static constexpr int kBytes = kTmem + 16;
+    // rows that take direct differences (h3_direct_rows): their queries, then a tile of entries, after
+    // the partial sums in the operands' space at 64 antennas, else behind everything
+    static constexpr int kDStride = M + 2;                  // float2 per entry row (groups of a warp: other banks)
+    static constexpr int kDirectQ = M > 32 ? 2 * KB * kPart * 4 : kBytes;
+    static constexpr int kDirectD = kDirectQ + kH3Rows * M * 8;
+    static constexpr int kDirectEnd = kDirectD + kH3Entries * kDStride * 8;
+    static_assert(M <= 32 || kDirectEnd <= kC, "within the operand space");
+    static_assert(kDirectQ % 16 == 0 && 2 * KB * kH3Rows * 4 <= kDirectEnd - kDirectQ, "aligned; the groups' sums fit");
     // what a launch asks for: more than half an SM, whatever the registers allow (kH3OneCta)
-    static constexpr int kLaunch = kBytes > kH3OneCta ? kBytes : kH3OneCta;
+    static constexpr int kLaunch = std::max({kBytes, kH3OneCta, M > 32 ? 0 : kDirectEnd});
     // the sums [2KB][kPart] reuse the operands when every MMA is done
     static_assert(2 * KB * kPart * 4 <= kC, "partial sums fit the operand space");
     static_assert(kLaunch <= 227 * 1024, "fits an SM");
@@ -166,8 +195,133 @@ __device__ __forceinline__ float ld_cluster(uint32_t smem_addr, uint32_t rank) {
     return v;
 }
 
+// Adds the kernel sums of the rows in `mask` (one bit per query row of the CTA) to their partial sums, by FP32
+// direct differences against this CTA's entries.  Called by the whole CTA when its operands are free.  The
+// rows are gathered into a power of two of 8 to 256 slots; 256 threads take a slot each and, with few rows, one
+// of 256 / slots groups of the entries, so that one such row in a tile costs a fraction of it.
 template <int M, int KB>
-__global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const TcArgs a) {
+__device__ __noinline__ void h3_direct_rows(const TcArgs &a, unsigned char *smem, const uint32_t *mask, int *count, int q0,
+                                            int t_lo, int J, int n_ent) {
+    using L = H3Smem<M, KB>;
+    constexpr int E = kH3Entries, S = L::kDStride;
+    float *s_part = reinterpret_cast<float *>(smem), *s_grp = reinterpret_cast<float *>(smem + L::kDirectQ);
+    float2 *sq = reinterpret_cast<float2 *>(smem + L::kDirectQ);  // [M][slots]
+    float2 *sd = reinterpret_cast<float2 *>(smem + L::kDirectD);  // [E][S]
+    float *sC = reinterpret_cast<float *>(smem + L::kC);
+    int *rows = reinterpret_cast<int *>(smem + L::kH);
+    static_assert(kH3Rows * 4 <= 4 * E * 8, "row list in the norms' stages");
+    const int tid = threadIdx.x, lane = tid & 31;
+    __syncthreads();  // the mask and the partial sums are complete, the operands and the norms' stages free
+    if (tid < 32) {
+        int n = 0;
+        for (int w = 0; w < kH3Rows / 32; ++w) {
+            const uint32_t m = mask[w];
+            if (m >> lane & 1) rows[n + __popc(m & ((1u << lane) - 1u))] = 32 * w + lane;
+            n += __popc(m);
+        }
+        if (lane == 0) *count = n;
+    }
+    __syncthreads();
+    const int n_rows = *count;
+    if (n_rows == 0) return;
+    int slots = 8;
+    while (slots < n_rows) slots *= 2;
+    for (int i = tid; i < slots * (M / 2); i += kH3Threads) {
+        const int r = i & (slots - 1), c = i / slots;
+        const float4 v = r < n_rows ? __ldg(reinterpret_cast<const float4 *>(a.rx + (size_t)(q0 + rows[r]) * M) + c)
+                                    : make_float4(0.f, 0.f, 0.f, 0.f);
+        sq[2 * c * slots + r] = make_float2(v.x, v.y);
+        sq[(2 * c + 1) * slots + r] = make_float2(v.z, v.w);
+    }
+    const int slot = tid & (slots - 1), grp = tid / slots, groups = kH3Rows / slots;
+    float acc1[KB], acc2[KB];
+#pragma unroll
+    for (int k = 0; k < KB; ++k) acc1[k] = acc2[k] = 0.f;
+    // this group's entries of a tile, kT at a time (a query component serves kT pairs), x and y parts of
+    // the differences as packed pairs
+    auto tile = [&](auto t_c, int cnt) {
+        constexpr int kT = decltype(t_c)::value;
+        const uint64_t neg = pack2(-1.f, -1.f), turn_b = pack2(-1.f, 1.f), turn_c = pack2(1.f, -1.f);
+#pragma unroll 1
+        for (int e = grp; e < cnt; e += kT * groups) {
+            uint64_t dA[kT], dB[kT], dC[kT];
+            const float2 *row[kT];
+#pragma unroll
+            for (int i = 0; i < kT; ++i) {
+                dA[i] = dB[i] = dC[i] = 0;
+                row[i] = sd + min(e + i * groups, cnt - 1) * S;
+            }
+#pragma unroll 2
+            for (int m = 0; m < M; m += 2) {
+                const float2 q[2] = {sq[m * slots + slot], sq[(m + 1) * slots + slot]};
+                const uint64_t qs[2] = {pack2(q[0].x, q[0].y), pack2(q[1].x, q[1].y)};
+                const uint64_t qt[2] = {pack2(q[0].y, q[0].x), pack2(q[1].y, q[1].x)};
+#pragma unroll
+                for (int i = 0; i < kT; ++i) {
+                    const float4 d = *reinterpret_cast<const float4 *>(row[i] + m);
+                    const uint64_t t[2] = {pack2(d.x, d.y), pack2(d.z, d.w)};
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const uint64_t x = ffma2(qs[h], neg, t[h]), y = ffma2(qt[h], turn_b, t[h]), z = ffma2(qt[h], turn_c, t[h]);
+                        dA[i] = ffma2(x, x, dA[i]);  // r_t - r_s
+                        dB[i] = ffma2(y, y, dB[i]);  // r_t + i r_s
+                        dC[i] = ffma2(z, z, dC[i]);  // r_t - i r_s
+                    }
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < kT; ++i) {
+                if (e + i * groups >= cnt) break;
+                const float eA = ex2(-a.k2 * sum2(dA[i])), eB = ex2(-a.k2 * sum2(dB[i])), eC = ex2(-a.k2 * sum2(dC[i]));
+                float g1[KB], gg[KB];
+                load_coef<KB>(sC + (e + i * groups) * 2 * KB, g1, gg);
+#pragma unroll
+                for (int k = 0; k < KB; k += 2) {
+                    fma2_pair(acc1[k], acc1[k + 1], gg[k], gg[k + 1], eC);
+                    fma2_pair(acc1[k], acc1[k + 1], g1[k], g1[k + 1], eA);
+                    fma2_pair(acc2[k], acc2[k + 1], gg[k], gg[k + 1], eA);
+                    fma2_pair(acc2[k], acc2[k + 1], g1[k], g1[k + 1], eB);
+                }
+            }
+        }
+    };
+    for (int j = 0; j < J; ++j) {
+        const int e0 = (t_lo + j) * E, cnt = min(E, n_ent - e0);
+        __syncthreads();
+        for (int i = tid; i < cnt * (M / 2); i += kH3Threads)
+            *reinterpret_cast<float4 *>(sd + i / (M / 2) * S + i % (M / 2) * 2) =
+                __ldg(reinterpret_cast<const float4 *>(a.dict + (size_t)e0 * M) + i);
+        for (int i = tid; i < cnt * 2 * KB; i += kH3Threads) {
+            const int t = e0 + i / (2 * KB), l = i / KB % 2, k = i % KB;
+            sC[i] = k < a.K ? __ldg(a.gamma + ((size_t)t * 2 + l) * a.K + k) : 0.f;
+        }
+        __syncthreads();
+        if (tid < kH3Rows) {
+            if (groups <= E / 4) tile(std::integral_constant<int, 4>{}, cnt);
+            else tile(std::integral_constant<int, 1>{}, cnt);
+        }
+    }
+    // the groups' sums [group][2KB][slots], added in group order
+    __syncthreads();
+    if (tid < kH3Rows) {
+#pragma unroll
+        for (int k = 0; k < KB; ++k) {
+            s_grp[(grp * 2 * KB + k) * slots + slot] = acc1[k];
+            s_grp[(grp * 2 * KB + KB + k) * slots + slot] = acc2[k];
+        }
+    }
+    __syncthreads();
+    for (int i = tid; i < 2 * KB * slots; i += kH3Threads) {
+        const int r = i & (slots - 1), k = i / slots;
+        if (r >= n_rows) continue;
+        float y = 0.f;
+        for (int g = 0; g < groups; ++g) y += s_grp[(g * 2 * KB + k) * slots + r];
+        s_part[k * L::kPart + rows[r]] = fmaf(a.wG, y, s_part[k * L::kPart + rows[r]]);
+    }
+}
+
+template <int M, int KB>
+__global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const __grid_constant__ TcArgs a) {
     using L = H3Smem<M, KB>;
     // 64 antennas and few users (whose outputs average the errors of the Gram the least): hi times hi in
     // two sums of half the antennas each, added in FP32; two such accumulators instead of four.  Error of
@@ -185,6 +339,7 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const TcArgs a
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L::kBar);
     uint64_t *full = bars, *mma_done = bars + 2, *epi_done = bars + 6, *a_ready = bars + 10;  // [2], [4], [4], [1]
     uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + L::kTmem);
+    uint32_t *s_mask = reinterpret_cast<uint32_t *>(bars + 12);  // [8] rows that take direct differences
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int split = (int)cluster_size(), rank = (int)cluster_rank();
@@ -208,6 +363,7 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const TcArgs a
         }
         mbar_init(a_ready, kH3Epi);
         fence_mbar_init();
+        for (int i = 0; i < 8; ++i) s_mask[i] = 0;
     }
     // ---- squared norms of the queries, eight loads in flight per lane (warp w: rows 32 w ..)
     bool in_rng = true;
@@ -238,87 +394,7 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const TcArgs a
     const uint32_t tmem = *s_tmem;
     bool ok = true;
 
-    if (!in_range) {
-        // ================= direct differences =================
-        // A query outside the factor range (k2 n_s > kFactorLimit): the inputs are not gain-controlled
-        // and the norm expansion may cancel, so the whole tile takes FP32 direct differences with the
-        // unfactored exponent, one query per thread, its vector transposed in shared memory.
-        float2 *sq = reinterpret_cast<float2 *>(smem + L::kA);  // [M][256]
-        float2 *sd = reinterpret_cast<float2 *>(smem + L::kB);  // [E][M]
-        for (int i = tid; i < kH3Rows * (M / 2); i += kH3Threads) {
-            const int r = i % kH3Rows, c = i / kH3Rows;
-            const float4 v = q0 + r < a.N ? __ldg(reinterpret_cast<const float4 *>(a.rx + (size_t)(q0 + r) * M) + c)
-                                          : make_float4(0.f, 0.f, 0.f, 0.f);
-            sq[2 * c * kH3Rows + r] = make_float2(v.x, v.y);
-            sq[(2 * c + 1) * kH3Rows + r] = make_float2(v.z, v.w);
-        }
-        float acc1[KB], acc2[KB];
-#pragma unroll
-        for (int k = 0; k < KB; ++k) acc1[k] = acc2[k] = 0.f;
-        for (int j = 0; j < J; ++j) {
-            const int e0 = (t_lo + j) * E, cnt = min(E, n_ent - e0);
-            __syncthreads();
-            for (int i = tid; i < cnt * (M / 2); i += kH3Threads)
-                reinterpret_cast<float4 *>(sd)[i] = __ldg(reinterpret_cast<const float4 *>(a.dict + (size_t)e0 * M) + i);
-            for (int i = tid; i < cnt * 2 * KB; i += kH3Threads) {
-                const int t = e0 + i / (2 * KB), l = i / KB % 2, k = i % KB;
-                sC[i] = k < a.K ? __ldg(a.gamma + ((size_t)t * 2 + l) * a.K + k) : 0.f;
-            }
-            __syncthreads();
-            if (tid < kH3Rows) {
-#pragma unroll 1
-                for (int e = 0; e < cnt; ++e) {
-                    float dA = 0.f, dB = 0.f, dC = 0.f;
-#pragma unroll 4
-                    for (int m = 0; m < M; ++m) {
-                        const float2 qq = sq[m * kH3Rows + tid], d = sd[e * M + m];
-                        const float ax = d.x - qq.x, ay = d.y - qq.y;  // r_t - r_s
-                        const float bx = d.x - qq.y, by = d.y + qq.x;  // r_t + i r_s
-                        const float cx = d.x + qq.y, cy = d.y - qq.x;  // r_t - i r_s
-                        dA = fmaf(ax, ax, fmaf(ay, ay, dA));
-                        dB = fmaf(bx, bx, fmaf(by, by, dB));
-                        dC = fmaf(cx, cx, fmaf(cy, cy, dC));
-                    }
-                    const float eA = ex2(-a.k2 * dA), eB = ex2(-a.k2 * dB), eC = ex2(-a.k2 * dC);
-                    float g1[KB], gg[KB];
-                    load_coef<KB>(sC + e * 2 * KB, g1, gg);
-#pragma unroll
-                    for (int k = 0; k < KB; ++k) {
-                        acc1[k] = fmaf(g1[k], eA, fmaf(gg[k], eC, acc1[k]));
-                        acc2[k] = fmaf(g1[k], eB, fmaf(gg[k], eA, acc2[k]));
-                    }
-                }
-            }
-        }
-        __syncthreads();
-        if (tid < kH3Rows) {
-#pragma unroll
-            for (int k = 0; k < KB; ++k) {
-                acc1[k] *= a.wG;
-                acc2[k] *= a.wG;
-            }
-            if (rank == 0) {  // the linear part w_L c_k^H r
-#pragma unroll 1
-                for (int m = 0; m < M; ++m) {
-                    const float2 x = sq[m * kH3Rows + tid];
-#pragma unroll
-                    for (int k = 0; k < KB; ++k) {
-                        const float2 c = k < a.K ? __ldg(a.clin + m * a.K + k) : make_float2(0.f, 0.f);
-                        acc1[k] = fmaf(a.wL, fmaf(c.x, x.x, c.y * x.y), acc1[k]);
-                        acc2[k] = fmaf(a.wL, fmaf(c.x, x.y, -c.y * x.x), acc2[k]);
-                    }
-                }
-            }
-        }
-        __syncthreads();  // the transposed queries are read; the sums replace them
-        if (tid < kH3Rows) {
-#pragma unroll
-            for (int k = 0; k < KB; ++k) {
-                s_part[k * L::kPart + tid] = acc1[k];
-                s_part[(KB + k) * L::kPart + tid] = acc2[k];
-            }
-        }
-    } else if (warp >= 8 && warp < 11) {
+    if (warp >= 8 && warp < 11) {
         // ================= converters =================
         // one task = eight antennas of one entry: both operand rows.  Of eight consecutive lanes four
         // take one piece and four the next; each stores row 2e + f first, f its piece's parity, so that
@@ -466,6 +542,10 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const TcArgs a
                 const int i = i0 + 32 * n + lane, r = 32 * warp + ((i & 7) | (i / (8 * P8) << 3)), p = (i >> 3) % P8;
                 float inv;
                 const float s = h3_scale(s_nq[r], inv);
+                if (s == 0.f) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) va[n][q] = make_float4(0.f, 0.f, 0.f, 0.f);
+                }
                 float re[8], im[8];
                 h3_unpack(va[n], s, re, im);
                 unsigned char *dst = smem + L::kA + (r >> 7) * 2 * L::kACopy + ((r & 127) >> 3) * L::SBO + (r & 7) * 16;
@@ -492,81 +572,107 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const TcArgs a
 #pragma unroll
             for (int k = 0; k < KB; ++k) acc1[i][k] = acc2[i][k] = 0.f;
         }
-        for (int j = 0; j < J; ++j) {
-            const int s = j & 3;
-            if (!__all_sync(0xffffffffu, mbar_wait_bounded(&mma_done[s], (j >> 2) & 1))) {
-                ok = false;
-                break;
+        // kGuard: a CTA with a query outside the factor range: -k2 n_s goes inside the exponent, and a row
+        // outside it whose terms the Gram's error reaches (H3Guard) is marked
+        auto run_tiles = [&](auto guard_c) {
+            constexpr bool kGuard = decltype(guard_c)::value;
+            float hq[2];  // -k2 n_s
+            H3Guard guard[2];
+            bool mark[2] = {false, false};
+            if constexpr (kGuard) {
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    hq[i] = -a.k2 * s_nq[row + 128 * i];
+                    guard[i] = h3_guard(-hq[i]);
+                }
             }
-            tc_fence_after();
-            const float *g = sC + (s * E + 16 * hf) * 2 * KB;
-            const float2 *hh = sH + s * E + 16 * hf;
-            const uint32_t col = tmem + lane_base + (uint32_t)(j % kAcc * (512 / kAcc) + 32 * hf);
-            uint32_t v0[8], v1[8], w0[8], w1[8];
-            h3_tmem_ld8(col, v0);
-            h3_tmem_ld8(col + 2 * E, v1);
-            if constexpr (kDual) {
-                h3_tmem_ld8(col + 4 * E, w0);
-                h3_tmem_ld8(col + 6 * E, w1);
-            }
+            for (int j = 0; j < J; ++j) {
+                const int s = j & 3;
+                if (!__all_sync(0xffffffffu, mbar_wait_bounded(&mma_done[s], (j >> 2) & 1))) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const float *g = sC + (s * E + 16 * hf) * 2 * KB;
+                const float2 *hh = sH + s * E + 16 * hf;
+                const uint32_t col = tmem + lane_base + (uint32_t)(j % kAcc * (512 / kAcc) + 32 * hf);
+                uint32_t v0[8], v1[8], w0[8], w1[8];
+                h3_tmem_ld8(col, v0);
+                h3_tmem_ld8(col + 2 * E, v1);
+                if constexpr (kDual) {
+                    h3_tmem_ld8(col + 4 * E, w0);
+                    h3_tmem_ld8(col + 6 * E, w1);
+                }
 #pragma unroll 1
-            for (int c = 0; c < 4; ++c) {  // four entries of both rows; the next four's accumulators follow
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                float x0[8], x1[8];
+                for (int c = 0; c < 4; ++c) {  // four entries of both rows; the next four's accumulators follow
+                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                    float x0[8], x1[8];
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    x0[i] = __uint_as_float(v0[i]);
-                    x1[i] = __uint_as_float(v1[i]);
-                    if constexpr (kDual) {
-                        x0[i] += __uint_as_float(w0[i]);
-                        x1[i] += __uint_as_float(w1[i]);
+                    for (int i = 0; i < 8; ++i) {
+                        x0[i] = __uint_as_float(v0[i]);
+                        x1[i] = __uint_as_float(v1[i]);
+                        if constexpr (kDual) {
+                            x0[i] += __uint_as_float(w0[i]);
+                            x1[i] += __uint_as_float(w1[i]);
+                        }
                     }
-                }
-                if (c < 3) {
-                    h3_tmem_ld8(col + 8 * (c + 1), v0);
-                    h3_tmem_ld8(col + 2 * E + 8 * (c + 1), v1);
-                    if constexpr (kDual) {
-                        h3_tmem_ld8(col + 4 * E + 8 * (c + 1), w0);
-                        h3_tmem_ld8(col + 6 * E + 8 * (c + 1), w1);
+                    if (c < 3) {
+                        h3_tmem_ld8(col + 8 * (c + 1), v0);
+                        h3_tmem_ld8(col + 2 * E + 8 * (c + 1), v1);
+                        if constexpr (kDual) {
+                            h3_tmem_ld8(col + 4 * E + 8 * (c + 1), w0);
+                            h3_tmem_ld8(col + 6 * E + 8 * (c + 1), w1);
+                        }
                     }
-                }
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const float2 mh = hh[4 * c + e];
-                    float g1[KB], gg[KB];
-                    load_coef<KB>(g + (4 * c + e) * 2 * KB, g1, gg);
+                    for (int e = 0; e < 4; ++e) {
+                        const float2 mh = hh[4 * c + e];
+                        float g1[KB], gg[KB];
+                        load_coef<KB>(g + (4 * c + e) * 2 * KB, g1, gg);
 #pragma unroll
-                    for (int i = 0; i < 2; ++i) {
-                        const float re = i ? x1[2 * e] : x0[2 * e], im = i ? x1[2 * e + 1] : x0[2 * e + 1];
-                        const float m = gq[i] * mh.x;
-                        const float eA = ex2(fmaf(m, re, mh.y)), eB = ex2(fmaf(m, im, mh.y)), eC = ex2(fmaf(-m, im, mh.y));
+                        for (int i = 0; i < 2; ++i) {
+                            const float re = i ? x1[2 * e] : x0[2 * e], im = i ? x1[2 * e + 1] : x0[2 * e + 1];
+                            const float m = gq[i] * mh.x;
+                            const float h = kGuard ? mh.y + hq[i] : mh.y;
+                            const float eA = ex2(fmaf(m, re, h)), eB = ex2(fmaf(m, im, h)), eC = ex2(fmaf(-m, im, h));
+                            if constexpr (kGuard) mark[i] |= m * fmaxf(re, fabsf(im)) > fmaf(guard[i].b1, h, guard[i].a);
 #pragma unroll
-                        for (int k = 0; k < KB; k += 2) {
-                            fma2_pair(acc1[i][k], acc1[i][k + 1], gg[k], gg[k + 1], eC);
-                            fma2_pair(acc1[i][k], acc1[i][k + 1], g1[k], g1[k + 1], eA);
-                            fma2_pair(acc2[i][k], acc2[i][k + 1], gg[k], gg[k + 1], eA);
-                            fma2_pair(acc2[i][k], acc2[i][k + 1], g1[k], g1[k + 1], eB);
+                            for (int k = 0; k < KB; k += 2) {
+                                fma2_pair(acc1[i][k], acc1[i][k + 1], gg[k], gg[k + 1], eC);
+                                fma2_pair(acc1[i][k], acc1[i][k + 1], g1[k], g1[k + 1], eA);
+                                fma2_pair(acc2[i][k], acc2[i][k + 1], gg[k], gg[k + 1], eA);
+                                fma2_pair(acc2[i][k], acc2[i][k + 1], g1[k], g1[k + 1], eB);
+                            }
                         }
                     }
                 }
+                tc_fence_before();
+                mbar_arrive(&epi_done[s]);
             }
-            tc_fence_before();
-            mbar_arrive(&epi_done[s]);
-        }
-        // query factor and weight
+            if constexpr (kGuard) {
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const float fq = a.wG * ex2(-a.k2 * s_nq[row + 128 * i]);
-#pragma unroll
-            for (int k = 0; k < KB; ++k) {
-                acc1[i][k] *= fq;
-                acc2[i][k] *= fq;
+                for (int i = 0; i < 2; ++i)
+                    if (mark[i]) atomicOr(s_mask + (row + 128 * i) / 32, 1u << (row & 31));
             }
-        }
+        };
+        if (in_range) run_tiles(std::false_type{});
+        else run_tiles(std::true_type{});
         // every MMA of this CTA is done (the last tile's wait above): the coefficient stages take the
         // filter as [antenna][Re, Im][user], the operands' space the sums
         const int p_lo = rank * P8 / split, p_hi = (rank + 1) * P8 / split;  // this CTA's share of the antennas
         asm volatile("bar.sync 1, 256;" ::: "memory");
+        // query factor (inside the exponent already in the guarded form) and weight; a marked row keeps
+        // nothing of the Gram
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const float fq = a.wG * (in_range ? ex2(-a.k2 * s_nq[row + 128 * i]) : 1.f);
+            const bool keep = in_range || !(s_mask[(row + 128 * i) / 32] >> (row & 31) & 1);
+#pragma unroll
+            for (int k = 0; k < KB; ++k) {
+                acc1[i][k] = keep ? acc1[i][k] * fq : 0.f;
+                acc2[i][k] = keep ? acc2[i][k] * fq : 0.f;
+            }
+        }
         for (int i = tid; i < 8 * (p_hi - p_lo) * KB; i += kH3Epi) {
             const int m = i / KB, k = i % KB;
             const float2 c = k < a.K ? __ldg(a.clin + (size_t)(8 * p_lo + m) * a.K + k) : make_float2(0.f, 0.f);
@@ -621,6 +727,7 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const TcArgs a
             s_part[(KB + k) * L::kPart + tid] = hf == 0 ? acc2[0][k] + o2 : o2 + acc2[1][k];
         }
     }
+    if (!in_range) h3_direct_rows<M, KB>(a, smem, s_mask, reinterpret_cast<int *>(s_tmem + 1), q0, t_lo, J, n_ent);
     if (!ok && lane == 0) report(a.status, APSM_ERR_TIMEOUT);
     __syncwarp();
     cluster_sync_all();  // every part of the cluster's query tile is in shared memory
