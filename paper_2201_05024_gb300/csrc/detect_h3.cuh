@@ -94,6 +94,18 @@ __device__ __forceinline__ H3Guard h3_guard(float k2_ns) {
     return H3Guard{2.f + e - __log2f(s0), e / s0 + kGuardF32 - 1.f};
 }
 
+// Sums that hi times hi of a pair is formed in, each over a share of the antennas, added in FP32: every MMA
+// truncates the sum it adds to, so shorter and smaller sums lose less.  Few users' outputs average the
+// errors of the Gram the least.  With four sums a stage takes all of TMEM, so its halves (16 entries each,
+// one half of the epilogue) are issued, waited for and released one by one, which keeps the MMAs running.
+// Error of the outputs against 64 bits at 64 antennas, FMA engine and this (rms over the output's):
+//   2 users, 300 / 700 / 1500 entries   1.64, 2.43, 3.88e-7   four sums 1.29, 1.78, 2.43e-7 (two 1.89, 2.78, 3.51e-7)
+//   3 users, 300 / 700                  1.23, 1.66e-7         two sums 1.15, 1.62e-7
+//   6 users, 300 / 4096                 1.08, 2.71e-7         two sums 0.64, 1.49e-7
+//   8, 12, 16 users, 300                1.06, 1.12, 1.17e-7   one sum 0.64, 0.65, 0.67e-7
+// Four sums cost time: 2 users, 1024 entries, 40000 vectors 152 us against 97 with two (FMA engine 666).
+constexpr int h3_sums(int M, int KB) { return M < 64 || KB > 6 ? 1 : KB > 2 ? 2 : 4; }
+
 template <int M, int KB>
 struct H3Smem {
     static constexpr int kCols = 2 * M / 8;                 // 16-byte k-columns of an operand row
@@ -108,7 +120,8 @@ struct H3Smem {
     static constexpr int kH = kC + 4 * kCStage;             // 4 stages of (1 / scale, -k2 n_t) [E]
     static constexpr int kN = kH + 4 * kH3Entries * 8;      // query norms [256]
     static constexpr int kBar = kN + kH3Rows * 4;
-    static constexpr int kTmem = kBar + 16 * 8;
+    static constexpr int kMask = kBar + 19 * 8;             // rows that take direct differences [8]
+    static constexpr int kTmem = round_up(kMask + 8 * 4, 16);
     static constexpr int kBytes = kTmem + 16;
     // rows that take direct differences (h3_direct_rows): their queries, then a tile of entries, after
     // the partial sums in the operands' space at 64 antennas, else behind everything
@@ -323,12 +336,9 @@ __device__ __noinline__ void h3_direct_rows(const TcArgs &a, unsigned char *smem
 template <int M, int KB>
 __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const __grid_constant__ TcArgs a) {
     using L = H3Smem<M, KB>;
-    // 64 antennas and few users (whose outputs average the errors of the Gram the least): hi times hi in
-    // two sums of half the antennas each, added in FP32; two such accumulators instead of four.  Error of
-    // the outputs against 64 bits (2 users, 1898 entries): 1.2e-6 with one sum and the three products
-    // interleaved, 7.5e-7 with the small products first, 3.8e-7 so, 4.4e-7 in the FP32 FMA form.
-    constexpr bool kDual = M == 64 && KB <= 6;
-    constexpr int kAcc = kDual ? 2 : 4;
+    constexpr int kSums = h3_sums(M, KB), kHalves = kSums == 4 ? 2 : 1;
+    constexpr int kAcc = 4 / kSums;                // accumulator stages
+    constexpr int kStageCols = 512 / kAcc, kNB = 2 * kH3Entries / kHalves;  // TMEM columns of one; MMA N
     constexpr int E = kH3Entries, P8 = M / 8;  // pieces of eight antennas per row
     static_assert(M % 16 == 0 && KB % 2 == 0, "whole MMA k-steps, users in pairs");
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -337,9 +347,9 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const __grid_c
     float *s_nq = reinterpret_cast<float *>(smem + L::kN);
     float *s_part = reinterpret_cast<float *>(smem);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L::kBar);
-    uint64_t *full = bars, *mma_done = bars + 2, *epi_done = bars + 6, *a_ready = bars + 10;  // [2], [4], [4], [1]
+    uint64_t *full = bars, *a_ready = bars + 2, *mma_done = bars + 3, *epi_done = mma_done + 4 * kHalves;  // [2], [1], [4][halves] x 2
     uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + L::kTmem);
-    uint32_t *s_mask = reinterpret_cast<uint32_t *>(bars + 12);  // [8] rows that take direct differences
+    uint32_t *s_mask = reinterpret_cast<uint32_t *>(smem + L::kMask);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int split = (int)cluster_size(), rank = (int)cluster_rank();
@@ -357,9 +367,9 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const __grid_c
     }
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) mbar_init(&full[i], kH3Conv);
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < 4 * kHalves; ++i) {
             mbar_init(&mma_done[i], 1 + kH3Conv);
-            mbar_init(&epi_done[i], kH3Epi);
+            mbar_init(&epi_done[i], kH3Epi / kHalves);
         }
         mbar_init(a_ready, kH3Epi);
         fence_mbar_init();
@@ -449,9 +459,11 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const __grid_c
             const float n_t = ct < E && e0 + ct < n_ent ? __ldg(a.dict_norm + e0 + ct) : 0.f;
             // the entry stage is free when the MMAs of tile j-2 are done, the coefficient stage when the
             // epilogue of tile j-4 is
-            if ((j >= 2 && !mbar_wait_sleepy(&mma_done[(j - 2) & 3], ((j - 2) >> 2) & 1)) ||
-                (j >= 4 && !mbar_wait_sleepy(&epi_done[sc], ((j - 4) >> 2) & 1)))
-                ok = false;
+#pragma unroll
+            for (int h = 0; h < kHalves; ++h)
+                if ((j >= 2 && !mbar_wait_sleepy(&mma_done[((j - 2) & 3) * kHalves + h], ((j - 2) >> 2) & 1)) ||
+                    (j >= 4 && !mbar_wait_sleepy(&epi_done[sc * kHalves + h], ((j - 4) >> 2) & 1)))
+                    ok = false;
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
 #pragma unroll
@@ -479,46 +491,56 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const __grid_c
             }
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             mbar_arrive(&full[sb]);
-            mbar_arrive(&mma_done[sc]);  // releases this thread's coefficients and norms to the epilogue
+#pragma unroll
+            for (int h = 0; h < kHalves; ++h)  // releases this thread's coefficients and norms to the epilogue
+                mbar_arrive(&mma_done[sc * kHalves + h]);
         }
     } else if (warp == 11) {
         // ================= MMA issue =================
         if (lane == 0) {
-            const uint32_t idesc = (1u << 4) | ((uint32_t)(2 * E >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);  // FP16, FP32 sums
+            const uint32_t idesc = (1u << 4) | ((uint32_t)(kNB >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);  // FP16, FP32 sums
             const uint32_t a0 = smem_u32(smem + L::kA);
             int committed = -1;
             if (J > 0 && !mbar_wait_bounded(a_ready, 0)) ok = false;
             for (int j = 0; j < J && ok; ++j) {
-                if (!mbar_wait_bounded(&full[j & 1], (j >> 1) & 1) ||
-                    (j >= kAcc && !mbar_wait_bounded(&epi_done[(j - kAcc) & 3], ((j - kAcc) >> 2) & 1))) {
+                if (!mbar_wait_bounded(&full[j & 1], (j >> 1) & 1)) {
                     ok = false;
                     break;
                 }
-                tc_fence_after();
-                const uint32_t b0 = smem_u32(smem + L::kB + (j & 1) * 2 * L::kBCopy);
-                const uint32_t d0 = tmem + (uint32_t)(j % kAcc * (512 / kAcc));
-                // the small products first: every MMA truncates the sum it adds to, so only the 2M / 16 of
-                // hi times hi do so at the size of the result
 #pragma unroll
-                for (int part = 0; part < 3; ++part) {
+                for (int h = 0; h < kHalves; ++h) {
+                    if (j >= kAcc && !mbar_wait_bounded(&epi_done[((j - kAcc) & 3) * kHalves + h], ((j - kAcc) >> 2) & 1)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint32_t b0 = smem_u32(smem + L::kB + (j & 1) * 2 * L::kBCopy) + h * (kNB / 8) * L::SBO;
+                    const uint32_t d0 = tmem + (uint32_t)(j % kAcc * kStageCols + h * (kStageCols / kHalves));
+                    // the small products first, into the first sum: only hi times hi adds at the size of the result
 #pragma unroll
-                    for (int ks = 0; ks < 2 * M / 16; ++ks) {
-                        const uint64_t bd = umma_sdesc(b0 + (part == 1 ? L::kBCopy : 0) + ks * 256, L::SBO);
+                    for (int part = 0; part < 3; ++part) {
 #pragma unroll
-                        for (int q = 0; q < 2; ++q) {
-                            const uint64_t ad = umma_sdesc(a0 + (q * 2 + (part == 0 ? 1 : 0)) * L::kACopy + ks * 256, L::SBO);
-                            const bool second = kDual && part == 2 && ks >= M / 16;  // the second sum, half of hi times hi
-                            umma_f16(d0 + q * 2 * E + (second ? 4 * E : 0), ad, bd, idesc,
-                                     second ? ks > M / 16 : part > 0 || ks > 0);
+                        for (int ks = 0; ks < 2 * M / 16; ++ks) {
+                            const uint64_t bd = umma_sdesc(b0 + (part == 1 ? L::kBCopy : 0) + ks * 256, L::SBO);
+                            constexpr int kPer = 2 * M / 16 / kSums;  // k-steps of hi times hi per sum
+                            const int sum = part == 2 ? ks / kPer : 0;
+#pragma unroll
+                            for (int q = 0; q < 2; ++q) {
+                                const uint64_t ad = umma_sdesc(a0 + (q * 2 + (part == 0 ? 1 : 0)) * L::kACopy + ks * 256, L::SBO);
+                                umma_f16(d0 + (2 * sum + q) * kNB, ad, bd, idesc, sum > 0 ? ks % kPer > 0 : part > 0 || ks > 0);
+                            }
                         }
                     }
+                    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                                     smem_u32(&mma_done[(j & 3) * kHalves + h]))
+                                 : "memory");
+                    committed = j * kHalves + h;
                 }
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                                 smem_u32(&mma_done[j & 3]))
-                             : "memory");
-                committed = j;
             }
-            if (committed >= 0) mbar_wait_bounded(&mma_done[committed & 3], (committed >> 2) & 1);
+            if (committed >= 0) {  // (of the last tile's halves the one committed last)
+                const int j = committed / kHalves;
+                mbar_wait_bounded(&mma_done[(j & 3) * kHalves + committed % kHalves], (j >> 2) & 1);
+            }
         }
         __syncwarp();
     } else {
@@ -588,42 +610,36 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const __grid_c
             }
             for (int j = 0; j < J; ++j) {
                 const int s = j & 3;
-                if (!__all_sync(0xffffffffu, mbar_wait_bounded(&mma_done[s], (j >> 2) & 1))) {
+                const int bar = s * kHalves + (kHalves > 1 ? hf : 0);
+                if (!__all_sync(0xffffffffu, mbar_wait_bounded(&mma_done[bar], (j >> 2) & 1))) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
                 const float *g = sC + (s * E + 16 * hf) * 2 * KB;
                 const float2 *hh = sH + s * E + 16 * hf;
-                const uint32_t col = tmem + lane_base + (uint32_t)(j % kAcc * (512 / kAcc) + 32 * hf);
-                uint32_t v0[8], v1[8], w0[8], w1[8];
-                h3_tmem_ld8(col, v0);
-                h3_tmem_ld8(col + 2 * E, v1);
-                if constexpr (kDual) {
-                    h3_tmem_ld8(col + 4 * E, w0);
-                    h3_tmem_ld8(col + 6 * E, w1);
-                }
+                const uint32_t col =
+                    tmem + lane_base + (uint32_t)(j % kAcc * kStageCols + (kHalves > 1 ? hf * (kStageCols / 2) : 32 * hf));
+                uint32_t v[kSums][2][8];  // [sum][query tile]
+                auto load = [&](int c) {
+#pragma unroll
+                    for (int w = 0; w < kSums; ++w)
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) h3_tmem_ld8(col + (2 * w + q) * kNB + 8 * c, v[w][q]);
+                };
+                load(0);
 #pragma unroll 1
                 for (int c = 0; c < 4; ++c) {  // four entries of both rows; the next four's accumulators follow
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    float x0[8], x1[8];
+                    float x[2][8];
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        x0[i] = __uint_as_float(v0[i]);
-                        x1[i] = __uint_as_float(v1[i]);
-                        if constexpr (kDual) {
-                            x0[i] += __uint_as_float(w0[i]);
-                            x1[i] += __uint_as_float(w1[i]);
+                    for (int q = 0; q < 2; ++q)
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            auto val = [&](int w) { return __uint_as_float(v[w < kSums ? w : 0][q][i]); };
+                            x[q][i] = kSums == 4 ? (val(0) + val(1)) + (val(2) + val(3)) : kSums == 2 ? val(0) + val(1) : val(0);
                         }
-                    }
-                    if (c < 3) {
-                        h3_tmem_ld8(col + 8 * (c + 1), v0);
-                        h3_tmem_ld8(col + 2 * E + 8 * (c + 1), v1);
-                        if constexpr (kDual) {
-                            h3_tmem_ld8(col + 4 * E + 8 * (c + 1), w0);
-                            h3_tmem_ld8(col + 6 * E + 8 * (c + 1), w1);
-                        }
-                    }
+                    if (c < 3) load(c + 1);
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         const float2 mh = hh[4 * c + e];
@@ -631,7 +647,7 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const __grid_c
                         load_coef<KB>(g + (4 * c + e) * 2 * KB, g1, gg);
 #pragma unroll
                         for (int i = 0; i < 2; ++i) {
-                            const float re = i ? x1[2 * e] : x0[2 * e], im = i ? x1[2 * e + 1] : x0[2 * e + 1];
+                            const float re = x[i][2 * e], im = x[i][2 * e + 1];
                             const float m = gq[i] * mh.x;
                             const float h = kGuard ? mh.y + hq[i] : mh.y;
                             const float eA = ex2(fmaf(m, re, h)), eB = ex2(fmaf(m, im, h)), eC = ex2(fmaf(-m, im, h));
@@ -647,7 +663,7 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const __grid_c
                     }
                 }
                 tc_fence_before();
-                mbar_arrive(&epi_done[s]);
+                mbar_arrive(&epi_done[bar]);
             }
             if constexpr (kGuard) {
 #pragma unroll
@@ -659,7 +675,12 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const __grid_c
         else run_tiles(std::true_type{});
         // every MMA of this CTA is done (the last tile's wait above): the coefficient stages take the
         // filter as [antenna][Re, Im][user], the operands' space the sums
-        const int p_lo = rank * P8 / split, p_hi = (rank + 1) * P8 / split;  // this CTA's share of the antennas
+        // this CTA's share of the antennas, in pieces of kLin: eight, whose short sums lose the least, but all at
+        // once with as many users as antennas, where the filter's terms are large and cancel, and a part of
+        // their sum added to the kernel sums costs bits (16 antennas and users, error of the outputs: 300 entries
+        // 2.59e-7 in two pieces, 2.36e-7 in one, 2.31e-7 in the TMA-staged form; 1500: 2.68e-7, 2.37e-7, 2.43e-7)
+        constexpr int kLin = M == 16 && KB == 16 ? 16 : 8, kPieces = M / kLin;
+        const int p_lo = rank * kPieces / split, p_hi = (rank + 1) * kPieces / split;
         asm volatile("bar.sync 1, 256;" ::: "memory");
         // query factor (inside the exponent already in the guarded form) and weight; a marked row keeps
         // nothing of the Gram
@@ -673,9 +694,9 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const __grid_c
                 acc2[i][k] = keep ? acc2[i][k] * fq : 0.f;
             }
         }
-        for (int i = tid; i < 8 * (p_hi - p_lo) * KB; i += kH3Epi) {
+        for (int i = tid; i < kLin * (p_hi - p_lo) * KB; i += kH3Epi) {
             const int m = i / KB, k = i % KB;
-            const float2 c = k < a.K ? __ldg(a.clin + (size_t)(8 * p_lo + m) * a.K + k) : make_float2(0.f, 0.f);
+            const float2 c = k < a.K ? __ldg(a.clin + (size_t)(kLin * p_lo + m) * a.K + k) : make_float2(0.f, 0.f);
             sC[2 * m * KB + k] = c.x;
             sC[(2 * m + 1) * KB + k] = c.y;
         }
@@ -685,16 +706,16 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const __grid_c
         const float2 *rq = a.rx + (size_t)min(q0 + tid, a.N - 1) * M;
 #pragma unroll 1
         for (int p = p_lo; p < p_hi; ++p) {
-            float4 v[4];
+            float4 v[kLin / 2];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) v[c] = __ldg(reinterpret_cast<const float4 *>(rq + 8 * p) + c);
-            float l1[KB], l2[KB];  // eight antennas, then added: short sums
+            for (int c = 0; c < kLin / 2; ++c) v[c] = __ldg(reinterpret_cast<const float4 *>(rq + kLin * p) + c);
+            float l1[KB], l2[KB];  // a piece's sums, then added
 #pragma unroll
             for (int k = 0; k < KB; ++k) l1[k] = l2[k] = 0.f;
 #pragma unroll
-            for (int m = 0; m < 8; ++m) {
+            for (int m = 0; m < kLin; ++m) {
                 const float x = m & 1 ? v[m >> 1].z : v[m >> 1].x, y = m & 1 ? v[m >> 1].w : v[m >> 1].y;
-                const float *cx = sC + 2 * (8 * (p - p_lo) + m) * KB, *cy = cx + KB;
+                const float *cx = sC + 2 * (kLin * (p - p_lo) + m) * KB, *cy = cx + KB;
 #pragma unroll
                 for (int k = 0; k < KB; k += 2) {
                     const float2 u = *reinterpret_cast<const float2 *>(cx + k), w = *reinterpret_cast<const float2 *>(cy + k);
