@@ -421,35 +421,69 @@ __global__ void __launch_bounds__(TccCfg<kHalfCta>::kThreads, TccCfg<kHalfCta>::
         const float one_m_theta = 1.f - kGuardHalf;
         const float thr_q = one_m_theta * a.k2 * nq;
         const float base_q = a.k2 * nq + hq;
-        // direct-difference pairs only: indexed in loops that stay loops, so that the sums live in local
-        // memory and leave the registers to the exponentials
+        // direct-difference pairs only: indexed by a variable, so that the sums live in local memory and leave
+        // the registers to the exponentials; set at the thread's first such pair (shared memory leaves next to
+        // no L1, so every access to them is a trip to L2)
         float acc[2 * KB];
-#pragma unroll 1
-        for (int k = 0; k < 2 * KB; ++k) acc[k] = 0.f;
         bool exact = false;
+        // A pair's loads go out in few rounds (the first eight users' coefficients, then eight antennas at a
+        // time): where such pairs are rare each is a chain of trips to L2 that the other warps of the CTA end
+        // up waiting for.  32 antennas, 11 users, 159 entries, 18688 vectors, 9 such pairs among them: 33.4 us with
+        // serial loads and sums set and read back one by one, 27.3 so, 25.1 without any such pair (one epilogue
+        // group and the sums in registers: 28.6 and 27.2).  16 antennas, 2 users, 1500 entries, 60000 vectors, such
+        // pairs in every warp: 2065 and 1356 (2602).
         auto exact_pair = [&](int t) {
             if (t >= n_ent || s_row >= a.N) return;
-            const float2 *rq = a.rx + (size_t)s_row * M;
-            const float2 *rt = a.dict + (size_t)t * M;
+            const float4 *rq = reinterpret_cast<const float4 *>(a.rx + (size_t)s_row * M);
+            const float4 *rt = reinterpret_cast<const float4 *>(a.dict + (size_t)t * M);
+            const float *gt = a.gamma + (size_t)t * 2 * a.K;
+            constexpr int kU = KB < 8 ? KB : 8;
+            float g1[kU], gg[kU];
+            auto load_users = [&](int k0) {
+#pragma unroll
+                for (int i = 0; i < kU; ++i) {
+                    g1[i] = k0 + i < a.K ? __ldg(gt + k0 + i) : 0.f;
+                    gg[i] = k0 + i < a.K ? __ldg(gt + a.K + k0 + i) : 0.f;
+                }
+            };
+            load_users(0);
             float dA = 0.f, dB = 0.f, dC = 0.f;
-#pragma unroll 4
-            for (int m = 0; m < M; ++m) {
-                const float2 q = __ldg(rq + m), d = __ldg(rt + m);
-                const float ax = d.x - q.x, ay = d.y - q.y;
-                const float bx = d.x - q.y, by = d.y + q.x;
-                const float cx = d.x + q.y, cy = d.y - q.x;
-                dA = fmaf(ax, ax, fmaf(ay, ay, dA));
-                dB = fmaf(bx, bx, fmaf(by, by, dB));
-                dC = fmaf(cx, cx, fmaf(cy, cy, dC));
+#pragma unroll 1
+            for (int m = 0; m < M / 2; m += 4) {
+                float4 q[4], d[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    q[i] = __ldg(rq + m + i);
+                    d[i] = __ldg(rt + m + i);
+                }
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const float qx = i & 1 ? q[i / 2].z : q[i / 2].x, qy = i & 1 ? q[i / 2].w : q[i / 2].y;
+                    const float dx = i & 1 ? d[i / 2].z : d[i / 2].x, dy = i & 1 ? d[i / 2].w : d[i / 2].y;
+                    const float ax = dx - qx, ay = dy - qy;
+                    const float bx = dx - qy, by = dy + qx;
+                    const float cx = dx + qy, cy = dy - qx;
+                    dA = fmaf(ax, ax, fmaf(ay, ay, dA));
+                    dB = fmaf(bx, bx, fmaf(by, by, dB));
+                    dC = fmaf(cx, cx, fmaf(cy, cy, dC));
+                }
             }
             const float eA = ex2(base_q - a.k2 * dA), eB = ex2(base_q - a.k2 * dB), eC = ex2(base_q - a.k2 * dC);
-            exact = true;
+            if (!exact) {
+#pragma unroll
+                for (int k = 0; k < 2 * KB; ++k) acc[k] = 0.f;
+                exact = true;
+            }
 #pragma unroll 1
-            for (int k = 0; k < a.K; ++k) {
-                const float g1 = __ldg(a.gamma + ((size_t)t * 2) * a.K + k);
-                const float gg = __ldg(a.gamma + ((size_t)t * 2 + 1) * a.K + k);
-                acc[k] = fmaf(g1, eA, fmaf(gg, eC, acc[k]));
-                acc[KB + k] = fmaf(g1, eB, fmaf(gg, eA, acc[KB + k]));
+            for (int k0 = 0; k0 < a.K; k0 += kU) {
+                if (k0 > 0) load_users(k0);
+#pragma unroll
+                for (int i = 0; i < kU; ++i) {
+                    if (k0 + i < a.K) {
+                        acc[k0 + i] = fmaf(g1[i], eA, fmaf(gg[i], eC, acc[k0 + i]));
+                        acc[KB + k0 + i] = fmaf(g1[i], eB, fmaf(gg[i], eA, acc[KB + k0 + i]));
+                    }
+                }
             }
         };
         for (int tile = 0; tile < n_tiles && ok; ++tile) {
@@ -551,8 +585,8 @@ __global__ void __launch_bounds__(TccCfg<kHalfCta>::kThreads, TccCfg<kHalfCta>::
         asm volatile("bar.sync 1, %0;" ::"n"(kEpi) : "memory");
         const bool some = *reinterpret_cast<volatile int *>(&s_some) != 0;
         if (some) {
-#pragma unroll 1
-            for (int n = 0; n < 2 * KB; ++n) s_acc[(grp * 2 * KB + n) * kTcRows + row] = acc[n];
+#pragma unroll
+            for (int n = 0; n < 2 * KB; ++n) s_acc[(grp * 2 * KB + n) * kTcRows + row] = exact ? acc[n] : 0.f;
             asm volatile("bar.sync 1, %0;" ::"n"(kEpi) : "memory");
         }
         constexpr int KG = (KB + kGroups - 1) / kGroups;  // users per group
