@@ -124,15 +124,16 @@ struct H3Smem {
     static constexpr int kTmem = round_up(kMask + 8 * 4, 16);
     static constexpr int kBytes = kTmem + 16;
     // rows that take direct differences (h3_direct_rows): their queries, then a tile of entries, after
-    // the partial sums in the operands' space at 64 antennas, else behind everything
+    // the partial sums in the operands' space and the first coefficient stages (the last holds theirs), at 16
+    // antennas behind everything, in what the launch asks for anyway
     static constexpr int kDStride = M + 2;                  // float2 per entry row (groups of a warp: other banks)
-    static constexpr int kDirectQ = M > 32 ? 2 * KB * kPart * 4 : kBytes;
+    static constexpr int kDirectQ = M > 16 ? 2 * KB * kPart * 4 : kBytes;
     static constexpr int kDirectD = kDirectQ + kH3Rows * M * 8;
     static constexpr int kDirectEnd = kDirectD + kH3Entries * kDStride * 8;
-    static_assert(M <= 32 || kDirectEnd <= kC, "within the operand space");
+    static_assert(kDirectEnd <= (M > 16 ? kC + 3 * kCStage : kH3OneCta), "within them");
     static_assert(kDirectQ % 16 == 0 && 2 * KB * kH3Rows * 4 <= kDirectEnd - kDirectQ, "aligned; the groups' sums fit");
     // what a launch asks for: more than half an SM, whatever the registers allow (kH3OneCta)
-    static constexpr int kLaunch = std::max({kBytes, kH3OneCta, M > 32 ? 0 : kDirectEnd});
+    static constexpr int kLaunch = std::max(kBytes, kH3OneCta);
     // the sums [2KB][kPart] reuse the operands when every MMA is done
     static_assert(2 * KB * kPart * 4 <= kC, "partial sums fit the operand space");
     static_assert(kLaunch <= 227 * 1024, "fits an SM");
@@ -220,7 +221,7 @@ __device__ __noinline__ void h3_direct_rows(const TcArgs &a, unsigned char *smem
     float *s_part = reinterpret_cast<float *>(smem), *s_grp = reinterpret_cast<float *>(smem + L::kDirectQ);
     float2 *sq = reinterpret_cast<float2 *>(smem + L::kDirectQ);  // [M][slots]
     float2 *sd = reinterpret_cast<float2 *>(smem + L::kDirectD);  // [E][S]
-    float *sC = reinterpret_cast<float *>(smem + L::kC);
+    float *sC = reinterpret_cast<float *>(smem + L::kC + 3 * L::kCStage);
     int *rows = reinterpret_cast<int *>(smem + L::kH);
     static_assert(kH3Rows * 4 <= 4 * E * 8, "row list in the norms' stages");
     const int tid = threadIdx.x, lane = tid & 31;
@@ -554,9 +555,10 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const __grid_c
 #pragma unroll
             for (int n = 0; n < kBatch; ++n) {
                 const int i = i0 + 32 * n + lane, r = 32 * warp + ((i & 7) | (i / (8 * P8) << 3)), p = (i >> 3) % P8;
+                const bool ok = q0 + r < a.N && fabsf(s_nq[r]) < INFINITY;  // (zeros where the norm is not finite)
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
-                    va[n][q] = q0 + r < a.N ? __ldg(reinterpret_cast<const float4 *>(a.rx + (size_t)(q0 + r) * M + p * 8) + q)
+                    va[n][q] = ok ? __ldg(reinterpret_cast<const float4 *>(a.rx + (size_t)(q0 + r) * M + p * 8) + q)
                                             : make_float4(0.f, 0.f, 0.f, 0.f);
             }
 #pragma unroll
@@ -564,10 +566,6 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const __grid_c
                 const int i = i0 + 32 * n + lane, r = 32 * warp + ((i & 7) | (i / (8 * P8) << 3)), p = (i >> 3) % P8;
                 float inv;
                 const float s = h3_scale(s_nq[r], inv);
-                if (s == 0.f) {
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) va[n][q] = make_float4(0.f, 0.f, 0.f, 0.f);
-                }
                 float re[8], im[8];
                 h3_unpack(va[n], s, re, im);
                 unsigned char *dst = smem + L::kA + (r >> 7) * 2 * L::kACopy + ((r & 127) >> 3) * L::SBO + (r & 7) * 16;
@@ -681,17 +679,29 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const __grid_c
         // 2.59e-7 in two pieces, 2.36e-7 in one, 2.31e-7 in the TMA-staged form; 1500: 2.68e-7, 2.37e-7, 2.43e-7)
         constexpr int kLin = M == 16 && KB == 16 ? 16 : 8, kPieces = M / kLin;
         const int p_lo = rank * kPieces / split, p_hi = (rank + 1) * kPieces / split;
-        asm volatile("bar.sync 1, 256;" ::: "memory");
         // query factor (inside the exponent already in the guarded form) and weight; a marked row keeps
         // nothing of the Gram
+        if (in_range) {
 #pragma unroll
-        for (int i = 0; i < 2; ++i) {
-            const float fq = a.wG * (in_range ? ex2(-a.k2 * s_nq[row + 128 * i]) : 1.f);
-            const bool keep = in_range || !(s_mask[(row + 128 * i) / 32] >> (row & 31) & 1);
+            for (int i = 0; i < 2; ++i) {
+                const float f = a.wG * ex2(-a.k2 * s_nq[row + 128 * i]);
 #pragma unroll
-            for (int k = 0; k < KB; ++k) {
-                acc1[i][k] = keep ? acc1[i][k] * fq : 0.f;
-                acc2[i][k] = keep ? acc2[i][k] * fq : 0.f;
+                for (int k = 0; k < KB; ++k) {
+                    acc1[i][k] *= f;
+                    acc2[i][k] *= f;
+                }
+            }
+        }
+        asm volatile("bar.sync 1, 256;" ::: "memory");  // (the halves' marks are complete)
+        if (!in_range) {
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const bool keep = !(s_mask[(row + 128 * i) / 32] >> (row & 31) & 1);
+#pragma unroll
+                for (int k = 0; k < KB; ++k) {
+                    acc1[i][k] = keep ? acc1[i][k] * a.wG : 0.f;
+                    acc2[i][k] = keep ? acc2[i][k] * a.wG : 0.f;
+                }
             }
         }
         for (int i = tid; i < kLin * (p_hi - p_lo) * KB; i += kH3Epi) {
