@@ -59,12 +59,12 @@ constexpr int kH3Epi = 256;       // epilogue threads
 constexpr int kH3Conv = 96;       // converter threads
 constexpr int kH3Threads = kH3Epi + kH3Conv + 32;
 constexpr int kH3MaxSplit = 8;    // CTAs per cluster
-// 16 antennas: dictionaries up to here keep the TMA-staged form and with it the last bit of their
-// outputs, which the gradient of a training-sized dictionary is taken of in FP64 (results compared at
-// 1e-9).  Above, this form is the faster one at every size measured (us of device time, TMA-staged form
-// and this): 6 users, 260 entries: 64 vectors 16.2 and 10.6, 16384: 34.8 and 17.1, 100000: 84.6 and 70.9;
-// 1024 entries: 64 vectors 25.7 and 13.8, 4000: 33.1 and 19.0, 65536: 138.6 and 128.0.  (2 users, 1024
-// entries, 65536 vectors: 93.1 and 84.5; 16 users: 258.8 and 236.9.)
+// 16 antennas: dictionaries up to here keep the TMA-staged form.  This is not where the forms cross (us of
+// device time, TMA-staged form and this; 6 users, 260 entries: 64 vectors 16.2 and 10.6, 16384: 34.8 and 17.1,
+// 100000: 84.6 and 70.9; 1024 entries: 64 vectors 25.7 and 13.8, 4000: 33.1 and 19.0, 65536: 138.6 and 128.0;
+// 2 users, 1024, 65536: 93.1 and 84.5; 16 users: 258.8 and 236.9), which lies lower.  It is the largest
+// dictionary whose results are kept to the last bit: gradient calls train on up to 256 pilots and return
+// their sums over these outputs in FP64, in which any other rounding of the Gram shows.
 constexpr int kH3MinEntries16 = 256;
 constexpr int kH3Devices = 16;    // devices whose cluster counts are kept
 // One CTA per SM is a condition of this kernel, not a matter of occupancy: a CTA holds all 512 TMEM
@@ -793,7 +793,11 @@ __global__ void __launch_bounds__(kH3Threads, 1) detect_h3_kernel(const __grid_c
 // How `nq` query tiles of `nt` entry tiles each are launched: `full` of them first, one CTA each in
 // whole waves, then the rest with `split` CTAs per tile, whichever costs the least in entry tiles per
 // SM (a CTA's set-up and merge count as kSetup of them; `resident` [s] clusters of s CTAs fit the GPU
-// at a time).
+// at a time).  The time of a full wave puts the set-up at 6 to 10 tiles at 16 antennas and 6 users, more
+// than kSetup; but of 99 sizes timed with 3 and with 8 (16, 32 and 64 antennas, 2 to 16 users, 300 to 4096
+// entries, 300 to 100003 vectors) 90 take the same time, and of the other nine five are faster with 3 (by
+// up to 4 %: 16 antennas, 6 users, 4096 entries, 20000 vectors 155 and 161 us) and four with 8 (64, 4, 2048,
+// 20000: 117 and 112).
 struct H3Plan {
     int full, split;
 };
