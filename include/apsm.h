@@ -249,6 +249,11 @@ apsm_status apsm_train_noalloc(const apsm_params *p, const float *rx_pilot, cons
  *   soft  device [N][K] complex      output
  *   hard  device [N][K] uint8        output, may be NULL
  * p->dtype selects the contraction precision (APSM_FP32 here).
+ * The same call gives the same bits.  A vector's last bits may depend on the call around it: in
+ * FP32 with 32 or 64 antennas, or 16 and a capacity above 256, the dictionary is summed in as many
+ * parts as fill the GPU, which depends on N and on whether the vector lies in the last, partial
+ * wave; with a workspace (apsm_detect_ws) likewise at 4, 8 and 16 antennas.  The difference is
+ * that of an FP32 sum in another order; APSM_OPT_DETECT_TMA = 0 sums every vector alike.
  * Errors as for apsm_train.
  */
 apsm_status apsm_detect(const apsm_params *p, const apsm_state *st, const float *rx, int32_t N, float *soft,
@@ -256,8 +261,8 @@ apsm_status apsm_detect(const apsm_params *p, const apsm_state *st, const float 
 
 /*
  * Detection with a workspace (the same results as apsm_detect up to rounding order; Sec. III-B
- * detection).  FP32 detection with 4, 8 or 16 antennas and an even user count in
- * {2, 4, 6, 8, 12, 16} splits its (query tile, dictionary tile) work evenly over a persistent
+ * detection).  FP32 detection with 4, 8 or (dictionary capacity up to 256) 16 antennas and an
+ * even user count in {2, 4, 6, 8, 12, 16} splits its (query tile, dictionary tile) work evenly over a persistent
  * grid; a query tile split between CTAs leaves each part's sums in the workspace and the CTA
  * that brings its last part adds the parts in a fixed order (results do not depend on timing).
  * BF16/FP16 detection with 16, 32 or 64 antennas packs the dictionary's operands into the
@@ -265,7 +270,9 @@ apsm_status apsm_detect(const apsm_params *p, const apsm_state *st, const float 
  * APSM_OPT_HALF_TC_COEF): the exponentials rounded to BF16 against the coefficients as a BF16
  * hi + lo pair, accumulated in FP32.
  *   apsm_detect_workspace_bytes: bytes for N data vectors on the current device; 0 where the
- *     balanced form does not apply (apsm_detect_ws then runs apsm_detect).
+ *     antennas and users have no balanced form (apsm_detect_ws then runs apsm_detect).  At 16
+ *     antennas it does not look at the capacity: above 256 entries apsm_detect_ws leaves a
+ *     workspace untouched and gives the bits of apsm_detect, so none need be allocated.
  *   workspace  device, 256-byte aligned, at least that many bytes, ZERO-FILLED before its first
  *     use.  It starts with one arrival counter per 128 data vectors (int32); every call that
  *     completes without a status error leaves them at zero again (the rest is scratch).  After
