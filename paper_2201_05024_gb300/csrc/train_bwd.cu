@@ -33,6 +33,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <type_traits>
 
 #include "apsm_common.cuh"
 #include "train_f32.cuh"
@@ -614,6 +615,11 @@ constexpr int kPfV = 4;    // float4 of a row per lane and table that are staged
 // 152 (304 CTAs): 2948 and 3020, 200: 4083 and 3603, 512: 9763 and 8021; window 16: 152: 2948 and 3568,
 // 256: 5356 and 4625.  Two team CTAs on an SM at 80 registers a thread: 256 instances 5597).
 constexpr int kTeamCtas = 2 * 152;
+// Rows from which on the entries past the staged ones are loaded sixteen (then four) to a lane together, instead
+// of one after the other, each a wait for L2 in the row warp (one call, 6 users, ms, one by one and together):
+// window 8: 600 entries 1.03 and 1.07, 800: 1.83 and 1.68, 1024: 3.29 and 2.37, 2000: 17.0 and 8.1, 4000: 140 and 35;
+// window 20: 1024 entries 3.64 and 3.83; window 24, 4 users, 64 instances: 1400 entries 8.58 and 7.74.
+constexpr int kLongRow = 768, kLongRowWide = 1280;  // windows up to 16, and wider ones
 constexpr int kAhead = 3;  // steps ahead that global reads are issued; a ring of kAhead + 1 slots
 
 // Reads of a later step, copied to the lane's own slots of a shared-memory ring (cp.async: no register
@@ -680,7 +686,8 @@ __host__ __device__ inline int bwd_team_floats(int S, int W, int L2) {
 // WM: a bound on the window (8, 16 or 30) over which the O(W) loops are unrolled: their operands are
 // loaded first, all in flight, and slots at or past |J_n| take a zero coefficient (the rings start at
 // zero, so every product is finite).
-template <int WM>
+// kLong: rows of more than kLongRow entries (a form of its own: short rows are up to 8 % slower with it).
+template <int WM, bool kLong>
 __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kernel(const TrainBwdArgs a0) {
     extern __shared__ __align__(16) float sm[];
     const TrainBwdArgs a = for_instance(a0, blockIdx.y);
@@ -867,7 +874,28 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
                         }
                     }
                     const float *grow = a.gtab + (size_t)jn * a.Sp, *drow = a.gdtab + (size_t)jn * a.Sp;
-                    for (int i = max(lo, lo4 + 4 * 32 * kPfV) + lane; i < jn; i += 32) {
+                    int i = max(lo, lo4 + 4 * 32 * kPfV) + lane;
+                    auto together = [&](auto n_c) {  // n entries of a lane with their loads in flight together
+                        constexpr int n = decltype(n_c)::value;
+                        for (; i + 32 * (n - 1) < jn; i += 32 * n) {
+                            float g[n], d[n];
+#pragma unroll
+                            for (int q = 0; q < n; ++q) {
+                                g[q] = ldg_if(true, grow + i + 32 * q);
+                                d[q] = ldg_if(true, drow + i + 32 * q);
+                            }
+#pragma unroll
+                            for (int q = 0; q < n; ++q) {
+                                y2[0] = fmaf(gam[i + 32 * q], g[q], y2[0]);
+                                d2[0] = fmaf(gam[i + 32 * q], d[q], d2[0]);
+                            }
+                        }
+                    };
+                    if constexpr (kLong) {
+                        together(std::integral_constant<int, 16>{});
+                        together(std::integral_constant<int, 4>{});
+                    }
+                    for (; i < jn; i += 32) {
                         y2[0] = fmaf(gam[i], __ldg(grow + i), y2[0]);
                         d2[0] = fmaf(gam[i], __ldg(drow + i), d2[0]);
                     }
@@ -1104,7 +1132,23 @@ __global__ void __launch_bounds__(kTeamThreads * kTeamUsers) train_bwd_team_kern
                         }
                     }
                 }
-                for (int i = max(lo, lo4 + 4 * 32 * kPfV) + lane; i < hi; i += 32)
+                int i = max(lo, lo4 + 4 * 32 * kPfV) + lane;
+                const int below = min(hi, s_lo);  // (no snapshot below s_lo)
+                auto together = [&](auto n_c) {
+                    constexpr int n = decltype(n_c)::value;
+                    for (; i + 32 * (n - 1) < below; i += 32 * n) {
+                        float g[n];
+#pragma unroll
+                        for (int q = 0; q < n; ++q) g[q] = ldg_if(true, grow + i + 32 * q);
+#pragma unroll
+                        for (int q = 0; q < n; ++q) g2[0] = fmaf(gam[i + 32 * q], g[q], g2[0]);
+                    }
+                };
+                if constexpr (kLong) {
+                    together(std::integral_constant<int, 16>{});
+                    together(std::integral_constant<int, 4>{});
+                }
+                for (; i < hi; i += 32)
                     g2[0] = fmaf(i >= s_lo ? gam[i] - sv[i - s_lo] : gam[i], __ldg(grow + i), g2[0]);
                 const float gs = warp_sum(g2[0] + g2[1]);
                 if (lane == 0) sums[0] = gs;
@@ -1255,9 +1299,8 @@ apsm_status train_bwd_run(const apsm_params *p, int n, const float *rx_pilot, co
         sizeof(float) * (2 * (size_t)((2 * P + 3) & ~3) + (size_t)p->K * bwd_warp_floats(2 * P, p->window, 2 * p->M));
     const int users = std::min(p->K, kTeamUsers), ctas = (p->K + users - 1) / users;
     const bool one_fits = p->window <= 32 && smem_1 <= 227 * 1024;
-    const bool team_form = p->window <= 30 && smem_w <= 227 * 1024 && (!one_fits || (long long)ctas * n <= kTeamCtas);
-    const bool one_form = !team_form && one_fits;
-    if (!team_form && !one_form && smem > 227 * 1024) return APSM_ERR_UNSUPPORTED;
+    const bool team_fits = p->window <= 30 && smem_w <= 227 * 1024;
+    if (!team_fits && !one_fits && smem > 227 * 1024) return APSM_ERR_UNSUPPORTED;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) {
         cudaGetLastError();
@@ -1267,6 +1310,17 @@ apsm_status train_bwd_run(const apsm_params *p, int n, const float *rx_pilot, co
     cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
     cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, dev);
     if (major != 10 || minor != 3) return APSM_ERR_NOT_SM103;
+    const int row = 2 * std::min(P, p->dict_cap);  // live centres
+    const bool is_long = row > (p->window <= 16 ? kLongRow : kLongRowWide);
+    auto team_kern = p->window <= 8    ? (is_long ? train_bwd_team_kernel<8, true> : train_bwd_team_kernel<8, false>)
+                     : p->window <= 16 ? (is_long ? train_bwd_team_kernel<16, true> : train_bwd_team_kernel<16, false>)
+                                       : (is_long ? train_bwd_team_kernel<30, true> : train_bwd_team_kernel<30, false>);
+    bool team_form = team_fits;
+    if (team_fits) {
+        if (cudaFuncSetAttribute(team_kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_w) != cudaSuccess)
+            return APSM_ERR_CUDA;
+        if (one_fits) team_form = (long long)ctas * n <= kTeamCtas;
+    }
     cudaStream_t strm = static_cast<cudaStream_t>(stream);
     unsigned char *ws = static_cast<unsigned char *>(workspace);
     TrainBwdArgs a{};
@@ -1302,15 +1356,12 @@ apsm_status train_bwd_run(const apsm_params *p, int n, const float *rx_pilot, co
     a.st_mk = (size_t)p->M * p->K;
     a.ws_stride = b.total;
     a.mode = mode;
+    const bool one_form = !team_form && one_fits;
     const long long pairs = 2LL * P * a.Sp;
     const int blocks = (int)std::min<long long>(std::max(1, 4096 / n), (pairs + 255) / 256);
     if (mode & 1) train_bwd_tables_kernel<<<dim3(blocks, n), 256, 0, strm>>>(a);
     if (team_form) {
-        auto kern = p->window <= 8 ? train_bwd_team_kernel<8>
-                    : p->window <= 16 ? train_bwd_team_kernel<16> : train_bwd_team_kernel<30>;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_w) != cudaSuccess)
-            return APSM_ERR_CUDA;
-        kern<<<dim3(ctas, n), kTeamThreads * users, smem_w, strm>>>(a);
+        team_kern<<<dim3(ctas, n), kTeamThreads * users, smem_w, strm>>>(a);
     } else if (one_form) {
         auto kern = p->window <= 8 ? train_bwd_warp_kernel<8>
                     : p->window <= 16 ? train_bwd_warp_kernel<16> : train_bwd_warp_kernel<32>;
