@@ -610,11 +610,19 @@ __global__ void __launch_bounds__(kBwdThreads, 6) train_bwd_kernel(const TrainBw
 constexpr int kTeamUsers = 3;
 constexpr int kTeamThreads = 128;
 constexpr int kPfV = 4;    // float4 of a row per lane and table that are staged ahead (512 entries)
-// Up to two CTAs of teams per SM's turn; more users run one warp each, all resident at once (16 antennas,
-// 6 users, 256 pilots, us for n instances, teams and single warps: window 8: 64: 1383 and 2295,
-// 152 (304 CTAs): 2948 and 3020, 200: 4083 and 3603, 512: 9763 and 8021; window 16: 152: 2948 and 3568,
-// 256: 5356 and 4625.  Two team CTAs on an SM at 80 registers a thread: 256 instances 5597).
-constexpr int kTeamCtas = 2 * 152;
+// The team form's launches: all of its CTAs on the GPU at once, or in two goes where rows are short and no
+// entry leaves, and not where the users leave a quarter of the teams empty with wide windows, nor for up to
+// 6 users over the shortest sequences; more run one warp per user, all resident at once.  16 antennas, window
+// 8 unless said, us as teams and as single warps:
+//   one go     6 users, 256 pilots, 64 instances 1360 and 2320; 1000 pilots 17370 and 22700
+//   two goes   6 users, 256 pilots, 100 instances 2400 and 2636, 150: 2820 and 3036; window 16: 2500 and 3159;
+//              7 users, 300 pilots, 64: 2588 and 2880;
+//              12 users, 64: 2120 and 2552; but 400 pilots, 6 users, 150: 6340 and 6130; 700 pilots over 200
+//              entries, 150: 15700 and 14900; window 24, 4 users, 150: 4570 and 4190; 40 pilots, 4 users,
+//              150: 326 and 308
+//   more       6 users, 256 pilots, 200 instances 4083 and 3603, 512: 9763 and 8021
+// (two team CTAs on an SM at 80 registers a thread: 256 instances 5597, 5356 without).
+constexpr int kTeamTwoRow = 128, kTeamTwoUsers = 6, kTeamTwoMax = 640, kTeamTwoMaxWide = 512;
 // Rows from which on the entries past the staged ones are loaded sixteen (then four) to a lane together, instead
 // of one after the other, each a wait for L2 in the row warp (one call, 6 users, ms, one by one and together):
 // window 8: 600 entries 1.03 and 1.07, 800: 1.83 and 1.68, 1024: 3.29 and 2.37, 2000: 17.0 and 8.1, 4000: 140 and 35;
@@ -1319,7 +1327,19 @@ apsm_status train_bwd_run(const apsm_params *p, int n, const float *rx_pilot, co
     if (team_fits) {
         if (cudaFuncSetAttribute(team_kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_w) != cudaSuccess)
             return APSM_ERR_CUDA;
-        if (one_fits) team_form = (long long)ctas * n <= kTeamCtas;
+        if (one_fits) {
+            const long long grid = (long long)ctas * n;
+            int sms = 0, per_sm = 1;
+            if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return APSM_ERR_CUDA;
+            if (grid > sms && cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, team_kern, kTeamThreads * users,
+                                                                            smem_w) != cudaSuccess)
+                return APSM_ERR_CUDA;
+            const bool two_goes = grid <= 2LL * sms * per_sm && P <= p->dict_cap &&
+                                  (p->window <= 16 ? row <= kTeamTwoMax
+                                                   : row <= kTeamTwoMaxWide && 4 * p->K >= 3 * users * ctas) &&
+                                  (row >= kTeamTwoRow || p->K > kTeamTwoUsers);
+            team_form = grid <= (long long)sms * per_sm || two_goes;
+        }
     }
     cudaStream_t strm = static_cast<cudaStream_t>(stream);
     unsigned char *ws = static_cast<unsigned char *>(workspace);
