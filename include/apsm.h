@@ -252,7 +252,7 @@ apsm_status apsm_train_noalloc(const apsm_params *p, const float *rx_pilot, cons
  * The same call gives the same bits.  A vector's last bits may depend on the call around it: in
  * FP32 with 32 or 64 antennas, or 16 and a capacity above 256, the dictionary is summed in as many
  * parts as fill the GPU, which depends on N and on whether the vector lies in the last, partial
- * wave; with a workspace (apsm_detect_ws) likewise at 4, 8 and 16 antennas.  The difference is
+ * wave, and with 32 or 64 antennas and at most 128 entries N also chooses the form; with a workspace (apsm_detect_ws) likewise at 4, 8 and 16 antennas.  The difference is
  * that of an FP32 sum in another order; APSM_OPT_DETECT_TMA = 0 sums every vector alike.
  * Errors as for apsm_train.
  */
@@ -469,7 +469,7 @@ apsm_status apsm_check_wait_timeout(const apsm_state *st, void *stream);
  *   APSM_OPT_DETECT_TMA   1 (default): FP32 detection with 4, 8 or 16 antennas and an even user
  *                         count in {2, 4, 6, 8, 12, 16} stages every operand by TMA (entry rows
  *                         as stored, the real split's rotation on the query side), and with 32
- *                         or 64 antennas, or 16 and a dictionary capacity above 256, forms the Gram
+ *                         or 64 antennas (but for few entries and vectors), or 16 and a dictionary capacity above 256, forms the Gram
  *                         from three FP16 products of scaled hi and lo copies; 0: the tensor-core form that converts entry rows to TF32 in
  *                         shared memory (64 antennas: the FP32 FMA engine)
  *   APSM_OPT_HALF_TC_COEF 1 (default): BF16/FP16 detection with 16, 32 or 64 antennas forms the

@@ -650,7 +650,7 @@ apsm_status apsm_detect_ws(const apsm_params *p, const apsm_state *st, const flo
         // BF16/FP16 with a workspace: the coefficient sums on the tensor cores too
         TccLauncher tcc = (prec == kHalf && workspace && g_opt_half_tc_coef.load()) ? detect_tcc_launcher(p->M, p->K)
                                                                                      : nullptr;
-        H3Launcher h3 = (p->dtype == APSM_FP32 && g_opt_detect_tma.load() && (p->M != 16 || p->dict_cap > kH3MinEntries16))
+        H3Launcher h3 = (p->dtype == APSM_FP32 && g_opt_detect_tma.load() && h3_pays(p->M, p->K, p->dict_cap, N))
                             ? detect_h3_launcher(p->M, p->K)
                             : nullptr;
         TmaLauncher tma = (p->dtype == APSM_FP32 && g_opt_detect_tma.load()) ? detect_tma_launcher(p->M, p->K) : nullptr;

@@ -66,6 +66,20 @@ constexpr int kH3MaxSplit = 8;    // CTAs per cluster
 // dictionary whose results are kept to the last bit: gradient calls train on up to 256 pilots and return
 // their sums over these outputs in FP64, in which any other rounding of the Gram shows.
 constexpr int kH3MinEntries16 = 256;
+// Whether this form takes a call of N vectors.  Its CTA is set up for 256 queries and its first tile of entries
+// takes as long as a full one, so small dictionaries over few vectors keep the former form (us of device
+// time, former and this):
+//   64 antennas (FMA engine)  6 users, 300 vectors: 1 entry 5.6 and 22.0, 64: 13.2 and 18.9, 96: 17.6 and 18.1, 97:
+//                             18.7 and 17.7; 16 users: 96: 20.0 and 25.2, 128: 24.2 and 25.1, 160: 28.5 and 26.6;
+//                             12000 vectors, 6 users: 32: 15.4 and 22.3, 64: 23.0 and 19.0; 11 users: 16: 22.9 and
+//                             26.2, 32: 31.0 and 26.3
+//   32 antennas (TF32 x3)     300 vectors, 2 users: 32: 10.0 and 12.1, 64: 10.7 and 10.9, 65: 13.0 and 10.5; 6 users: 32:
+//                             12.3 and 14.5, 33: 12.6 and 12.8; 24000 vectors, 2 users, 1 entry: 18.4 and 12.7
+inline bool h3_pays(int M, int K, int dict_cap, int N) {
+    if (M == 16) return dict_cap > kH3MinEntries16;
+    if (M == 32) return dict_cap > (K <= 4 ? 64 : 32) || N > 16384;
+    return dict_cap > (K > 12 ? 128 : 96) || (long long)N * dict_cap > (K <= 8 ? 400000 : 300000);
+}
 constexpr int kH3Devices = 16;    // devices whose cluster counts are kept
 // One CTA per SM is a condition of this kernel, not a matter of occupancy: a CTA holds all 512 TMEM
 // columns while it waits for its cluster, so of two on one SM the second would wait in its allocation,

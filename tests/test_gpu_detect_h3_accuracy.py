@@ -38,7 +38,8 @@ def test_error_is_not_above_the_form_without_it(M, K, D):
     assert rms(e_new) <= 1.05 * rms(e_old)
 
 
-@pytest.mark.parametrize("M,K,D", [(16, 2, 300), (16, 6, 290), (32, 5, 100), (64, 2, 70), (64, 6, 40), (64, 9, 70)])
+@pytest.mark.parametrize("M,K,D", [(16, 2, 300), (16, 6, 290), (32, 5, 100), (32, 16, 1), (32, 7, 31), (32, 2, 33),
+                                   (64, 2, 70), (64, 6, 33), (64, 9, 32), (64, 16, 31)])
 @pytest.mark.parametrize("extra", [-1, 0, 1, 300])
 def test_edges_of_whole_waves(M, K, D, extra):
     wave = 256 * torch.cuda.get_device_properties(0).multi_processor_count
@@ -56,3 +57,27 @@ def test_edges_of_whole_waves(M, K, D, extra):
     ref = oracle.detect(op, oracle_state_fp32(M, ent, gam, clin), np.ascontiguousarray(rx[rows]))
     assert_soft_close(soft.cpu().numpy()[rows], ref, tol=1e-5)
     assert apsm.read_status(st) == 0
+
+
+@pytest.mark.parametrize("M,K,D,N", [(64, 6, 96, 700), (64, 6, 97, 700), (64, 16, 128, 300), (64, 16, 129, 300),
+                                     (64, 2, 32, 12500), (64, 2, 32, 12501), (64, 11, 20, 15000), (64, 11, 20, 15001),
+                                     (32, 4, 64, 500), (32, 4, 65, 500), (32, 5, 32, 500), (32, 5, 33, 500),
+                                     (32, 5, 32, 16384), (32, 5, 32, 16385)])
+def test_either_side_of_the_line_to_the_former_form(M, K, D, N):
+    ent, gam, clin = synth.random_state(M, K, D, instance=M + K)
+    rx = synth.random_state(M, 1, N, instance=9)[0]
+    op = oracle.Params(M=M, K=K, W=1, D=D, sigma=0.5, w_L=0.5)
+    gp = gpu_params(op)
+    st = load_state(gp, ent, gam, clin)
+    soft = apsm.detect(gp, st, to_dev(rx))[0].cpu().numpy()
+    rows = np.unique(np.concatenate([np.arange(0, N, 37), np.arange(max(N - 300, 0), N)]))
+    ref = oracle.detect(op, oracle_state_fp32(M, ent, gam, clin), np.ascontiguousarray(rx[rows]))
+    assert_soft_close(soft[rows], ref, tol=1e-5)
+    try:   # the same call in the form without FP16 products, of which the outputs are an FP32 rounding away
+        apsm.set_option("detect_tma", 0)
+        plain = apsm.detect(gp, st, to_dev(rx))[0].cpu().numpy()
+    finally:
+        apsm.set_option("detect_tma", 1)
+    former = not (D > (64 if K <= 4 else 32) or N > 16384) if M == 32 else \
+        not (D > (128 if K > 12 else 96) or N * D > (400000 if K <= 8 else 300000))
+    assert np.array_equal(soft, plain) == former
