@@ -174,15 +174,28 @@ TrainGeom train_geom(const apsm_params *p, int P, int n_prev, int evict = -1) {
     g.WP = padded_window(g.W);
     g.slice = kTileEntries;
     const bool want_track = g_opt_train_track.load() != 0;
-    for (;; --T) {  // the largest chunk whose phase-B tables fit in shared memory
-        g.T = T;
+    auto set = [&](int t) {
+        T = g.T = t;
         g.RMAX = 2 * T + g.W;
         g.RS = round_up(g.RMAX, 32);
         g.KXS = round_up(2 * T, 32);
         // tracking needs the blocked form (padded window <= 24), whose other warps do it, and a live
         // range of more than one warp
         g.track = want_track && g.WP <= 24 && g.RS >= 64 && 2 * T <= 2 * (g.RS - 32) ? 1 : 0;
-        if (T == 1 || ChunkSmem(g).bytes <= kMaxSmemBytes) break;
+    };
+    const int most = T;
+    for (set(T); T > 1 && ChunkSmem(g).bytes > kMaxSmemBytes; set(T - 1)) {}  // the largest chunk whose phase-B tables fit
+    if (T < most && g.WP <= 24) {
+        // A chunk that shared memory cuts short (64 antennas with entries that leave) ends on a whole block where
+        // that takes no more chunks; and with blocks of up to 12 steps, behind which the other warps' second round
+        // of the next chunk's samples does not hide, it has no more of them than those warps have threads (64
+        // antennas, 16 users, 600 pilots over 300 entries, us with the largest chunk and this: window 13 275 and
+        // 261, 17: 333 and 294, 20: 322 and 294; 16: 257 either way).
+        const int half = (32 - g.WP) / 2;  // vectors per block
+        int t = T / half * half;
+        if (half <= 6 && 2 * t > g.RS - 32 && P >= 4 * T) t = (g.RS - 32) / 2 / half * half;
+        else if (t > 0 && (P + t - 1) / t != (P + T - 1) / T) t = T;
+        if (t > 0 && t < T && round_up(2 * t + g.W, 32) == g.RS) set(t);
     }
     g.n_chunks = P > 0 ? (P + T - 1) / T : 0;
     return g;
