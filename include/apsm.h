@@ -469,8 +469,9 @@ apsm_status apsm_check_wait_timeout(const apsm_state *st, void *stream);
  *   APSM_OPT_DETECT_TMA   1 (default): FP32 detection with 4, 8 or 16 antennas and an even user
  *                         count in {2, 4, 6, 8, 12, 16} stages every operand by TMA (entry rows
  *                         as stored, the real split's rotation on the query side), and with 32
- *                         or 64 antennas (but for few entries and vectors), or 16 and a dictionary capacity above 256, forms the Gram
- *                         from three FP16 products of scaled hi and lo copies; 0: the tensor-core form that converts entry rows to TF32 in
+ *                         or 64 antennas (but for few entries and vectors), or 16 and a dictionary
+ *                         capacity above 256, forms the Gram from three FP16 products of scaled hi
+ *                         and lo copies; 0: the tensor-core form that converts entry rows to TF32 in
  *                         shared memory (64 antennas: the FP32 FMA engine)
  *   APSM_OPT_HALF_TC_COEF 1 (default): BF16/FP16 detection with 16, 32 or 64 antennas forms the
  *                         coefficient sums on the tensor cores too (the exponentials rounded to

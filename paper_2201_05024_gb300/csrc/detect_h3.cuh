@@ -1,4 +1,4 @@
-// detect_h3.cuh -- FP32-accuracy detection for 32 and 64 antennas with the complex dist-Gram on the
+// detect_h3.cuh -- FP32-accuracy detection for 16, 32 and 64 antennas with the complex dist-Gram on the
 // tensor cores as three FP16 products (Sec. III-B detection; the same result as detect_tc.cuh).
 //
 // FP16 and TF32 hold the same 11 significant bits, so hi*hi + hi*lo + lo*hi with hi = fp16(x),
@@ -29,8 +29,8 @@
 // Roles (384 threads): warps 0-7 prepare the query operand, then are the epilogue (TMEM lanes
 // 32 (w mod 4) .., entries 16 (w / 4) .. of a tile), warps 8-10 convert entry tiles (hi and lo copies,
 // coefficients, norms; a tile's global loads are issued before the wait for its stage), warp 11
-// issues the MMAs.  Entry operand two stages, coefficients and accumulators four.  All waits on an
-// mbarrier are bounded; a timed-out CTA still meets its cluster at both barriers.  Those and the TMEM
+// issues the MMAs.  Entry operand two stages, coefficients four, accumulators four over the sums
+// (h3_sums).  All waits on an mbarrier are bounded; a timed-out CTA still meets its cluster at both barriers.  Those and the TMEM
 // allocation are the hardware's own waits, without a limit, and end because a CTA has its SM to itself as
 // far as this kernel goes (kH3OneCta) and no other kernel waits for another CTA while it holds TMEM.
 //
@@ -38,8 +38,8 @@
 // epilogue of a tile takes 6700 cycles, 5700 while the converters rest, against 4400 of packed FMAs;
 // the MMAs 3000, beside it; ncu: FMA pipe 66 % active).
 // Measured (FP32, 64 antennas, 16 users, 4096 entries, 100003 vectors): 8025 us on the FMA engine
-// (323 FMA per pair), 1288 us here.  32 antennas, 11 users, 1500 entries, 10001 vectors: 110 us in the
-// TF32 x3 converter form (79 CTAs of 128 queries for 152 SMs), 64 us here.  16 antennas, 6 users, 1024
+// (323 FMA per pair), 1290 us here.  32 antennas, 11 users, 1500 entries, 10001 vectors: 110 us in the
+// TF32 x3 converter form (79 CTAs of 128 queries for 152 SMs), 62 us here.  16 antennas, 6 users, 1024
 // entries: an entry tile takes 3340 cycles (1800 of FMAs) against 3950 per 32 entries and 256 queries in
 // the TMA-staged TF32 x3 form; resting the converters, dropping the exponentials or the coefficient reads
 // saves 5, 5 and 10 %, four epilogue groups instead of two nothing: warps wait for the FMA pipe.
@@ -83,8 +83,8 @@ inline bool h3_pays(int M, int K, int dict_cap, int N) {
 constexpr int kH3Devices = 16;    // devices whose cluster counts are kept
 // One CTA per SM is a condition of this kernel, not a matter of occupancy: a CTA holds all 512 TMEM
 // columns while it waits for its cluster, so of two on one SM the second would wait in its allocation,
-// and two clusters that meet on two SMs in opposite order would wait for each other for ever.  (At 16
-// antennas and up to 2 users two would fit: 77 registers a thread, 53 KB.)  So every launch asks for
+// and two clusters that meet on two SMs in opposite order would wait for each other for ever.  (Registers do
+// not see to it: at 16 antennas and 2 users two fitted with 77 a thread and 53 KB of shared memory.)  So every launch asks for
 // more than half of an SM's 228 KB, of which each CTA has 1 KB reserved.
 constexpr int kH3OneCta = 116 * 1024;
 static_assert(2 * (kH3OneCta + 1024) > 228 * 1024, "two CTAs of any instantiations do not fit an SM");
