@@ -154,6 +154,8 @@ DetectShape detect_shape(int M, int K, int dtype) {
 // Geometry of one training call: P new vectors after n_prev earlier ones (of which the last
 // nc0 = min(n_prev, W/2) pilots are carried, because the first new window reaches back into
 // them).  evict: -1 = decide from the counts, 0/1 = forced (workspace bounds over both cases).
+size_t train_ws_total(const TrainGeom &g);  // bytes of a fresh training's workspace
+
 TrainGeom train_geom(const apsm_params *p, int P, int n_prev, int evict = -1) {
     TrainGeom g;
     g.M = p->M;
@@ -182,6 +184,7 @@ TrainGeom train_geom(const apsm_params *p, int P, int n_prev, int evict = -1) {
         // tracking needs the blocked form (padded window <= 24), whose other warps do it, and a live
         // range of more than one warp
         g.track = want_track && g.WP <= 24 && g.RS >= 64 && 2 * T <= 2 * (g.RS - 32) ? 1 : 0;
+        g.n_chunks = P > 0 ? (P + T - 1) / T : 0;
     };
     const int most = T;
     for (set(T); T > 1 && ChunkSmem(g).bytes > kMaxSmemBytes; set(T - 1)) {}  // the largest chunk whose phase-B tables fit
@@ -195,9 +198,13 @@ TrainGeom train_geom(const apsm_params *p, int P, int n_prev, int evict = -1) {
         int t = T / half * half;
         if (half <= 6 && 2 * t > g.RS - 32 && P >= 4 * T) t = (g.RS - 32) / 2 / half * half;
         else if (t > 0 && (P + t - 1) / t != (P + T - 1) / T) t = T;
-        if (t > 0 && t < T && round_up(2 * t + g.W, 32) == g.RS) set(t);
+        if (t > 0 && t < T && round_up(2 * t + g.W, 32) == g.RS) {
+            const int largest = T;
+            const bool fitted = train_ws_total(g) <= (size_t)APSM_NOALLOC_SCRATCH_BYTES;
+            set(t);  // (but for a sequence that only so would outgrow the library's scratch array)
+            if (fitted && train_ws_total(g) > (size_t)APSM_NOALLOC_SCRATCH_BYTES) set(largest);
+        }
     }
-    g.n_chunks = P > 0 ? (P + T - 1) / T : 0;
     return g;
 }
 
@@ -240,6 +247,8 @@ TrainWs train_ws(const TrainGeom &g, bool ext) {
     w.total = g.n_chunks > 0 ? off : 0;
     return w;
 }
+
+size_t train_ws_total(const TrainGeom &g) { return train_ws(g, false).total; }
 
 // Workspace bound of a continuation of P vectors, whatever n_prev (carried pilots at most W/2,
 // with or without eviction).
